@@ -71,23 +71,21 @@ cdf_nn_status cdf_nn_mse(const float *pred, const float *target, float *grad, fl
 cdf_nn_status cdf_nn_adam(float *w, const float *g, float *m, float *v, void *w_bf16, long long n, float lr, float b1,
                           float b2, float eps, long long step, void *stream);
 const char *cdf_nn_last_error(void);
-/* Tensor-core path of the convolutions above.  1 (the default): the 5th-generation
- * tensor cores (tcgen05.mma, accumulators in tensor memory) with the faster operand
- * staging for the layer's depth -- for a forward pass whose image rows are whole
- * 128-pixel tiles with 16, 32 or 64 input channels, the kernel without im2col copy
- * (each tile's three input rows staged once; every tap's operand is the same rows
- * seen through a shifted descriptor; persistent CTAs); otherwise tiles copied by
- * cp.async through three stage buffers when the GEMM input has at least 128
- * channels, two buffers filled by ordinary loads below that (more CTAs per SM hide
- * more latency at short K); 4: the kernel without im2col copy where the shape
- * allows it, else as 1;
- * 2: tcgen05 with the two-buffer staging for every layer; 3: the forward pass on a
- * persistent warp-specialised tcgen05 kernel (producer warps, one MMA thread, epilogue
- * warps, two accumulators; slower than 1 at the surrogate's layer shapes, where one
- * CTA per SM leaves too few warps to hide latency), the backward pass as in 1;
- * 0: the warp-level MMA kernels.  The weight gradient runs on tcgen05 for 1 to 4.
+/* Tensor-core path of the convolutions above.  1 (the default) and 4: the
+ * 5th-generation tensor cores (tcgen05.mma, accumulators in tensor memory) without
+ * im2col copies: the positions a tile reads are staged once with all input channels
+ * and every tap's operand is the same rows seen through a shifted descriptor, for any
+ * image size whose staged positions fit in shared memory (at 32 channels up to about
+ * W = 1500, at 256 up to W = 140); wider images take the im2col staging that is faster
+ * for the layer's depth -- three cp.async stage buffers when the GEMM input has at
+ * least 128 channels, two buffers filled by ordinary loads below that;
+ * 2: tcgen05 with the two-buffer im2col staging for every layer; 3: the forward pass
+ * on a persistent warp-specialised im2col kernel, the backward pass on im2col staging;
+ * 0: the warp-level MMA kernels.  The weight gradient runs on tcgen05 for 1 to 4 (an
+ * image of 2^30 padded pixels and more on the warp-level kernel, which adds atomically).
  * Process-wide; all give the same results up to the order of the FP32 accumulation
- * (1 to 4 issue the same MMAs in the same order: the same bits). */
+ * (forward and input gradient: 1 to 4 issue the same MMAs in the same order, the same
+ * bits). */
 cdf_nn_status cdf_nn_set_tensor_path(int tcgen05);
 /* *out = 1 if a bounded wait of a tcgen05 convolution ever ran out (its output is
  * then undefined), else 0.  Synchronises with the device. */

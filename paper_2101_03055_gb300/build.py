@@ -24,7 +24,8 @@ OBJ = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libcdflb.so")
 LIB_CHECKS = os.path.join(PKG, "libcdflb_checks.so")
 HEADERS = [os.path.join(ROOT, "include", "cdf_lb.h"), os.path.join(ROOT, "include", "cdf_lb3d.h"),
-           os.path.join(ROOT, "include", "cdf_nn.h"), os.path.join(CSRC, "lb_internal.h"), os.path.join(CSRC, "lb_device.cuh")]
+           os.path.join(ROOT, "include", "cdf_nn.h"), os.path.join(CSRC, "lb_internal.h"), os.path.join(CSRC, "lb_device.cuh"),
+           os.path.join(CSRC, "nn_conv.cuh")]
 SOURCES = ["lb_kernels.cu", "lb_reduce.cu", "lb_host.cu", "lb_static.cu", "lb_batch.cu", "lb_resident.cu", "lb_split.cu",
            "lb_checks.cu", "lb3d.cu", "nn_kernels.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

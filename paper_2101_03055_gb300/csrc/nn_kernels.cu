@@ -5,12 +5,16 @@
 // channel copies for skip connections, 1x1 output head, MSE loss, Adam).
 // Activations are NHWC with the channel count a multiple of 16; 3x3 weights
 // are [Cout][3][3][Cin].
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <mma.h>
 
 #include <algorithm>
+#include <atomic>
+#include <cmath>
 #include <cstdint>
+#include <utility>
 
 #include "../../include/cdf_nn.h"
 
@@ -757,226 +761,7 @@ cudaError_t launch_conv_ws(const __nv_bfloat16 *in, const __nv_bfloat16 *w, cons
     return cudaGetLastError();
 }
 
-// ---------------------------------------------------------------------------
-// Forward 3x3 convolution without an im2col copy, for images whose rows are a
-// whole number of 128-pixel tiles and Cin = 8 G (16, 32 or 64 channels).  An
-// output tile is 128 consecutive pixels of one image row.  For each tile the CTA
-// stages the three input rows that the tile reads, 130 pixels each (one pixel of
-// zero padding on either side), once in shared memory, laid out
-// [ky][channel group g][pixel][8 channels]: 8 consecutive pixels of one group form
-// one 128-byte core matrix.  The A operand of tap (ky, kx) and channels 16j..16j+15
-// is that slab seen from pixel kx: a K-major descriptor whose start address moves
-// 16 bytes per pixel, with 128 bytes between 8-pixel groups and 130 x 16 bytes
-// between the two channel groups of one MMA.  So every input element is staged
-// once per tile, where the im2col staging copies it nine times.  The weights of
-// all nine taps for the CTA's BN output channels are staged once per CTA,
-// [tap][g][co][8 channels].  The CTA is persistent over tiles: the slab of the
-// next tile is copied (cp.async, zero fill outside the image) while the tensor
-// core works on the current one, and two accumulators in tensor memory let the
-// epilogue of one tile run while the next accumulates.  Every wait is bounded;
-// on a time-out the kernel sets g_tc_error, waits (bounded) for its own MMAs and
-// copies, frees its tensor memory and returns.
-// ---------------------------------------------------------------------------
-constexpr int kSlabW = kTM + 2;  // staged pixels per input row
-
-__host__ __device__ constexpr uint32_t slab_bytes(int G) {
-    return (uint32_t)((3 * G * kSlabW * 16 + 127) / 128 * 128);
-}
-
-template <int BN, int G>
-__global__ void __launch_bounds__(kTcThreads) conv3x3_slab_kernel(const __nv_bfloat16 *__restrict__ in,
-                                                                  const __nv_bfloat16 *__restrict__ w,
-                                                                  const float *__restrict__ bias,
-                                                                  __nv_bfloat16 *__restrict__ out, int N, int H,
-                                                                  int Wd, int Cout, int relu) {
-    constexpr int Cin = 8 * G;
-    constexpr int kAcc = BN < 32 ? 32 : BN;  // TMEM columns of one accumulator
-    constexpr int kCols = 2 * kAcc;
-    constexpr uint32_t kSlab = slab_bytes(G);
-    extern __shared__ __align__(128) unsigned char sl_smem[];
-    unsigned char *const Wsm = sl_smem + 2 * kSlab;
-    __shared__ __align__(8) uint64_t mbar[2];
-    __shared__ uint32_t tmem_slot;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int n0 = blockIdx.y * BN;
-    const int tiles_x = Wd / kTM;
-    const long long ntiles = (long long)N * H * tiles_x;
-
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
-                     "r"(kCols)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mbar[0])) : "memory");
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mbar[1])) : "memory");
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = tmem_slot;
-
-    // weights: W[n0 + co][t][8g .. 8g + 7] -> Wsm[(t G + g) BN + co]
-    for (int e = tid; e < 9 * G * BN; e += kTcThreads) {
-        const int g = e % G, co = (e / G) % BN, t = e / (G * BN);
-        cp_async16(Wsm + ((t * G + g) * BN + co) * 16, w + ((long long)(n0 + co) * 9 + t) * Cin + 8 * g, 16);
-    }
-    // the three input rows of a tile, channel group fastest (coalesced reads)
-    const auto stage = [&](long long tile, unsigned char *dst) {
-        const int tx = (int)(tile % tiles_x);
-        const long long ry = tile / tiles_x;
-        const int y = (int)(ry % H), n = (int)(ry / H), x0 = tx * kTM;
-        for (int e = tid; e < 3 * G * kSlabW; e += kTcThreads) {
-            const int g = e % G, px = (e / G) % kSlabW, ky = e / (G * kSlabW);
-            const int sy = y + ky - 1, sx = x0 + px - 1;
-            const bool inside = sy >= 0 && sy < H && sx >= 0 && sx < Wd;
-            const __nv_bfloat16 *src = inside ? in + (((long long)n * H + sy) * Wd + sx) * Cin + 8 * g : in;
-            cp_async16(dst + ((ky * G + g) * kSlabW + px) * 16, src, inside ? 16 : 0);
-        }
-    };
-    const auto epilogue = [&](long long tile, int acc) {
-        const int tx = (int)(tile % tiles_x);
-        const long long row = tile / tiles_x;  // n H + y
-        const long long p = row * Wd + tx * kTM + warp * 32 + lane;
-#pragma unroll
-        for (int c = 0; c < BN; c += 8) {
-            uint32_t r[8];
-            asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-                           "=r"(r[7])
-                         : "r"(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(acc * kAcc + c)));
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            __align__(16) __nv_bfloat16 o[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                float v = __uint_as_float(r[q]);
-                if (bias) v += bias[n0 + c + q];
-                if (relu) v = fmaxf(v, 0.f);
-                o[q] = __float2bfloat16_rn(v);
-            }
-            *reinterpret_cast<uint4 *>(out + p * Cout + n0 + c) = *reinterpret_cast<const uint4 *>(o);
-        }
-    };
-
-    constexpr uint32_t idesc = mma_idesc(kTM, BN);
-    long long tile = blockIdx.x;
-    if (tile < ntiles) stage(tile, sl_smem);
-    cp_async_commit();  // the weights and the first slab
-    bool ok = true;
-    int i = 0;
-    long long prev = -1;
-    for (; tile < ntiles; tile += gridDim.x, ++i) {
-        const int b = i & 1;
-        cp_async_wait<0>();
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncthreads();
-        if (tid == 0) {
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t a0 = smem_u32(sl_smem + b * kSlab), w0 = smem_u32(Wsm);
-            int k = 0;
-#pragma unroll
-            for (int t = 0; t < 9; ++t) {
-                const int ky = t / 3, kx = t % 3;
-#pragma unroll
-                for (int j = 0; j < G / 2; ++j, ++k) {
-                    const uint64_t ad = smem_desc(a0 + (uint32_t)(((ky * G + 2 * j) * kSlabW + kx) * 16), kSlabW * 16, 128);
-                    const uint64_t bd = smem_desc(w0 + (uint32_t)((t * G + 2 * j) * BN * 16), BN * 16, 128);
-                    const uint32_t accum = k > 0 ? 1u : 0u;
-                    asm volatile(
-                        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem + (uint32_t)(b * kAcc)),
-                        "l"(ad), "l"(bd), "r"(idesc), "r"(accum)
-                        : "memory");
-                }
-            }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                             smem_u32(&mbar[b]))
-                         : "memory");
-        }
-        // the previous tile's MMAs: done -> its slab buffer and accumulator are free
-        if (i > 0) {
-            const bool mine = ok && mbar_wait(smem_u32(&mbar[b ^ 1]), (uint32_t)(((i - 1) >> 1) & 1));
-            ok = __syncthreads_and(mine) != 0;  // one decision for the whole CTA
-        }
-        const long long next = tile + gridDim.x;
-        if (ok && next < ntiles) stage(next, sl_smem + (b ^ 1) * kSlab);
-        cp_async_commit();
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        if (ok && i > 0) epilogue(prev, b ^ 1);
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        prev = tile;
-        if (!ok) {
-            ++i;
-            break;
-        }
-    }
-    // the last tile (its commit tracks every earlier MMA of the issuing thread;
-    // waited for also after a time-out, before the tensor memory is freed)
-    if (i > 0) {
-        const bool done = mbar_wait(smem_u32(&mbar[(i - 1) & 1]), (uint32_t)(((i - 1) >> 1) & 1));
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        if (ok && done) epilogue(prev, (i - 1) & 1);
-    }
-    cp_async_wait<0>();
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols) : "memory");
-}
-
-template <int BN, int G>
-cudaError_t launch_conv_slab(const __nv_bfloat16 *in, const __nv_bfloat16 *w, const float *bias, __nv_bfloat16 *out,
-                             int N, int H, int W, int Cout, int relu, cudaStream_t s) {
-    const size_t smem = 2 * (size_t)slab_bytes(G) + 9 * (size_t)G * BN * 16;
-    cudaError_t e = cudaFuncSetAttribute(conv3x3_slab_kernel<BN, G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    // the whole unified L1 / shared memory as shared memory, so that several CTAs fit on an SM
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(conv3x3_slab_kernel<BN, G>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 (int)cudaSharedmemCarveoutMaxShared);
-    if (e != cudaSuccess) return e;
-    int dev = 0, sms = 0, smem_sm = 0;
-    e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-    if (e != cudaSuccess) return e;
-    // CTAs per SM (the persistent grid): as many as the shared memory (1 KB reserved a
-    // CTA) and the tensor memory (512 columns per SM, two accumulators a CTA) hold; 48
-    // registers a thread never limit it.  (The occupancy query answered one CTA per SM
-    // here, which left two thirds of the SMs' slots empty: 142 against 93 us.)
-    const int per_sm = std::max(1, std::min((int)(smem_sm / (smem + 1024)), 512 / (2 * (BN < 32 ? 32 : BN))));
-    const long long tiles = (long long)N * H * (W / kTM);
-    const int gx = (int)std::max<long long>(1, std::min<long long>(tiles, (long long)sms * per_sm / (Cout / BN)));
-    dim3 grid(gx, Cout / BN);
-    conv3x3_slab_kernel<BN, G><<<grid, kTcThreads, smem, s>>>(in, w, bias, out, N, H, W, Cout, relu);
-    return cudaGetLastError();
-}
-
-// The slab kernel's shapes: forward, rows of whole 128-pixel tiles, Cin 16, 32 or 64.
-bool slab_shape(int W, int Cin_g, int Cout_g) {
-    return W % kTM == 0 && (Cin_g == 16 || Cin_g == 32 || Cin_g == 64) && Cout_g % 16 == 0;
-}
-
-cudaError_t conv_dispatch_slab(const __nv_bfloat16 *in, const __nv_bfloat16 *w, const float *bias, __nv_bfloat16 *out,
-                               int N, int H, int W, int Cin_g, int Cout_g, int relu, cudaStream_t s) {
-    // (for 64 input channels at most 64 output channels a CTA: the staged weights of
-    // 128 would not fit beside the two slabs)
-    int BN = Cout_g % 128 == 0 ? 128 : (Cout_g % 64 == 0 ? 64 : (Cout_g % 32 == 0 ? 32 : 16));
-    if (Cin_g == 64 && BN > 64) BN = 64;
-#define CDF_SLAB(G, WIDE)                                                                               \
-    switch (BN) {                                                                                       \
-        case 128: return launch_conv_slab<WIDE, G>(in, w, bias, out, N, H, W, Cout_g, relu, s);         \
-        case 64: return launch_conv_slab<64, G>(in, w, bias, out, N, H, W, Cout_g, relu, s);            \
-        case 32: return launch_conv_slab<32, G>(in, w, bias, out, N, H, W, Cout_g, relu, s);            \
-        default: return launch_conv_slab<16, G>(in, w, bias, out, N, H, W, Cout_g, relu, s);            \
-    }
-    if (Cin_g == 16) CDF_SLAB(2, 128)
-    if (Cin_g == 32) CDF_SLAB(4, 128)
-    CDF_SLAB(8, 64)  // BN is at most 64 here
-#undef CDF_SLAB
-}
+#include "nn_conv.cuh"  // the convolutions without im2col copies (the default path)
 
 template <bool kBwdData, int BN>
 cudaError_t launch_conv_tc_pipe(const __nv_bfloat16 *in, const __nv_bfloat16 *w, const float *bias,
@@ -1006,10 +791,10 @@ cudaError_t launch_conv_tc(const __nv_bfloat16 *in, const __nv_bfloat16 *w, cons
     return cudaGetLastError();
 }
 
-// Convolution path: 1 = tcgen05, the faster staging per shape (default), 2 = tcgen05
-// with synchronous staging, 3 = tcgen05 persistent warp-specialised forward,
-// 4 = the forward without im2col copy (conv3x3_slab_kernel) where the shape allows it,
-// else as 1, 0 = the warp-level MMA kernels.
+// Convolution path: 1 = tcgen05 without im2col copy (conv3x3_lin_kernel) where the
+// staged positions fit in shared memory, else the faster im2col staging per shape
+// (default; 4 is the same), 2 = tcgen05 with synchronous im2col staging, 3 = tcgen05
+// persistent warp-specialised forward, 0 = the warp-level MMA kernels.
 int g_path = 1;
 bool g_use_tc = true;
 
@@ -1028,8 +813,11 @@ template <bool kBwdData>
 cudaError_t conv_dispatch(const __nv_bfloat16 *in, const __nv_bfloat16 *w, const float *bias, __nv_bfloat16 *out,
                           int N, int H, int W, int Cin_g, int Cout_g, int relu, cudaStream_t s) {
     const int BN = Cout_g % 128 == 0 ? 128 : (Cout_g % 64 == 0 ? 64 : (Cout_g % 32 == 0 ? 32 : 16));
-    if ((g_path == 1 || g_path == 4) && !kBwdData && slab_shape(W, Cin_g, Cout_g))
-        return conv_dispatch_slab(in, w, bias, out, N, H, W, Cin_g, Cout_g, relu, s);
+    if (g_path == 1 || g_path == 4) {
+        bool ran = false;
+        const cudaError_t e = conv_lin<kBwdData>(in, w, bias, out, N, H, W, Cin_g, Cout_g, relu, s, &ran);
+        if (ran) return e;
+    }
     if (g_path == 3 && !kBwdData) {  // forward: the persistent warp-specialised kernel
         switch (BN) {
             case 128: return launch_conv_ws<128, 4>(in, w, bias, out, N, H, W, Cin_g, Cout_g, relu, s);
@@ -1037,7 +825,7 @@ cudaError_t conv_dispatch(const __nv_bfloat16 *in, const __nv_bfloat16 *w, const
             default: return launch_conv_ws<32, 6>(in, w, bias, out, N, H, W, Cin_g, Cout_g, relu, s);
         }
     }
-    // the default picks by the measured faster form: the cp.async pipeline for long K
+    // im2col staging: the cp.async pipeline for long K
     // (Cin >= 128, e.g. 159 against 101 TFLOP/s at 32^2 x 256 -> 256), two-buffer
     // synchronous staging for short K, where more CTAs per SM hide more latency
     // (80 against 72 TFLOP/s at 256^2 x 32 -> 32)
@@ -1127,303 +915,57 @@ __global__ void __launch_bounds__(kThreads) conv3x3_wgrad_kernel(const __nv_bflo
     }
 }
 
-// ---------------------------------------------------------------------------
-// 3x3 convolution, weight gradient, on the tcgen05 tensor cores with a
-// deterministic split over the pixels:
-//   dW[co][t][ci] = sum_p dY[p][co] X[p + d(t)][ci].
-// GEMM: M = 9 Cin rows m = t Cin + ci (tile 128), N = Cout (one tile, <= 256),
-// K = pixels in stages of 64, split over blockIdx.y into `splits` contiguous
-// pixel ranges.  Both operands are channel-contiguous in memory (NHWC) while the
-// MMA reads K-major tiles, so each thread stages an 8 x 8 block -- 8 rows (8
-// consecutive channels) x 8 pixels -- with eight 16-byte loads, transposes it in
-// registers and writes eight 16-byte K-major rows.  Each split writes its FP32
-// partial tile to the workspace; wgrad_reduce_kernel then adds the splits in a
-// fixed order (no atomics: the result is the same bits on every run).
-// ---------------------------------------------------------------------------
-// 8 x 8 BF16 transpose: in[k] holds channels 0..7 of pixel k; out[c] holds
-// pixels 0..7 of channel c.
-__device__ __forceinline__ void transpose8x8(const uint4 (&in)[8], uint4 (&out)[8]) {
-    const __nv_bfloat16 *e = reinterpret_cast<const __nv_bfloat16 *>(in);
-    __nv_bfloat16 *o = reinterpret_cast<__nv_bfloat16 *>(out);
-#pragma unroll
-    for (int c = 0; c < 8; ++c)
-#pragma unroll
-        for (int k = 0; k < 8; ++k) o[c * 8 + k] = e[k * 8 + c];
-}
-
-template <int BN, int MT>
-__global__ void __launch_bounds__(kTcThreads) conv3x3_wgrad_tc_kernel(const __nv_bfloat16 *__restrict__ x,
-                                                                      const __nv_bfloat16 *__restrict__ dy,
-                                                                      float *__restrict__ part, int N, int H, int Wd,
-                                                                      int Cin, int Cout, long long pix_per_split) {
-    // MT accumulators of 128 x BN in tensor memory, columns mt * BN (a power of two >= 32 allocated)
-    constexpr int kNeed = MT * BN;
-    constexpr int kCols = kNeed <= 32 ? 32 : (kNeed <= 64 ? 64 : (kNeed <= 128 ? 128 : (kNeed <= 256 ? 256 : 512)));
-    constexpr uint32_t kABytes = kTM * kTK * 2, kBBytes = BN * kTK * 2;
-    extern __shared__ __align__(128) unsigned char tc_smem[];
-    unsigned char *A = tc_smem;                     // [2 stages][MT tiles][kABytes]
-    unsigned char *B = tc_smem + 2 * MT * kABytes;  // [2 stages][kBBytes]
-    __shared__ __align__(8) uint64_t mbar[2];
-    __shared__ uint32_t tmem_slot;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const long long P = (long long)N * H * Wd;
-    const int M = 9 * Cin, mtiles = (M + kTM - 1) / kTM;
-    const int t0 = blockIdx.x * MT, n0 = blockIdx.z * BN;
-    const int nt = mtiles - t0 < MT ? mtiles - t0 : MT;  // M tiles of this CTA (>= 1)
-    const long long pbeg = (long long)blockIdx.y * pix_per_split;
-    const long long pend = pbeg + pix_per_split < P ? pbeg + pix_per_split : P;
-    const int nst = (int)((pend - pbeg + kTK - 1) / kTK);
-
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
-                     "r"(kCols)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+// dw[i] += sum_{split} part[split][i] and db[c] += sum_{split} bpart[split][c], each in
+// a fixed order: a block of 256 threads covers 32 runs of four values, eight
+// threads a run, each with an eighth of the splits, added in order; the eight
+// sums are then added in order.  (One thread per run would walk up to 132 splits
+// one load after the other.)  Blocks from `wblocks` on take the bias.
+__global__ void __launch_bounds__(256) weight_sum_kernel(const float *__restrict__ part, float *__restrict__ dw,
+                                                         int n4, int splits, int wblocks,
+                                                         const float *__restrict__ bpart, float *__restrict__ db,
+                                                         int c4, int bsplits) {
+    const bool bias = (int)blockIdx.x >= wblocks;
+    const float4 *src = reinterpret_cast<const float4 *>(bias ? bpart : part);
+    float *dst = bias ? db : dw;
+    const int n = bias ? c4 : n4, ns = bias ? bsplits : splits;
+    const int i = (blockIdx.x - (bias ? wblocks : 0)) * 32 + (threadIdx.x & 31), sl = threadIdx.x >> 5;
+    const int z0 = (int)((long long)ns * sl / 8), z1 = (int)((long long)ns * (sl + 1) / 8);
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (i < n) {
+#pragma unroll 8
+        for (int z = z0; z < z1; ++z) {
+            const float4 v = __ldg(src + (long long)z * n + i);
+            a.x += v.x;
+            a.y += v.y;
+            a.z += v.z;
+            a.w += v.w;
+        }
     }
-    if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mbar[0])) : "memory");
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mbar[1])) : "memory");
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __shared__ float4 red[8][32];
+    red[sl][threadIdx.x & 31] = a;
     __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = tmem_slot;
-
-    // this thread's A block in each M tile: rows (t0 + mt) * 128 + mg * 8 .. + 7 (one tap, eight
-    // consecutive channels), pixels kg * 8 .. + 7 of the stage
-    const int mg = tid >> 3, kg = tid & 7;
-    int ddy[MT], ddx[MT], cib[MT];
-    bool rok[MT];
+    if (sl == 0 && i < n) {
 #pragma unroll
-    for (int mt = 0; mt < MT; ++mt) {
-        const int ma = (t0 + mt) * kTM + mg * 8;
-        rok[mt] = mt < nt && ma < M;  // M is a multiple of 8 (Cin % 16 == 0)
-        const int tap = rok[mt] ? ma / Cin : 0;
-        cib[mt] = rok[mt] ? ma - tap * Cin : 0;
-        ddy[mt] = tap / 3 - 1;
-        ddx[mt] = tap % 3 - 1;
-    }
-    const long long hw = (long long)H * Wd;
-    constexpr uint32_t idesc = mma_idesc(kTM, BN);
-    bool ok = true;
-    int last = -1;
-    for (int s = 0; s < nst && ok; ++s) {
-        const int buf = s & 1;
-        if (s >= 2) ok = mbar_wait(smem_u32(&mbar[buf]), (uint32_t)(((s - 2) >> 1) & 1));
-        if (!ok) break;
-        unsigned char *Bs = B + buf * kBBytes;
-        const long long pk = pbeg + (long long)s * kTK + kg * 8;
-        // image coordinates of this thread's eight pixels (one division per stage, then a walk)
-        int pn[8], py[8], px[8];
-        {
-            int n = (int)(pk / hw);
-            const int rem = (int)(pk - (long long)n * hw);
-            int yy = rem / Wd, xx = rem - (rem / Wd) * Wd;
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                pn[k] = n;
-                py[k] = yy;
-                px[k] = xx;
-                if (++xx == Wd) {
-                    xx = 0;
-                    if (++yy == H) {
-                        yy = 0;
-                        ++n;
-                    }
-                }
-            }
+        for (int k = 1; k < 8; ++k) {
+            const float4 v = red[k][threadIdx.x];
+            a.x += v.x;
+            a.y += v.y;
+            a.z += v.z;
+            a.w += v.w;
         }
-        // A: X at the tap-shifted pixels, 8 channels each (zero outside the image, the range or M)
-#pragma unroll
-        for (int mt = 0; mt < MT; ++mt) {
-            if (mt >= nt) break;
-            uint4 v[8], t[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                v[k] = make_uint4(0, 0, 0, 0);
-                const int yy = py[k] + ddy[mt], xx = px[k] + ddx[mt];
-                if (rok[mt] && pk + k < pend && yy >= 0 && yy < H && xx >= 0 && xx < Wd)
-                    v[k] = *reinterpret_cast<const uint4 *>(x + (((long long)pn[k] * H + yy) * Wd + xx) * Cin + cib[mt]);
-            }
-            transpose8x8(v, t);
-            unsigned char *As = A + (buf * MT + mt) * kABytes;
-#pragma unroll
-            for (int c = 0; c < 8; ++c) *reinterpret_cast<uint4 *>(As + cm_offset(mg * 8 + c, kg * 8, kTM)) = t[c];
-        }
-        // B: dY rows of the same pixels, 8 output channels per block, spread from the last thread
-        // down (the first threads carry the most A work when the last M tile is partial)
-        for (int e = kTcThreads - 1 - tid; e < (BN / 8) * 8; e += kTcThreads) {
-            const int ng = e >> 3, kb = e & 7;
-            const long long pb = pbeg + (long long)s * kTK + kb * 8;
-            uint4 v[8], t[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                v[k] = make_uint4(0, 0, 0, 0);
-                if (pb + k < pend) v[k] = *reinterpret_cast<const uint4 *>(dy + (pb + k) * Cout + n0 + ng * 8);
-            }
-            transpose8x8(v, t);
-#pragma unroll
-            for (int c = 0; c < 8; ++c) *reinterpret_cast<uint4 *>(Bs + cm_offset(ng * 8 + c, kb * 8, BN)) = t[c];
-        }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncthreads();
-        if (tid == 0) {
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t b0 = smem_u32(Bs);
-#pragma unroll
-            for (int mt = 0; mt < MT; ++mt) {
-                if (mt >= nt) break;
-                const uint32_t a0 = smem_u32(A + (buf * MT + mt) * kABytes);
-#pragma unroll
-                for (int j = 0; j < kTK / 16; ++j) {
-                    const uint64_t ad = smem_desc(a0 + 2 * j * (kTM / 8) * 128, (kTM / 8) * 128, 128);
-                    const uint64_t bd = smem_desc(b0 + 2 * j * (BN / 8) * 128, (BN / 8) * 128, 128);
-                    const uint32_t acc = (s > 0 || j > 0) ? 1u : 0u;
-                    asm volatile(
-                        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem + (uint32_t)(mt * BN)),
-                        "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
-                        : "memory");
-                }
-            }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                             smem_u32(&mbar[buf]))
-                         : "memory");
-        }
-        last = s;
+        float *d = dst + 4ll * i;
+        d[0] += a.x;
+        d[1] += a.y;
+        d[2] += a.z;
+        d[3] += a.w;
     }
-    if (last >= 0) ok = mbar_wait(smem_u32(&mbar[last & 1]), (uint32_t)((last >> 1) & 1)) && ok;
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (ok) {
-        // TMEM lane = tile row; each tile's partial sums into part[split][m][co]
-        // (a split without pixels writes zeros)
-#pragma unroll
-        for (int mt = 0; mt < MT; ++mt) {
-            if (mt >= nt) break;
-            const int m = (t0 + mt) * kTM + warp * 32 + lane;
-            float *row = part + ((long long)blockIdx.y * M + m) * Cout + n0;
-#pragma unroll
-            for (int c = 0; c < BN; c += 8) {
-                uint32_t r[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-                if (nst > 0) {
-                    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
-                                   "=r"(r[6]), "=r"(r[7])
-                                 : "r"(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(mt * BN + c)));
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                }
-                if (m < M) {
-                    float4 *d = reinterpret_cast<float4 *>(row + c);
-                    d[0] = make_float4(__uint_as_float(r[0]), __uint_as_float(r[1]), __uint_as_float(r[2]),
-                                       __uint_as_float(r[3]));
-                    d[1] = make_float4(__uint_as_float(r[4]), __uint_as_float(r[5]), __uint_as_float(r[6]),
-                                       __uint_as_float(r[7]));
-                }
-            }
-        }
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols) : "memory");
 }
 
-// dW[co][m] += sum_{split = 0..splits-1} part[split][m][co], in that order.
-__global__ void wgrad_reduce_kernel(const float *__restrict__ part, float *__restrict__ dw, int M, int Cout,
-                                    int splits) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;  // i = co * M + m
-    if (i >= (long long)M * Cout) return;
-    const int co = (int)(i / M), m = (int)(i - (long long)co * M);
-    float acc = 0.f;
-    for (int z = 0; z < splits; ++z) acc += part[((long long)z * M + m) * Cout + co];
-    dw[i] += acc;
-}
-
-// Bias gradient with a fixed summation order, db[c] += sum_p dY[p][c], in two
-// passes: bias_partial_kernel gives each block of 256 threads 8 channels and one
-// run of `per` pixels (each thread a strided part of the run, then a tree in
-// shared memory) and writes its sums to part[split][c]; bias_sum_kernel adds the
-// splits in order.
-__global__ void bias_partial_kernel(const __nv_bfloat16 *__restrict__ dy, float *__restrict__ part, long long P,
-                                    int C, long long per) {
-    const int c0 = blockIdx.x * 8;
-    const long long p0 = (long long)blockIdx.y * per, p1 = min(P, p0 + per);
-    float s[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (long long p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
-        const uint4 v = *reinterpret_cast<const uint4 *>(dy + p * C + c0);
-        const __nv_bfloat16 *e = reinterpret_cast<const __nv_bfloat16 *>(&v);
-#pragma unroll
-        for (int q = 0; q < 8; ++q) s[q] += __bfloat162float(e[q]);
-    }
-    __shared__ float red[8][256];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) red[q][threadIdx.x] = s[q];
-    __syncthreads();
-    for (int st = blockDim.x / 2; st > 0; st >>= 1) {
-        if ((int)threadIdx.x < st)
-#pragma unroll
-            for (int q = 0; q < 8; ++q) red[q][threadIdx.x] += red[q][threadIdx.x + st];
-        __syncthreads();
-    }
-    if (threadIdx.x < 8) part[(long long)blockIdx.y * C + c0 + threadIdx.x] = red[threadIdx.x][0];
-}
-
-__global__ void bias_sum_kernel(const float *__restrict__ part, float *__restrict__ db, int C, int splits) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= C) return;
-    float acc = 0.f;
-    for (int z = 0; z < splits; ++z) acc += part[(long long)z * C + c];
-    db[c] += acc;
-}
-
-// Pixel splits of the bias gradient: about two blocks per SM over the C / 8
-// channel groups, at least 2048 pixels a split.
-long long bias_splits(long long P, int C) {
-    const long long groups = C / 8;
-    long long s = (304 + groups - 1) / groups;
-    const long long cap = (P + 2047) / 2048;
-    if (s > cap) s = cap;
-    return s < 1 ? 1 : s;
-}
-
-// The weight gradient's tiling: output-channel tile BN (the largest of 256, 128,
-// 64, 32 that divides Cout); MT of the 128-row M tiles per CTA, which share each
-// staged tile of dY (at most 256 tensor-memory columns, MT * BN, and three tiles),
-// spread evenly over gx CTAs; pixel splits for about two CTAs per SM in all with at
-// least 16 stages of 64 pixels each, and the pixels per split (a multiple of 64;
-// no split is empty).
-struct WgradPlan {
-    int bn, mt, gx, splits;
-    long long per;
-};
-WgradPlan wgrad_plan(long long P, int Cin, int Cout) {
-    WgradPlan w;
-    w.bn = Cout % 256 == 0 ? 256 : (Cout % 128 == 0 ? 128 : (Cout % 64 == 0 ? 64 : 32));
-    const int mtiles = (9 * Cin + kTM - 1) / kTM;
-    const int mtmax = w.bn >= 256 ? 1 : (w.bn >= 128 ? 2 : 3);
-    w.gx = (mtiles + mtmax - 1) / mtmax;
-    w.mt = (mtiles + w.gx - 1) / w.gx;
-    const long long tiles = (long long)w.gx * (Cout / w.bn);
-    long long s = (304 + tiles - 1) / tiles;
-    const long long cap = (P + 16 * kTK - 1) / (16 * kTK);
-    if (s > cap) s = cap;
-    if (s < 1) s = 1;
-    w.per = ((P + s - 1) / s + kTK - 1) / kTK * kTK;
-    w.splits = (int)((P + w.per - 1) / w.per);
-    return w;
-}
-
-template <int BN, int MT>
-cudaError_t launch_wgrad_tc(const __nv_bfloat16 *x, const __nv_bfloat16 *dy, float *part, int N, int H, int W,
-                            int Cin, int Cout, const WgradPlan &w, cudaStream_t s) {
-    const size_t smem = 2 * MT * (size_t)(kTM * kTK * 2) + 2 * (size_t)(BN * kTK * 2);
-    cudaError_t e = cudaFuncSetAttribute(conv3x3_wgrad_tc_kernel<BN, MT>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    dim3 grid((unsigned)w.gx, (unsigned)w.splits, (unsigned)(Cout / BN));
-    conv3x3_wgrad_tc_kernel<BN, MT><<<grid, kTcThreads, smem, s>>>(x, dy, part, N, H, W, Cin, Cout, w.per);
-    return cudaGetLastError();
+// Images of one launch of the weight gradient: as many as keep the padded positions
+// below 2^30 (0: one image alone has more; the warp-level kernel takes it).
+int wgrad_images(int N, int H, int W) {
+    const long long one = ((long long)H + 1) * ((long long)W + 1);
+    return (int)std::min<long long>(N, ((1ll << 30) - 1) / one);
 }
 
 // ---------------------------------------------------------------------------
@@ -1676,9 +1218,10 @@ cdf_nn_status cdf_nn_conv3x3_bwd_data(const void *dy, const void *w, void *dx, i
 
 long long cdf_nn_conv3x3_bwd_weight_workspace(int N, int H, int W, int Cin, int Cout) {
     if (N < 1 || H < 1 || W < 1 || Cin < 16 || Cin % 16 || Cout < 32 || Cout % 32) return -1;
-    const long long P = (long long)N * H * W;
-    const WgradPlan w = wgrad_plan(P, Cin, Cout);
-    return ((long long)w.splits * 9 * Cin * Cout + bias_splits(P, Cout) * Cout) * (long long)sizeof(float);
+    const int images = wgrad_images(N, H, W);
+    if (images == 0) return 4;  // the warp-level kernel adds to dw directly
+    const WgLinPlan w = wgrad_lin_plan((long long)images * (H + 1) * (W + 1), (long long)images * H * W, Cin, Cout);
+    return ((long long)w.splits * 9 * Cin + w.bias_splits) * Cout * (long long)sizeof(float);
 }
 
 cdf_nn_status cdf_nn_conv3x3_bwd_weight(const void *x, const void *dy, float *dw, float *db, int N, int H, int W,
@@ -1689,32 +1232,26 @@ cdf_nn_status cdf_nn_conv3x3_bwd_weight(const void *x, const void *dy, float *dw
     auto s = static_cast<cudaStream_t>(stream);
     const auto *xb = static_cast<const __nv_bfloat16 *>(x);
     const auto *dyb = static_cast<const __nv_bfloat16 *>(dy);
-    if (g_use_tc) {
+    const int images = wgrad_images(N, H, W);
+    if (g_use_tc && images > 0) {
         const long long need = cdf_nn_conv3x3_bwd_weight_workspace(N, H, W, Cin, Cout);
         if (!workspace || workspace_bytes < need)
             return nn_fail("conv3x3_bwd_weight: the workspace is missing or smaller than "
                            "cdf_nn_conv3x3_bwd_weight_workspace()");
-        const WgradPlan w = wgrad_plan(P, Cin, Cout);
         float *part = static_cast<float *>(workspace);
-        cudaError_t e;
-        // M = 9 Cin >= 144 spans at least two tiles, so MT = 1 occurs only with BN = 256
-        switch (w.bn * 4 + w.mt) {
-            case 256 * 4 + 1: e = launch_wgrad_tc<256, 1>(xb, dyb, part, N, H, W, Cin, Cout, w, s); break;
-            case 128 * 4 + 2: e = launch_wgrad_tc<128, 2>(xb, dyb, part, N, H, W, Cin, Cout, w, s); break;
-            case 64 * 4 + 2: e = launch_wgrad_tc<64, 2>(xb, dyb, part, N, H, W, Cin, Cout, w, s); break;
-            case 64 * 4 + 3: e = launch_wgrad_tc<64, 3>(xb, dyb, part, N, H, W, Cin, Cout, w, s); break;
-            case 32 * 4 + 2: e = launch_wgrad_tc<32, 2>(xb, dyb, part, N, H, W, Cin, Cout, w, s); break;
-            case 32 * 4 + 3: e = launch_wgrad_tc<32, 3>(xb, dyb, part, N, H, W, Cin, Cout, w, s); break;
-            default: return nn_fail("conv3x3_bwd_weight: no kernel for this tiling");
-        }
-        if (e != cudaSuccess) { cudaGetLastError(); return nn_fail(cudaGetErrorString(e)); }
-        const long long n = 9LL * Cin * Cout;
-        wgrad_reduce_kernel<<<blocks_for(n), 256, 0, s>>>(part, dw, 9 * Cin, Cout, w.splits);
-        if (db) {
-            float *bpart = part + (long long)w.splits * 9 * Cin * Cout;  // after the weight partials
-            const long long bs = bias_splits(P, Cout), per = (P + bs - 1) / bs;
-            bias_partial_kernel<<<dim3(Cout / 8, (unsigned)bs), 256, 0, s>>>(dyb, bpart, P, Cout, per);
-            bias_sum_kernel<<<(Cout + 127) / 128, 128, 0, s>>>(bpart, db, Cout, (int)bs);
+        for (int n0 = 0; n0 < N; n0 += images) {
+            const int n = std::min(images, N - n0);
+            const long long Pn = (long long)n * H * W;
+            const auto *xn = xb + (long long)n0 * H * W * Cin, *dyn = dyb + (long long)n0 * H * W * Cout;
+            LinImage im;
+            if (!lin_image(n, H, W, &im)) return nn_fail("conv3x3_bwd_weight: too many positions");
+            const WgLinPlan w = wgrad_lin_plan(im.L, Pn, Cin, Cout);
+            float *bpart = db ? part + (long long)w.splits * 9 * Cin * Cout : nullptr;  // after the weight partials
+            const cudaError_t e = wgrad_lin(xn, dyn, part, bpart, im, Pn, Cin, Cout, w, s);
+            if (e != cudaSuccess) { cudaGetLastError(); return nn_fail(cudaGetErrorString(e)); }
+            const int n4 = 9 * Cin * Cout / 4, wblocks = (n4 + 31) / 32, bblocks = db ? (Cout / 4 + 31) / 32 : 0;
+            weight_sum_kernel<<<wblocks + bblocks, 256, 0, s>>>(part, dw, n4, w.splits, wblocks, bpart, db, Cout / 4,
+                                                                w.bias_splits);
         }
     } else {
         // the warp-level MMA path: split-K partial sums added atomically (order-dependent)

@@ -59,10 +59,10 @@ def nn_lib():
 
 
 def set_tensor_path(tcgen05):
-    """Convolutions on the 5th-generation tensor cores (True or 1, the default: the faster
-    staging per layer; 2: synchronous staging; 3: persistent warp-specialised forward;
-    4: the forward without im2col copy where the shape allows it) or on the warp-level
-    MMA kernels (False or 0)."""
+    """Convolutions on the 5th-generation tensor cores (True, 1 or 4, the default: without
+    im2col copies where the staged positions fit, else the faster im2col staging per layer;
+    2: synchronous im2col staging; 3: persistent warp-specialised im2col forward) or on the
+    warp-level MMA kernels (False or 0)."""
     _call("cdf_nn_set_tensor_path", int(tcgen05))
 
 
