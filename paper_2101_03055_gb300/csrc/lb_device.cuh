@@ -230,6 +230,35 @@ __device__ __forceinline__ F2 vrsqrt(F2 a) { return pack2(rsqrtf(a.v.x), rsqrtf(
 __device__ __forceinline__ float vstep(float a, float t) { return a >= t ? 1.f : 0.f; }
 __device__ __forceinline__ F2 vstep(F2 a, float t) { return pack2(vstep(a.v.x, t), vstep(a.v.y, t)); }
 
+// ---- closure kinds -----------------------------------------------------------------
+// Which terms of the model a lattice uses, as a template argument K of the node
+// update: kAnyClosure decides by the parameters at run time, a set of the bits below
+// compiles the terms that are absent out of the kernel.  They are exact zeros there
+// (a source that is 0, a force whose g is 0, omega_10 = 0, a reference gradient of 0),
+// so every kind gives the bits of kAnyClosure.  The update is bound by the
+// instructions it issues: without the absent terms the two-step kernel executes 427
+// instead of 500 warp instructions per 32 updates of the cavity.  closure_kind()
+// (lb_kernels.cu) picks the kind of a lattice.
+constexpr int kAnyClosure = -1;
+constexpr int kChemo = 1;    // D_01 += -chi phi_0 r(phi_1)
+constexpr int kConsume = 2;  // S_1 = -k phi_0 r(phi_1)
+constexpr int kForce = 4;    // g != 0
+constexpr int kShift = 8;    // the fluid's deviations refer to a pressure gradient G != 0
+// omega_10 = 0, as for every diagonal constant part: the lower left entry of the
+// relaxation matrix stays 0 and its diagonal the constant one
+constexpr int kUpper = 16;
+// Kinds without kConsume have no source, kinds other than kAnyClosure no second-order force.
+template <int K>
+__device__ __forceinline__ constexpr bool closure_has(int bit, bool at_run_time) {
+    return K < 0 ? at_run_time : (K & bit) != 0;
+}
+
+// p_ref at the node (0 in a kind without a reference gradient)
+template <int K>
+__device__ __forceinline__ float node_pref(const LbParams &p, int x, int y) {
+    return K < 0 || (K & kShift) ? pref_at(p, x, y) : 0.f;
+}
+
 // c_i . (ax, ay) for a lattice direction (components 0 or +-1, at least one
 // nonzero), without multiplications by the components.
 template <class V>
@@ -324,7 +353,7 @@ template <int M, class V = float>
 struct ScalarState {
     V phid[M], phi[M], S[M], Sp[M], r;
 };
-template <int M, class V>
+template <int M, int K = kAnyClosure, class V>
 __device__ __forceinline__ void scalar_closures(const LbParams &p, const V (&f)[M][5], V sp1, bool first,
                                                 ScalarState<M, V> &s) {
 #pragma unroll
@@ -333,13 +362,14 @@ __device__ __forceinline__ void scalar_closures(const LbParams &p, const V (&f)[
         s.phi[a] = p.phi_ref[a] + s.phid[a];
     }
     s.r = splat<V>(0.f);
-    if (M >= 2 && (p.chemotaxis || p.skind == 2)) s.r = cutoff(p, s.phi[M >= 2 ? 1 : 0]);
+    const bool consume = closure_has<K>(kConsume, p.skind == 2);
+    if (M >= 2 && (closure_has<K>(kChemo, p.chemotaxis) || consume)) s.r = cutoff(p, s.phi[M >= 2 ? 1 : 0]);
 #pragma unroll
     for (int a = 0; a < M; ++a) {
-        s.S[a] = splat<V>((p.skind == 1) ? p.S[a] : 0.f);
+        s.S[a] = splat<V>(closure_has<K>(0, p.skind == 1) ? p.S[a] : 0.f);
         s.Sp[a] = s.S[a];
     }
-    if (M >= 2 && p.skind == 2) {
+    if (M >= 2 && consume) {
         s.S[1] = -p.k * s.phi[0] * s.r;
         s.Sp[1] = first ? s.S[1] : sp1;
     }
@@ -347,13 +377,20 @@ __device__ __forceinline__ void scalar_closures(const LbParams &p, const V (&f)[
 
 // Eq. omega-D.  Constant D: omega from the host.  Chemotaxis: omega^-1 =
 // B + delta e_0 e_1^T with delta = -3 chi phi_0 r, inverted by Sherman-Morrison.
-template <int M, class V>
+template <int M, int K = kAnyClosure, class V>
 __device__ __forceinline__ void relaxation_matrix(const LbParams &p, const ScalarState<M, V> &s, V (&om)[M][M]) {
 #pragma unroll
     for (int a = 0; a < M; ++a)
 #pragma unroll
         for (int b = 0; b < M; ++b) om[a][b] = splat<V>(p.omega[a * M + b]);
-    if (M >= 2 && p.chemotaxis) {
+    if (M >= 2 && K >= 0 && (K & kUpper)) {
+        // omega_10 = 0: of delta (omega e_0)(e_1^T omega) only the entry (0, 1) is left
+        om[M >= 2 ? 1 : 0][0] = splat<V>(0.f);
+        if (K & kChemo) {
+            const V delta = -p.chi3 * s.phi[0] * s.r;
+            om[0][M >= 2 ? 1 : 0] = vfma(-vmul(delta, p.omega[0]), p.omega[M >= 2 ? M + 1 : 0], om[0][M >= 2 ? 1 : 0]);
+        }
+    } else if (M >= 2 && closure_has<K>(kChemo, p.chemotaxis)) {
         const V delta = -p.chi3 * s.phi[0] * s.r;
         // 1 / (1 + delta omega_10); omega_10 = 0 (a diagonal constant part, as in
         // the benchmark closures) makes it exactly 1, so the quotient is skipped
@@ -380,7 +417,7 @@ __device__ __forceinline__ void relaxation_matrix(const LbParams &p, const Scala
 // difference of phi u in Case 1 of Sec. 2.1).  The non-equilibrium part f - f^eq
 // is formed first, so a node at equilibrium stays there exactly (no rounding-level
 // forcing of the conserved scalar mass).
-template <int M, class V>
+template <int M, int K = kAnyClosure, bool kAux = true, class V>
 __device__ __forceinline__ void scalar_collide(V (&f)[M][5], const ScalarState<M, V> &s, V ux, V uy,
                                                const V (&om)[M][M], const V (&Jx)[M], const V (&Jy)[M]) {
     V feq[M][5];
@@ -394,9 +431,15 @@ __device__ __forceinline__ void scalar_collide(V (&f)[M][5], const ScalarState<M
         for (int a = 0; a < M; ++a) {
             V coll = splat<V>(0.f);
 #pragma unroll
-            for (int b = 0; b < M; ++b) coll = vfma(om[a][b], neq[b], coll);
-            const V G = (i == 0) ? splat<V>(0.f) : vmul(3.f * kW5, cdot(kC5x(i), kC5y(i), Jx[a], Jy[a]));
-            f[a][i] = (f[a][i] - coll) + vfma(kWs(i), vfma(1.5f, s.S[a], vmul(-0.5f, s.Sp[a])), G);
+            for (int b = 0; b < M; ++b)
+                if (!(K >= 0 && (K & kUpper) && a == 1 && b == 0)) coll = vfma(om[a][b], neq[b], coll);
+            f[a][i] = f[a][i] - coll;
+            // kAux: the auxiliary source is not identically zero
+            const bool source = K < 0 || ((K & kConsume) && a == 1);
+            V G = splat<V>(0.f);
+            if (kAux && i != 0) G = vmul(3.f * kW5, cdot(kC5x(i), kC5y(i), Jx[a], Jy[a]));
+            if (source) G = vfma(kWs(i), vfma(1.5f, s.S[a], vmul(-0.5f, s.Sp[a])), G);
+            if (source || (kAux && i != 0)) f[a][i] = f[a][i] + G;
         }
     }
 }
@@ -405,32 +448,39 @@ __device__ __forceinline__ void scalar_collide(V (&f)[M][5], const ScalarState<M
 // f, h: pre-collision deviations, overwritten by the post-collision ones.  prx:
 // p_ref at the node.  sp1: S_1(t-1) of the consumption closure; `first` uses
 // S(t-1) = S(t) (initialisation).  V = F2: two nodes, one per lane.
-template <int M, class V>
+template <int M, int K = kAnyClosure, class V>
 __device__ __forceinline__ void collide(const LbParams &p, V (&f)[M][5], V (&h)[9], V prx, V sp1, bool first,
                                         NodeOut<M, V> &o) {
     ScalarState<M, V> s;
-    scalar_closures<M>(p, f, sp1, first, s);
-    V fm = splat<V>(p.Fbase);
+    constexpr bool kWithForce = K < 0 || (K & kForce);
+    const bool second = closure_has<K>(0, p.varphi != 0.f);
+    scalar_closures<M, K>(p, f, sp1, first, s);
+    V Fx = splat<V>(0.f), Fy = splat<V>(0.f);
+    if (kWithForce) {
+        V fm = splat<V>(p.Fbase);
 #pragma unroll
-    for (int a = 0; a < M; ++a) fm = vfma(p.beta[a], s.phi[a], fm);
-    const V Fx = p.g[0] * fm, Fy = p.g[1] * fm;
+        for (int a = 0; a < M; ++a) fm = vfma(p.beta[a], s.phi[a], fm);
+        Fx = p.g[0] * fm;
+        Fy = p.g[1] * fm;
+    }
 
     // Eq. sum-u and Eq. sum-p (varphi = 0):
     // p = cs^2/(1 - W0) [sum_{i!=0} h_i - W0 u.u / (2 cs^2)] = (sum_{i!=0} h_i - kQ u.u) / kC,
     // taken as a product with fl(1 / kC) (one rounding more than the quotient)
     const V jx = (h[1] - h[3]) + (h[5] - h[6]) + (h[8] - h[7]);
     const V jy = (h[2] - h[4]) + (h[5] - h[8]) + (h[6] - h[7]);
-    const V ux = vfma(0.5f, Fx, jx), uy = vfma(0.5f, Fy, jy);
+    const V ux = kWithForce ? vfma(0.5f, Fx, jx) : jx, uy = kWithForce ? vfma(0.5f, Fy, jy) : jy;
     const V usq = usq_of(ux, uy);
     const V snr = ((h[1] + h[2]) + (h[3] + h[4])) + ((h[5] + h[6]) + (h[7] + h[8]));
     V prd = vmul(vfma(-kQ, usq, snr), kInvC);
     // varphi != 0 (a branch uniform over the launch): the appendix's pressure,
     // p = (sum_{i!=0} h_i - kQ u.u - varphi (1/omega - 1/2) (W_0/cs^2) u.F) / kC
-    const V uF = vfma(ux, Fx, vmul(uy, Fy));
-    if (p.varphi != 0.f) prd = vmul(vfma(-p.varphi_p, uF, vfma(-kQ, usq, snr)), kInvC);
+    V uF = splat<V>(0.f);
+    if (second) uF = vfma(ux, Fx, vmul(uy, Fy));
+    if (second) prd = vmul(vfma(-p.varphi_p, uF, vfma(-kQ, usq, snr)), kInvC);
 
     V om[M][M];
-    relaxation_matrix<M>(p, s, om);
+    relaxation_matrix<M, K>(p, s, om);
 
     // Eq. Gi: G_{i,a} = 3 W_i c_i . J_a,  J_a = sum_b (delta_ab - omega_ab / 2)(u S_b + phi_b F)
     V Jx[M], Jy[M];
@@ -439,14 +489,19 @@ __device__ __forceinline__ void collide(const LbParams &p, V (&f)[M][5], V (&h)[
         V jxa = splat<V>(0.f), jya = splat<V>(0.f);
 #pragma unroll
         for (int b = 0; b < M; ++b) {
+            if (K >= 0 && (K & kUpper) && a == 1 && b == 0) continue;
+            const bool source = K < 0 || ((K & kConsume) && b == 1);
             const V c = vfma(-0.5f, om[a][b], a == b ? 1.f : 0.f);
-            jxa = vfma(c, vfma(ux, s.S[b], s.phi[b] * Fx), jxa);
-            jya = vfma(c, vfma(uy, s.S[b], s.phi[b] * Fy), jya);
+            V qx = s.phi[b] * Fx, qy = s.phi[b] * Fy;
+            if (source) qx = vfma(ux, s.S[b], qx);
+            if (source) qy = vfma(uy, s.S[b], qy);
+            jxa = vfma(c, qx, jxa);
+            jya = vfma(c, qy, jya);
         }
         Jx[a] = jxa;
         Jy[a] = jya;
     }
-    scalar_collide<M>(f, s, ux, uy, om, Jx, Jy);
+    scalar_collide<M, K, kWithForce || K == kAnyClosure || (K & kConsume) != 0>(f, s, ux, uy, om, Jx, Jy);
 
     // Eq. evolution3 with Eq. force, weighted by (1 - omega_f / 2):
     //   h*_i = h_i - wf (h_i - h^eq_i) + fw F_i,   fw = 1 - wf / 2,
@@ -458,25 +513,27 @@ __device__ __forceinline__ void collide(const LbParams &p, V (&f)[M][5], V (&h)[
     // opposite signs, so each pair forms them once.
     const float wf = p.omega_f, fw = 1.f - 0.5f * wf;
     {
-        V F0 = splat<V>(0.f);
-        if (p.varphi != 0.f) F0 = vmul(p.varphi, force2_dir(0, ux, uy, Fx, Fy, uF));
-        h[0] = vfma(fw, F0, vfma(-wf, h[0] - fluid_equilibrium(0, prd, ux, uy, usq), h[0]));
+        h[0] = vfma(-wf, h[0] - fluid_equilibrium(0, prd, ux, uy, usq), h[0]);
+        if (second) h[0] = vfma(fw, vmul(p.varphi, force2_dir(0, ux, uy, Fx, Fy, uF)), h[0]);
     }
     const V q = vfma(-0.5f, usq, prd);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const int i = k < 2 ? k + 1 : k + 3, io = i + 2;  // i = 1, 2, 5, 6 and their opposites io = 3, 4, 7, 8
         const float kA = kA9(i);
-        const V cu = cdot(kC9x(i), kC9y(i), ux, uy), cF = cdot(kC9x(i), kC9y(i), Fx, Fy);
-        const V E = heq_even(i, q, ux, uy), O = heq_odd(i, ux, uy), Fo = vmul(kA, cF);
+        const V E = heq_even(i, q, ux, uy), O = heq_odd(i, ux, uy);
+        h[i] = vfma(-wf, h[i] - (E + O), h[i]);
+        h[io] = vfma(-wf, h[io] - (E - O), h[io]);
+        if (!kWithForce) continue;
+        const V cu = cdot(kC9x(i), kC9y(i), ux, uy), cF = cdot(kC9x(i), kC9y(i), Fx, Fy), Fo = vmul(kA, cF);
         V Fi = Fo, Fopp = -Fo;
-        if (p.varphi != 0.f) {
+        if (second) {
             const V f2 = vmul(kA, vfma(vmul(3.f, cu), cF, -uF));  // even in c_i
             Fi = vfma(p.varphi, f2, Fo);
             Fopp = vfma(p.varphi, f2, -Fo);
         }
-        h[i] = vfma(fw, Fi, vfma(-wf, h[i] - (E + O), h[i]));
-        h[io] = vfma(fw, Fopp, vfma(-wf, h[io] - (E - O), h[io]));
+        h[i] = vfma(fw, Fi, h[i]);
+        h[io] = vfma(fw, Fopp, h[io]);
     }
 #pragma unroll
     for (int a = 0; a < M; ++a) o.phi[a] = s.phi[a];
@@ -491,13 +548,13 @@ __device__ __forceinline__ void collide(const LbParams &p, V (&f)[M][5], V (&h)[
 // G_i,a = sum_b (delta_ab - omega_ab / 2) W_i c_i . d_t(phi_b u) / cs^2 with the
 // first-order explicit difference d_t(phi_b u) = u (phi_b - phi_prev_b).
 // phi_prev: phi(t - 1), overwritten with phi(t).
-template <int M>
+template <int M, int K = kAnyClosure>
 __device__ __forceinline__ void collide_case1(const LbParams &p, float (&f)[M][5], float ux, float uy,
                                               float (&phi_prev)[M], float sp1, bool first, NodeOut<M> &o) {
     ScalarState<M> s;
-    scalar_closures<M>(p, f, sp1, first, s);
+    scalar_closures<M, K>(p, f, sp1, first, s);
     float om[M][M];
-    relaxation_matrix<M>(p, s, om);
+    relaxation_matrix<M, K>(p, s, om);
     float Jx[M], Jy[M];
 #pragma unroll
     for (int a = 0; a < M; ++a) {
@@ -507,7 +564,7 @@ __device__ __forceinline__ void collide_case1(const LbParams &p, float (&f)[M][5
         Jx[a] = __fmul_rn(ux, ja);
         Jy[a] = __fmul_rn(uy, ja);
     }
-    scalar_collide<M>(f, s, ux, uy, om, Jx, Jy);
+    scalar_collide<M, K>(f, s, ux, uy, om, Jx, Jy);
 #pragma unroll
     for (int a = 0; a < M; ++a) {
         o.phi[a] = s.phi[a];
@@ -660,7 +717,7 @@ __device__ __forceinline__ PullTable<decltype(std::declval<MakePos>()(0, 0))> pu
 // Pre-collision populations of node (x, y) in deviation variables: the loads of
 // the pull table through ld(plane, pos), then the pressure-reference shifts and,
 // in deviations, the anti-bounce-back value -f'*_opp(i)(x) + 2 W_i (phi_w - phi_ref).
-template <int M, bool kInterior, class MakePos, class Load>
+template <int M, bool kInterior, int K = kAnyClosure, class MakePos, class Load>
 __device__ __forceinline__ void pull_node(const LbParams &p, int x, int y, const MakePos &mk, const Load &ld,
                                           float (&f)[M][5], float (&h)[9]) {
     const auto t = pull_table<kInterior>(p, x, y, mk);
@@ -670,8 +727,10 @@ __device__ __forceinline__ void pull_node(const LbParams &p, int x, int y, const
     for (int a = 0; a < M; ++a)
 #pragma unroll
         for (int i = 0; i < 5; ++i) f[a][i] = ld(9 + 5 * a + t.splane[i], t.spos[i]);
+    if (K < 0 || (K & kShift)) {
 #pragma unroll
-    for (int i = 0; i < 9; ++i) h[i] += t.hshift[i];
+        for (int i = 0; i < 9; ++i) h[i] += t.hshift[i];
+    }
     if (!kInterior) {
 #pragma unroll
         for (int i = 1; i < 5; ++i) {
@@ -738,7 +797,7 @@ __device__ __forceinline__ void step_node(const LbParams &p, int x, int y, const
 
 // step_node with the planes given one pointer each (Planes): the form of the
 // single-lattice step kernels.  Same node update, same bits.
-template <int M, typename T, bool kInterior = false>
+template <int M, typename T, bool kInterior = false, int K = kAnyClosure>
 __device__ __forceinline__ void step_node_planes(const LbParams &p, int x, int y, const Planes<T> &pl,
                                                  const float *sp_in, float *sp_out, float *__restrict__ moments) {
     const int pitch = p.pitch;
@@ -747,13 +806,13 @@ __device__ __forceinline__ void step_node_planes(const LbParams &p, int x, int y
         return Store<T>::load(pl.in[plane] + CDF_CHK(p, off, p.plane, 1));
     };
     const int o0 = CDF_CHK(p, y * pitch + x, p.plane, 2);
-    const bool consume = (M >= 2 && p.skind == 2);
+    const bool consume = M >= 2 && closure_has<K>(kConsume, p.skind == 2);
     const float sp1 = consume ? sp_in[o0] : 0.f;
     float h[9], f[M][5];
-    pull_node<M, kInterior>(p, x, y, mk, ld, f, h);
+    pull_node<M, kInterior, K>(p, x, y, mk, ld, f, h);
 
     NodeOut<M> o;
-    collide<M>(p, f, h, pref_at(p, x, y), sp1, false, o);
+    collide<M, K>(p, f, h, node_pref<K>(p, x, y), sp1, false, o);
 #pragma unroll
     for (int i = 0; i < 9; ++i) Store<T>::store(pl.out[i] + o0, h[i]);
 #pragma unroll

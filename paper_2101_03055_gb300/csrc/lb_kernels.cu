@@ -66,8 +66,69 @@ Planes<T> planes_of(const LbParams &p, const T *in, T *out) {
     return pl;
 }
 
+// ---- closure kinds (lb_device.cuh) ----------------------------------------------
+// The kinds with kernels of their own, for two scalars (every experiment of the paper): the
+// chemotaxis plume, constant D under a body force (the cavity), constant D alone
+// (periodic boxes, Case 1).
+constexpr int kKindPlume = kChemo | kConsume | kForce | kShift | kUpper;
+constexpr int kKindForced = kForce | kShift;
+constexpr int kKindPlain = 0;
+
+// The kind whose kernels may run lattice p: every term that p uses is in it.
+int closure_kind(const LbParams &p) {
+    if (p.m != 2 || p.varphi != 0.f) return kAnyClosure;
+    if (p.chemotaxis && p.skind == 2 && p.omega[2] == 0.f) return kKindPlume;
+    if (p.chemotaxis || p.skind != 0) return kAnyClosure;
+    if (p.case1) return kKindPlain;
+    return (p.g[0] != 0.f || p.g[1] != 0.f || p.gref[0] != 0.f || p.gref[1] != 0.f) ? kKindForced : kKindPlain;
+}
+
+// Case 1 has no force: its kernels exist for the plain kind and for any closure.
+constexpr int case1_kind(int kind) { return kind == kKindPlain ? kKindPlain : kAnyClosure; }
+
+// 16-bit storage keeps no reference gradient.
+constexpr int mr_kind(int kind) { return kind < 0 ? kind : (kind & ~kShift); }
+
+template <int N>
+using Const = std::integral_constant<int, N>;
+
+// f(Const<m>, Const<kind>) for the lattice p.
+template <class F>
+cudaError_t for_model(const LbParams &p, const F &f) {
+    switch (p.m) {
+        case 1: return f(Const<1>{}, Const<kAnyClosure>{});
+        case 2:
+            switch (closure_kind(p)) {
+                case kKindPlume: return f(Const<2>{}, Const<kKindPlume>{});
+                case kKindForced: return f(Const<2>{}, Const<kKindForced>{});
+                case kKindPlain: return f(Const<2>{}, Const<kKindPlain>{});
+                default: return f(Const<2>{}, Const<kAnyClosure>{});
+            }
+        case 3: return f(Const<3>{}, Const<kAnyClosure>{});
+        case 4: return f(Const<4>{}, Const<kAnyClosure>{});
+    }
+    return cudaErrorInvalidValue;
+}
+
+// The opt-in to more than 48 KB of dynamic shared memory, once per device and kernel (one
+// object of this type per kernel).
+struct SmemOptIn {
+    std::atomic<bool> done[64];
+    template <typename... KArgs>
+    cudaError_t operator()(void (*kern)(KArgs...)) {
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+        if (done[dev].load()) return cudaSuccess;
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kStep2MaxSmem);
+        if (e == cudaSuccess) done[dev].store(true);
+        return e;
+    }
+};
+
 // ---- the fused step ------------------------------------------------------------
-template <int M, typename T>
+template <int M, typename T, int K>
 __global__ void __launch_bounds__(256) step_kernel(const LbParams p, const Planes<T> pl, const float *sp_in,
                                                    float *sp_out, float *__restrict__ moments) {
     pdl_wait_and_release();
@@ -77,13 +138,13 @@ __global__ void __launch_bounds__(256) step_kernel(const LbParams p, const Plane
     // all lie inside the boundary ring runs the pull without boundary selects.
     // (halo rows of a slab, y = 0 or ny - 1, are never inner nodes)
     if (__all_sync(0xffffffffu, inner_node(p, x, y)))
-        step_node_planes<M, T, true>(p, x, y, pl, sp_in, sp_out, moments);
+        step_node_planes<M, T, true, K>(p, x, y, pl, sp_in, sp_out, moments);
     else if (x < p.nx && y >= p.row_lo && y < p.row_hi)
-        step_node_planes<M, T>(p, x, y, pl, sp_in, sp_out, moments);
+        step_node_planes<M, T, false, K>(p, x, y, pl, sp_in, sp_out, moments);
 }
 
 // Flat launch: one thread per node over nx * ny (no idle threads in ragged rows).
-template <int M, typename T>
+template <int M, typename T, int K>
 __global__ void __launch_bounds__(256) step_kernel_flat(const LbParams p, const Planes<T> pl, const float *sp_in,
                                                         float *sp_out, float *__restrict__ moments) {
     pdl_wait_and_release();
@@ -91,9 +152,9 @@ __global__ void __launch_bounds__(256) step_kernel_flat(const LbParams p, const 
     const bool valid = idx < p.nx * p.ny;
     const int y = idx / p.nx, x = idx - y * p.nx;
     if (__all_sync(0xffffffffu, valid && inner_node(p, x, y)))
-        step_node_planes<M, T, true>(p, x, y, pl, sp_in, sp_out, moments);
+        step_node_planes<M, T, true, K>(p, x, y, pl, sp_in, sp_out, moments);
     else if (valid && y >= p.row_lo && y < p.row_hi)
-        step_node_planes<M, T>(p, x, y, pl, sp_in, sp_out, moments);
+        step_node_planes<M, T, false, K>(p, x, y, pl, sp_in, sp_out, moments);
 }
 
 template <int M>
@@ -202,7 +263,7 @@ __global__ void __launch_bounds__(256) step_kernel_flat_x2(const LbParams p, con
 // shape known, the shared-memory plane stride is a constant, every
 // shared-memory access is a register plus an immediate offset and the row
 // loops unroll; the node update is the same, so are the bits.
-template <int M, int FW = 0, int FY = 0, int FT = 0>
+template <int M, int K, int FW = 0, int FY = 0, int FT = 0>
 __global__ void __launch_bounds__(FW ? FW * FY : step2_max_threads(M), FW ? step2_max_threads(M) / (FW * FY) : 1)
     step2_kernel(const LbParams p, int TH, const Planes<float> pl, const float *sp_in, float *sp_out,
                  float *__restrict__ moments) {
@@ -214,7 +275,7 @@ __global__ void __launch_bounds__(FW ? FW * FY : step2_max_threads(M), FW ? step
     const int X0 = blockIdx.x * TW, Y0 = blockIdx.y * THv;
     const long long P = p.plane;
     const int pitch = p.pitch, nx = p.nx, ny = p.ny;
-    const bool consume = M >= 2 && p.skind == 2;
+    const bool consume = M >= 2 && closure_has<K>(kConsume, p.skind == 2);
     const int lx = threadIdx.x;
 
     // Column lx of R1: unwrapped x = X0 - 1 + lx.  It is needed when some tile
@@ -237,14 +298,14 @@ __global__ void __launch_bounds__(FW ? FW * FY : step2_max_threads(M), FW ? step
             float h[9], f[M][5];
             if (!__any_sync(0xffffffffu, general)) {
                 if (!ok) continue;
-                pull_node<M, true>(p, gx, gy, mk, ld, f, h);
+                pull_node<M, true, K>(p, gx, gy, mk, ld, f, h);
             } else {
                 if (!ok) continue;
-                pull_node<M, false>(p, gx, gy, mk, ld, f, h);
+                pull_node<M, false, K>(p, gx, gy, mk, ld, f, h);
             }
             const int o0 = CDF_CHK(p, gy * pitch + gx, P, 2), l0 = CDF_CHK(p, ly * W1 + lx, SP, 3);
             NodeOut<M> o;
-            collide<M>(p, f, h, pref_at(p, gx, gy), consume ? sp_in[o0] : 0.f, false, o);
+            collide<M, K>(p, f, h, node_pref<K>(p, gx, gy), consume ? sp_in[o0] : 0.f, false, o);
 #pragma unroll
             for (int i = 0; i < 9; ++i) sm[i * SP + l0] = h[i];
 #pragma unroll
@@ -275,14 +336,14 @@ __global__ void __launch_bounds__(FW ? FW * FY : step2_max_threads(M), FW ? step
         float h[9], f[M][5];
         if (!__any_sync(0xffffffffu, general)) {
             if (!ok) continue;
-            pull_node<M, true>(p, x, y, mk_in, lds, f, h);
+            pull_node<M, true, K>(p, x, y, mk_in, lds, f, h);
         } else {
             if (!ok) continue;
-            pull_node<M, false>(p, x, y, mk_gen, lds, f, h);
+            pull_node<M, false, K>(p, x, y, mk_gen, lds, f, h);
         }
         const int o0 = CDF_CHK(p, y * pitch + x, P, 2);
         NodeOut<M> o;
-        collide<M>(p, f, h, pref_at(p, x, y), consume ? sm[NP * SP + CDF_CHK(p, ly * W1 + lx, SP, 4)] : 0.f, false, o);
+        collide<M, K>(p, f, h, node_pref<K>(p, x, y), consume ? sm[NP * SP + CDF_CHK(p, ly * W1 + lx, SP, 4)] : 0.f, false, o);
 #pragma unroll
         for (int i = 0; i < 9; ++i) pl.out[i][o0] = h[i];
 #pragma unroll
@@ -423,7 +484,7 @@ __global__ void __launch_bounds__(256, 2)
 // velocity (p.vel) and phi(t - 1) (p.php_in), collide with the Case-1
 // auxiliary source, store the scalars and phi(t) (p.php_out, the other phi
 // set).  Algorithmic bytes: 2 x 5m x 4 + 8 + 2 x 4m.
-template <int M>
+template <int M, int K>
 __global__ void __launch_bounds__(256) step_kernel_case1(const LbParams p, const float *__restrict__ in,
                                                          float *__restrict__ out, const float *sp_in, float *sp_out,
                                                          float *__restrict__ moments) {
@@ -443,10 +504,10 @@ __global__ void __launch_bounds__(256) step_kernel_case1(const LbParams p, const
     float php[M];
 #pragma unroll
     for (int a = 0; a < M; ++a) php[a] = p.php_in[a * P + o0];
-    const bool consume = (M >= 2 && p.skind == 2);
+    const bool consume = M >= 2 && closure_has<K>(kConsume, p.skind == 2);
     const float sp1 = consume ? sp_in[o0] : 0.f;
     NodeOut<M> o;
-    collide_case1<M>(p, f, ux, uy, php, sp1, false, o);
+    collide_case1<M, K>(p, f, ux, uy, php, sp1, false, o);
 #pragma unroll
     for (int a = 0; a < M; ++a)
 #pragma unroll
@@ -463,7 +524,7 @@ __global__ void __launch_bounds__(256) step_kernel_case1(const LbParams p, const
 // velocity is read from global memory at every node; phi is read from
 // p.php_in and written to p.php_out (different sets: the halo of one CTA is the
 // tile of another).  Bitwise equal to two launches of step_kernel_case1.
-template <int M>
+template <int M, int K>
 __global__ void __launch_bounds__(step2_max_threads(M)) step2_kernel_case1(const LbParams p, int TH,
                                                                            const Planes<float> pl,
                                                                            const float *sp_in, float *sp_out,
@@ -475,7 +536,7 @@ __global__ void __launch_bounds__(step2_max_threads(M)) step2_kernel_case1(const
     const int X0 = blockIdx.x * TW, Y0 = blockIdx.y * TH;
     const long long P = p.plane;
     const int pitch = p.pitch, nx = p.nx, ny = p.ny;
-    const bool consume = M >= 2 && p.skind == 2;
+    const bool consume = M >= 2 && closure_has<K>(kConsume, p.skind == 2);
     const int lx = threadIdx.x;
     const int xu = X0 - 1 + lx;
     const bool colv = xu <= min(X0 + TW, nx) && (p.periodic_x || (xu >= 0 && xu < nx));
@@ -498,7 +559,7 @@ __global__ void __launch_bounds__(step2_max_threads(M)) step2_kernel_case1(const
 #pragma unroll
             for (int a = 0; a < M; ++a) php[a] = p.php_in[a * P + o0];
             NodeOut<M> o;
-            collide_case1<M>(p, f, ux, uy, php, consume ? sp_in[o0] : 0.f, false, o);
+            collide_case1<M, K>(p, f, ux, uy, php, consume ? sp_in[o0] : 0.f, false, o);
 #pragma unroll
             for (int a = 0; a < M; ++a)
 #pragma unroll
@@ -529,7 +590,7 @@ __global__ void __launch_bounds__(step2_max_threads(M)) step2_kernel_case1(const
 #pragma unroll
         for (int a = 0; a < M; ++a) php[a] = sm[(NS + a) * SP + l0];
         NodeOut<M> o;
-        collide_case1<M>(p, f, ux, uy, php, consume ? sm[(NS + M) * SP + l0] : 0.f, false, o);
+        collide_case1<M, K>(p, f, ux, uy, php, consume ? sm[(NS + M) * SP + l0] : 0.f, false, o);
 #pragma unroll
         for (int a = 0; a < M; ++a)
 #pragma unroll
@@ -812,16 +873,16 @@ __device__ __forceinline__ void store_node_mr(int o0, const Planes<T> &pl, const
 }
 
 // One node of the 16-bit step.
-template <int M, typename T, bool kInterior>
+template <int M, typename T, bool kInterior, int K>
 __device__ __forceinline__ void step_node_mr(const LbParams &p, int x, int y, const Planes<T> &pl,
                                              const MomentPlanes &mp, const float *sp_in, float *sp_out) {
     const int o0 = CDF_CHK(p, y * p.pitch + x, p.plane, 2);
     float f[M][5], h[9];
     pull_node_mr<M, T, kInterior>(p, x, y, pl, mp, f, h);
-    const bool consume = (M >= 2 && p.skind == 2);
+    const bool consume = M >= 2 && closure_has<K>(kConsume, p.skind == 2);
     const float sp1 = consume ? sp_in[o0] : 0.f;
     NodeOut<M> o;
-    collide<M>(p, f, h, 0.f, sp1, false, o);
+    collide<M, K>(p, f, h, 0.f, sp1, false, o);
     store_node_mr<M, T>(o0, pl, mp, f, h, o);
     if (consume) sp_out[o0] = o.s1;
 }
@@ -834,7 +895,7 @@ __device__ __forceinline__ void step_node_mr(const LbParams &p, int x, int y, co
 // are rounded to 16 bits once, so the results differ from two one-step
 // launches by that saved rounding (both are held to the FP64 oracle).
 // FW, FY, FT != 0: a copy for one CTA shape and tile height, as for step2_kernel.
-template <int M, typename T, int FW = 0, int FY = 0, int FT = 0>
+template <int M, typename T, int K, int FW = 0, int FY = 0, int FT = 0>
 __global__ void __launch_bounds__(step2_mr_max_threads(M), (M <= 2 ? 3 : 1)) step2_kernel_mr(
     const LbParams p, int TH, const Planes<T> pl, const MomentPlanes mp, const float *sp_in, float *sp_out) {
     constexpr int NP = 9 + 5 * M;
@@ -844,7 +905,7 @@ __global__ void __launch_bounds__(step2_mr_max_threads(M), (M <= 2 ? 3 : 1)) ste
     const int H1 = THv + 2, SP = W1 * H1, TW = W1 - 2;
     const int X0 = blockIdx.x * TW, Y0 = blockIdx.y * THv;
     const int pitch = p.pitch, nx = p.nx, ny = p.ny;
-    const bool consume = M >= 2 && p.skind == 2;
+    const bool consume = M >= 2 && closure_has<K>(kConsume, p.skind == 2);
     const int lx = threadIdx.x;
     const int xu = X0 - 1 + lx;
     const bool colv = xu <= min(X0 + TW, nx) && (p.periodic_x || (xu >= 0 && xu < nx));
@@ -867,7 +928,7 @@ __global__ void __launch_bounds__(step2_mr_max_threads(M), (M <= 2 ? 3 : 1)) ste
         }
         const int o0 = CDF_CHK(p, gy * pitch + gx, p.plane, 2), l0 = CDF_CHK(p, ly * W1 + lx, SP, 3);
         NodeOut<M> o;
-        collide<M>(p, f, h, 0.f, consume ? sp_in[o0] : 0.f, false, o);
+        collide<M, K>(p, f, h, 0.f, consume ? sp_in[o0] : 0.f, false, o);
 #pragma unroll
         for (int i = 0; i < 9; ++i) sm[i * SP + l0] = h[i];
 #pragma unroll
@@ -895,20 +956,20 @@ __global__ void __launch_bounds__(step2_mr_max_threads(M), (M <= 2 ? 3 : 1)) ste
         float h[9], f[M][5];
         if (!__any_sync(0xffffffffu, general)) {
             if (!ok) continue;
-            pull_node<M, true>(p, x, y, mk_in, lds, f, h);
+            pull_node<M, true, K>(p, x, y, mk_in, lds, f, h);
         } else {
             if (!ok) continue;
-            pull_node<M, false>(p, x, y, mk_gen, lds, f, h);
+            pull_node<M, false, K>(p, x, y, mk_gen, lds, f, h);
         }
         const int o0 = CDF_CHK(p, y * pitch + x, p.plane, 2);
         NodeOut<M> o;
-        collide<M>(p, f, h, 0.f, consume ? sm[NP * SP + CDF_CHK(p, ly * W1 + lx, SP, 4)] : 0.f, false, o);
+        collide<M, K>(p, f, h, 0.f, consume ? sm[NP * SP + CDF_CHK(p, ly * W1 + lx, SP, 4)] : 0.f, false, o);
         store_node_mr<M, T>(o0, pl, mp, f, h, o);
         if (consume) sp_out[o0] = o.s1;
     }
 }
 
-template <int M, typename T>
+template <int M, typename T, int K>
 __global__ void __launch_bounds__(256, (M <= 2 ? 3 : 1)) step_kernel_mr(const LbParams p, const Planes<T> pl,
                                                                        const MomentPlanes mp, const float *sp_in,
                                                                        float *sp_out) {
@@ -917,9 +978,9 @@ __global__ void __launch_bounds__(256, (M <= 2 ? 3 : 1)) step_kernel_mr(const Lb
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     // warp-uniform interior path, as in step_kernel
     if (__all_sync(0xffffffffu, inner_node(p, x, y)))
-        step_node_mr<M, T, true>(p, x, y, pl, mp, sp_in, sp_out);
+        step_node_mr<M, T, true, K>(p, x, y, pl, mp, sp_in, sp_out);
     else if (x < p.nx && y < p.ny)
-        step_node_mr<M, T, false>(p, x, y, pl, mp, sp_in, sp_out);
+        step_node_mr<M, T, false, K>(p, x, y, pl, mp, sp_in, sp_out);
 }
 
 template <int M, typename T>
@@ -995,14 +1056,10 @@ cudaError_t step_mr_dispatch(const LbParams &p, const void *in, const float *min
     T *o = static_cast<T *>(out);
     const Planes<T> pl = planes_of(p, i, o);
     const MomentPlanes mp = moments_of(p, min, mout);
-    cudaError_t e = cudaSuccess;
-    switch (p.m) {
-        case 1: e = launch_pdl(step_kernel_mr<1, T>, grid, block, s, p, pl, mp, sp_in, sp_out); break;
-        case 2: e = launch_pdl(step_kernel_mr<2, T>, grid, block, s, p, pl, mp, sp_in, sp_out); break;
-        case 3: e = launch_pdl(step_kernel_mr<3, T>, grid, block, s, p, pl, mp, sp_in, sp_out); break;
-        case 4: e = launch_pdl(step_kernel_mr<4, T>, grid, block, s, p, pl, mp, sp_in, sp_out); break;
-        default: return cudaErrorInvalidValue;
-    }
+    const cudaError_t e = for_model(p, [&](auto m, auto kind) {
+        constexpr int M = decltype(m)::value, K = mr_kind(decltype(kind)::value);
+        return launch_pdl(step_kernel_mr<M, T, K>, grid, block, s, p, pl, mp, sp_in, sp_out);
+    });
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -1044,14 +1101,10 @@ cudaError_t step_dispatch(const LbParams &p, const void *in, void *out, const fl
         if constexpr (std::is_same<T, float>::value) {
             const dim3 b2(block.x, block.y ? block.y : 1);
             dim3 grid((p.nx + b2.x - 1) / b2.x, (p.ny + b2.y - 1) / b2.y);
-            cudaError_t e = cudaSuccess;
-            switch (p.m) {
-                case 1: e = launch_pdl(step_kernel_case1<1>, grid, b2, s, p, i, o, sp_in, sp_out, mom); break;
-                case 2: e = launch_pdl(step_kernel_case1<2>, grid, b2, s, p, i, o, sp_in, sp_out, mom); break;
-                case 3: e = launch_pdl(step_kernel_case1<3>, grid, b2, s, p, i, o, sp_in, sp_out, mom); break;
-                case 4: e = launch_pdl(step_kernel_case1<4>, grid, b2, s, p, i, o, sp_in, sp_out, mom); break;
-                default: return cudaErrorInvalidValue;
-            }
+            const cudaError_t e = for_model(p, [&](auto m, auto kind) {
+                constexpr int M = decltype(m)::value, K = case1_kind(decltype(kind)::value);
+                return launch_pdl(step_kernel_case1<M, K>, grid, b2, s, p, i, o, sp_in, sp_out, mom);
+            });
             return e != cudaSuccess ? e : cudaGetLastError();
         }
         return cudaErrorInvalidValue;
@@ -1075,25 +1128,17 @@ cudaError_t step_dispatch(const LbParams &p, const void *in, void *out, const fl
     if (block.y == 0) {  // flat launch
         const long long n = (long long)p.nx * p.ny;
         dim3 fb(block.x), grid((unsigned)((n + block.x - 1) / block.x));
-        cudaError_t e = cudaSuccess;
-        switch (p.m) {
-            case 1: e = launch_pdl(step_kernel_flat<1, T>, grid, fb, s, p, pl, sp_in, sp_out, mom); break;
-            case 2: e = launch_pdl(step_kernel_flat<2, T>, grid, fb, s, p, pl, sp_in, sp_out, mom); break;
-            case 3: e = launch_pdl(step_kernel_flat<3, T>, grid, fb, s, p, pl, sp_in, sp_out, mom); break;
-            case 4: e = launch_pdl(step_kernel_flat<4, T>, grid, fb, s, p, pl, sp_in, sp_out, mom); break;
-            default: return cudaErrorInvalidValue;
-        }
+        const cudaError_t e = for_model(p, [&](auto m, auto kind) {
+            constexpr int M = decltype(m)::value, K = decltype(kind)::value;
+            return launch_pdl(step_kernel_flat<M, T, K>, grid, fb, s, p, pl, sp_in, sp_out, mom);
+        });
         return e != cudaSuccess ? e : cudaGetLastError();
     }
     dim3 grid((p.nx + block.x - 1) / block.x, (p.ny + block.y - 1) / block.y);
-    cudaError_t e = cudaSuccess;
-    switch (p.m) {
-        case 1: e = launch_pdl(step_kernel<1, T>, grid, block, s, p, pl, sp_in, sp_out, mom); break;
-        case 2: e = launch_pdl(step_kernel<2, T>, grid, block, s, p, pl, sp_in, sp_out, mom); break;
-        case 3: e = launch_pdl(step_kernel<3, T>, grid, block, s, p, pl, sp_in, sp_out, mom); break;
-        case 4: e = launch_pdl(step_kernel<4, T>, grid, block, s, p, pl, sp_in, sp_out, mom); break;
-        default: return cudaErrorInvalidValue;
-    }
+    const cudaError_t e = for_model(p, [&](auto m, auto kind) {
+        constexpr int M = decltype(m)::value, K = decltype(kind)::value;
+        return launch_pdl(step_kernel<M, T, K>, grid, block, s, p, pl, sp_in, sp_out, mom);
+    });
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -1162,56 +1207,30 @@ cudaError_t launch_step2(const LbParams &p, const float *in, float *out, const f
     const bool x2 = block.z == 2;
     if (x2 && (p.case1 || block.x != 32 || block.y != 8 || (th != 14 && th != 30))) return cudaErrorInvalidValue;
     const dim3 threads(block.x, block.y, 1);
-    // the opt-in to more than 48 KB of dynamic shared memory, once per device and m
-    static std::atomic<bool> attr_set[64][kMaxM + 1];
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     // the shape that the autotuners pick for large lattices and for the batched
     // sweep has its own copy of the kernel (constant shared-memory strides)
-    const bool fixed = !p.case1 && block.x == 32 && block.y == 8 && th == 14;
-    switch (p.m) {
-#define CDF_STEP2_CASE(MM)                                                                               \
-    case MM:                                                                                             \
-        if (!attr_set[dev][MM].load()) {                                                                 \
-            e = cudaFuncSetAttribute(step2_kernel<MM>, cudaFuncAttributeMaxDynamicSharedMemorySize,      \
-                                     kStep2MaxSmem);                                                     \
-            if (e == cudaSuccess)                                                                        \
-                e = cudaFuncSetAttribute(step2_kernel<MM, 32, 8, 14>,                                    \
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kStep2MaxSmem);    \
-            if (e == cudaSuccess)                                                                        \
-                e = cudaFuncSetAttribute(step2_kernel_case1<MM>,                                         \
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kStep2MaxSmem);    \
-            if (e == cudaSuccess && MM <= 2)                                                             \
-                e = cudaFuncSetAttribute(step2_kernel_x2<(MM <= 2 ? MM : 2), 14>,                        \
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kStep2MaxSmem);    \
-            if (e == cudaSuccess && MM <= 2)                                                             \
-                e = cudaFuncSetAttribute(step2_kernel_x2<(MM <= 2 ? MM : 2), 30>,                        \
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kStep2MaxSmem);    \
-            if (e != cudaSuccess) return e;                                                              \
-            attr_set[dev][MM].store(true);                                                               \
-        }                                                                                                \
-        if (p.case1)                                                                                     \
-            e = launch_pdl_smem(step2_kernel_case1<MM>, grid, threads, smem, s, p, th, pl, sp_in, sp_out, moments); \
-        else if (x2)                                                                                     \
-            e = MM > 2 ? cudaErrorInvalidValue                                                           \
-                       : launch_pdl_smem(th == 14 ? step2_kernel_x2<(MM <= 2 ? MM : 2), 14>              \
-                                                  : step2_kernel_x2<(MM <= 2 ? MM : 2), 30>,             \
-                                         grid, threads, smem, s, p, th, pl, sp_in, sp_out, moments);     \
-        else if (fixed)                                                                                  \
-            e = launch_pdl_smem(step2_kernel<MM, 32, 8, 14>, grid, threads, smem, s, p, th, pl, sp_in, sp_out,   \
-                                moments);                                                                \
-        else                                                                                             \
-            e = launch_pdl_smem(step2_kernel<MM>, grid, threads, smem, s, p, th, pl, sp_in, sp_out, moments); \
-        break;
-        CDF_STEP2_CASE(1)
-        CDF_STEP2_CASE(2)
-        CDF_STEP2_CASE(3)
-        CDF_STEP2_CASE(4)
-#undef CDF_STEP2_CASE
-        default: return cudaErrorInvalidValue;
-    }
+    const bool fixed = block.x == 32 && block.y == 8 && th == 14;
+    const cudaError_t e = for_model(p, [&](auto m, auto kind) {
+        constexpr int M = decltype(m)::value, K = decltype(kind)::value;
+        const auto run = [&](auto *kern, SmemOptIn &opt_in) {
+            const cudaError_t e1 = opt_in(kern);
+            if (e1 != cudaSuccess) return e1;
+            return launch_pdl_smem(kern, grid, threads, smem, s, p, th, pl, sp_in, sp_out, moments);
+        };
+        if (p.case1) {
+            static SmemOptIn opt_in;
+            return run(step2_kernel_case1<M, case1_kind(K)>, opt_in);
+        }
+        if (x2) {
+            if constexpr (M <= 2) {
+                static SmemOptIn opt_in14, opt_in30;
+                return th == 14 ? run(step2_kernel_x2<M, 14>, opt_in14) : run(step2_kernel_x2<M, 30>, opt_in30);
+            }
+            return cudaErrorInvalidValue;
+        }
+        static SmemOptIn opt_in_fixed, opt_in;
+        return fixed ? run(step2_kernel<M, K, 32, 8, 14>, opt_in_fixed) : run(step2_kernel<M, K>, opt_in);
+    });
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -1224,35 +1243,17 @@ cudaError_t step2_mr_dispatch(const LbParams &p, const void *in, const float *mi
     T *o = static_cast<T *>(out);
     const Planes<T> pl = planes_of(p, i, o);
     const MomentPlanes mp = moments_of(p, min, mout);
-    static std::atomic<bool> attr_set[64][kMaxM + 1];
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     const bool fixed = block.x == 32 && block.y == 8 && th == 14;  // the shape with its own copy
-    switch (p.m) {
-#define CDF_STEP2MR_CASE(MM)                                                                             \
-    case MM:                                                                                             \
-        if (!attr_set[dev][MM].load()) {                                                                 \
-            e = cudaFuncSetAttribute(step2_kernel_mr<MM, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                     kStep2MaxSmem);                                                     \
-            if (e == cudaSuccess)                                                                        \
-                e = cudaFuncSetAttribute(step2_kernel_mr<MM, T, 32, 8, 14>,                              \
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kStep2MaxSmem);    \
-            if (e != cudaSuccess) return e;                                                              \
-            attr_set[dev][MM].store(true);                                                               \
-        }                                                                                                \
-        e = fixed ? launch_pdl_smem(step2_kernel_mr<MM, T, 32, 8, 14>, grid, block, smem, s, p, th, pl, mp, sp_in, \
-                                    sp_out)                                                              \
-                  : launch_pdl_smem(step2_kernel_mr<MM, T>, grid, block, smem, s, p, th, pl, mp, sp_in, sp_out); \
-        break;
-        CDF_STEP2MR_CASE(1)
-        CDF_STEP2MR_CASE(2)
-        CDF_STEP2MR_CASE(3)
-        CDF_STEP2MR_CASE(4)
-#undef CDF_STEP2MR_CASE
-        default: return cudaErrorInvalidValue;
-    }
+    const cudaError_t e = for_model(p, [&](auto m, auto kind) {
+        constexpr int M = decltype(m)::value, K = mr_kind(decltype(kind)::value);
+        const auto run = [&](auto *kern, SmemOptIn &opt_in) {
+            const cudaError_t e1 = opt_in(kern);
+            if (e1 != cudaSuccess) return e1;
+            return launch_pdl_smem(kern, grid, block, smem, s, p, th, pl, mp, sp_in, sp_out);
+        };
+        static SmemOptIn opt_in_fixed, opt_in;
+        return fixed ? run(step2_kernel_mr<M, T, K, 32, 8, 14>, opt_in_fixed) : run(step2_kernel_mr<M, T, K>, opt_in);
+    });
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
