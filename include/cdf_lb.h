@@ -368,7 +368,9 @@ typedef struct {
     double barrier_timeout_s;    /* bound of every grid-barrier wait; 0 = 1 s */
     int test_unreachable_barrier;/* test hook: the barrier expects one block more than runs,
                                     so every wait runs out and cdf_batch_step returns CDF_ETIMEOUT */
-    int mode;                    /* with tile_x > 0: 0 = persistent kernel (tile = tile shape),
+    int mode;                    /* with tile_x > 0: 0 = whole-batch kernels: two steps of all instances
+                                    per launch (every periodic axis at least 6 nodes long), else (and
+                                    with the test hook) the persistent kernel with this tile shape,
                                     1 = graph of per-instance kernel chains (tile = CTA shape),
                                     2 = the same chains of two-step launches (step2_kernel of
                                     cdf_options.temporal; tile = its CTA shape, tile_x 32 or 64);
@@ -385,7 +387,7 @@ typedef struct {
     int tile_x, tile_y, grid_blocks, steps_per_launch;
     double bytes_per_lup;
     long long t;
-    int mode;                    /* 0 persistent kernel, 1 graph of per-instance chains,
+    int mode;                    /* 0 whole-batch kernels, 1 graph of per-instance chains,
                                     2 chains of two-step launches */
     int chain_block_x, chain_block_y;
     int chain_tile_y;            /* mode 2: output tile height of the two-step kernel */

@@ -1,8 +1,10 @@
-// Batched solver: many lattices of uneven size advanced by one persistent
-// kernel.  Work is scheduled as (instance, tile) units; a bounded grid barrier
+// Batched solver: many lattices of uneven size.  Where every lattice fits the
+// two-step tiling, one launch advances all of them by two steps
+// (step2_batch_kernel: a CTA per tile of any instance).  Otherwise a persistent
+// kernel: work is scheduled as (instance, tile) units; a bounded grid barrier
 // separates time steps inside a launch, so one launch advances every instance
-// by `steps_per_launch` steps.  Each node runs the same step_node() as the
-// single-lattice kernel, with its instance's parameters staged in shared memory.
+// by `steps_per_launch` steps.  Or chains of the single-lattice kernels per
+// instance over a pool of streams.  Each node runs the same update in all of them.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -19,15 +21,6 @@
 
 namespace cdflb {
 namespace {
-
-struct BatchInst {
-    LbParams p;
-    long long pop_off;  // element offset of the instance's planes in a population buffer
-    long long sp_off;   // offset in the S(t-1) buffer
-    long long mom_off;  // offset in the moment buffer
-    int tile_base;      // first tile of the instance
-    int tiles_x;
-};
 
 // Grid-wide barrier for a co-resident (cooperative) grid.  bar[0] counts
 // arrivals, bar[1] is the generation.  Every wait is bounded: after timeout_ns
@@ -73,10 +66,11 @@ __device__ bool grid_barrier(unsigned *bar, unsigned expected, unsigned long lon
     return ok != 0;
 }
 
+// (sp_in and sp_out: the same plane set for several steps, S(t - 1) is then updated in place)
 template <int M>
 __global__ void __launch_bounds__(256, 4) batch_kernel(const BatchInst *__restrict__ inst, const int *__restrict__ tile_inst,
-                                                    int total_tiles, float *buf0, float *buf1, float *sprev,
-                                                    float *moments, int nsteps, int parity0, int moments_last,
+                                                    int total_tiles, float *buf0, float *buf1,
+                                                    const float *sp_in, float *sp_out, float *moments, int nsteps, int parity0, int moments_last,
                                                     unsigned *bar, unsigned expected, unsigned long long timeout_ns,
                                                     int *err) {
     __shared__ LbParams sp;
@@ -114,8 +108,8 @@ __global__ void __launch_bounds__(256, 4) batch_kernel(const BatchInst *__restri
             const int ty = lt / s_tile[1], tx = lt - ty * s_tile[1];
             const int x = tx * blockDim.x + threadIdx.x, y = ty * blockDim.y + threadIdx.y;
             if (x < sp.nx && y < sp.ny)
-                dev::step_node<M, float, true>(sp, x, y, in + s_off[0], out + s_off[0], sprev + s_off[1],
-                                               sprev + s_off[1], mom ? mom + s_off[2] : nullptr);
+                dev::step_node<M, float, true>(sp, x, y, in + s_off[0], out + s_off[0], sp_in + s_off[1],
+                                               sp_out + s_off[1], mom ? mom + s_off[2] : nullptr);
         }
         if (s + 1 < nsteps && !grid_barrier(bar, expected, timeout_ns, err, s)) return;
     }
@@ -150,7 +144,7 @@ struct cdf_batch {
     int device = 0;
     int count = 0, m = 0;
     std::vector<LbParams> params;
-    std::vector<long long> pop_off, sp_off, mom_off;
+    std::vector<long long> pop_off, sp_off, mom_off, node_off;
     long long pop_total = 0, sp_total = 0, mom_total = 0, nodes = 0;
     int sprev_planes = 0;
     float *buf[2] = {nullptr, nullptr};
@@ -178,9 +172,14 @@ struct cdf_batch {
     // instance (each launch reads its parameters as kernel operands), fanned out
     // over a pool of streams and captured as one CUDA graph; instances are
     // independent, so the chains need no barrier between them.
-    int mode = 0;  // 0: persistent kernel, 1: graph of per-instance chains, 2: chains of two-step launches
+    int mode = 0;  // 0: whole-batch kernels, 1: graph of per-instance chains, 2: chains of two-step launches
     dim3 chain_block{128, 1, 1};
     int chain_th = 14;  // mode 2: output tile height of step2_kernel (chain_block is its CTA)
+    // mode 0: two steps of all instances per launch instead of the persistent kernel
+    bool fused = false;
+    int kind = 0, pair_tiles = 0;  // closure kind of all instances, tiles of all of them
+    int *d_pair_inst = nullptr;
+    long long max_nodes = 0;
     std::vector<cudaStream_t> pool;
     cudaEvent_t ev_fork = nullptr;
     std::vector<cudaEvent_t> ev_join;
@@ -209,6 +208,7 @@ void brelease(cdf_batch *b) {
     dev_free(b->dense);
     cudaFree(b->d_inst);
     cudaFree(b->d_tile_inst);
+    cudaFree(b->d_pair_inst);
     cudaFree(b->d_bar);
     cudaFree(b->d_err);
     if (b->h_err) cudaFreeHost(b->h_err);
@@ -219,10 +219,32 @@ void brelease(cdf_batch *b) {
     delete b;
 }
 
+// The tile of step2_batch_kernel for one lattice: the least node updates in all (tile and
+// ring, rounded to warps, and about 128 more per CTA for its start) with the region
+// in kBatchRegion nodes and, on a periodic axis, inside the lattice.  false: none fits (a
+// periodic axis of fewer than 6 nodes).
+bool pair_tile(const LbParams &p, int *tw, int *th) {
+    double least = 1e30;
+    for (int w = 4; w <= 128; ++w) {
+        if (p.periodic_x && p.nx < w + 2) break;
+        for (int h = 4; h <= 128 && (w + 2) * (h + 2) <= kBatchRegion; ++h) {
+            if (p.periodic_y && p.ny < h + 2) break;
+            const double tiles = (double)((p.nx + w - 1) / w) * ((p.ny + h - 1) / h);
+            const int warps = ((w + 2) * (h + 2) + 31) / 32 + (w * h + 31) / 32;
+            if (tiles * (32 * warps + 128) < least) {
+                least = tiles * (32 * warps + 128);
+                *tw = w;
+                *th = h;
+            }
+        }
+    }
+    return least < 1e30;
+}
+
 // Tile table and instance descriptors for a tile shape; sets the grid size.
 cdf_status setup_tiles(cdf_batch *b, dim3 tile) {
     std::vector<BatchInst> inst(b->count);
-    std::vector<int> tiles;
+    std::vector<int> tiles, pairs;
     for (int k = 0; k < b->count; ++k) {
         const LbParams &p = b->params[k];
         const int tx = (p.nx + tile.x - 1) / tile.x, ty = (p.ny + tile.y - 1) / tile.y;
@@ -232,7 +254,23 @@ cdf_status setup_tiles(cdf_batch *b, dim3 tile) {
         inst[k].mom_off = b->mom_off[k];
         inst[k].tile_base = (int)tiles.size();
         inst[k].tiles_x = tx;
-        for (int i = 0; i < tx * ty; ++i) tiles.push_back(k);
+        tiles.insert(tiles.end(), (size_t)tx * ty, k);
+        inst[k].node_off = b->node_off[k];
+        int tw = 1, th = 1;
+        pair_tile(p, &tw, &th);
+        const int px = (p.nx + tw - 1) / tw, py = (p.ny + th - 1) / th;
+        inst[k].pair_base = (int)pairs.size();
+        inst[k].pair_x = px;
+        inst[k].tw = tw;
+        inst[k].th = th;
+        inst[k].inv_w1 = ((1u << 20) + tw + 1) / (tw + 2);
+        inst[k].inv_tw = ((1u << 20) + tw - 1) / tw;
+        pairs.insert(pairs.end(), (size_t)px * py, k);
+    }
+    if (!b->d_pair_inst) {
+        BCK(cudaMalloc(&b->d_pair_inst, pairs.size() * sizeof(int)));
+        BCK(cudaMemcpy(b->d_pair_inst, pairs.data(), pairs.size() * sizeof(int), cudaMemcpyHostToDevice));
+        b->pair_tiles = (int)pairs.size();
     }
     cudaFree(b->d_tile_inst);
     b->d_tile_inst = nullptr;
@@ -242,8 +280,8 @@ cdf_status setup_tiles(cdf_batch *b, dim3 tile) {
     b->total_tiles = (int)tiles.size();
     b->tile = tile;
     int per_sm = 0, sms = 0;
-    void (*kern)(const BatchInst *, const int *, int, float *, float *, float *, float *, int, int, int, unsigned *,
-                 unsigned, unsigned long long, int *) = nullptr;
+    void (*kern)(const BatchInst *, const int *, int, float *, float *, const float *, float *, float *, int, int, int,
+                 unsigned *, unsigned, unsigned long long, int *) = nullptr;
     switch (b->m) {
         case 1: kern = batch_kernel<1>; break;
         case 2: kern = batch_kernel<2>; break;
@@ -256,12 +294,13 @@ cdf_status setup_tiles(cdf_batch *b, dim3 tile) {
     return CDF_OK;
 }
 
-cdf_status launch_batch(cdf_batch *b, int nsteps, bool moments_last) {
+// nsteps of the persistent kernel from buffer `parity` (sp_in != sp_out: one step).
+cdf_status enqueue_batch(cdf_batch *b, int nsteps, bool moments_last, int parity, const float *sp_in, float *sp_out) {
     BCK(cudaMemsetAsync(b->d_err, 0, 4 * sizeof(int), b->s));
     BCK(cudaMemsetAsync(b->d_bar, 0, 2 * sizeof(unsigned), b->s));
     unsigned expected = (unsigned)b->grid_blocks + (unsigned)b->extra_arrivals;
-    int parity = b->cur, ml = moments_last ? 1 : 0;
-    void *args[] = {&b->d_inst, &b->d_tile_inst, &b->total_tiles, &b->buf[0], &b->buf[1], &b->sprev, &b->mom,
+    int ml = moments_last ? 1 : 0;
+    void *args[] = {&b->d_inst, &b->d_tile_inst, &b->total_tiles, &b->buf[0], &b->buf[1], &sp_in, &sp_out, &b->mom,
                     &nsteps, &parity, &ml, &b->d_bar, &expected, &b->timeout_ns, &b->d_err};
     const void *kern = nullptr;
     switch (b->m) {
@@ -272,6 +311,12 @@ cdf_status launch_batch(cdf_batch *b, int nsteps, bool moments_last) {
     }
     BCK(cudaLaunchCooperativeKernel(kern, dim3(b->grid_blocks), b->tile, args, 0, b->s));
     BCK(cudaMemcpyAsync(b->h_err, b->d_err, 4 * sizeof(int), cudaMemcpyDeviceToHost, b->s));
+    return CDF_OK;
+}
+
+cdf_status launch_batch(cdf_batch *b, int nsteps, bool moments_last) {
+    cdf_status st = enqueue_batch(b, nsteps, moments_last, b->cur, b->sprev, b->sprev);
+    if (st != CDF_OK) return st;
     if (nsteps & 1) b->cur ^= 1;
     b->t += nsteps;
     return CDF_OK;
@@ -281,15 +326,42 @@ constexpr int kPoolStreams = 32;
 constexpr int kChainGraphSteps = 32;  // even: the buffer parity returns
 
 // S_1(t - 1) plane set that belongs to population buffer `par`.
-float *sprev_of(cdf_batch *b, int par) { return (b->mode == 0 || par == 0) ? b->sprev : b->sprev2; }
+float *sprev_of(cdf_batch *b, int par) {
+    return ((b->mode == 0 && !b->fused) || par == 0) ? b->sprev : b->sprev2;
+}
+
+// Do the steps run as launches that each flip the buffers (all but the persistent kernel)?
+bool in_launches(const cdf_batch *b) { return b->mode >= 1 || b->fused; }
 
 // Kernel launches of the chains for n steps: one per step, or in mode 2 one per
 // two steps plus one single step for an odd n.  Each launch flips the parity.
-int chain_launches(const cdf_batch *b, int nsteps) { return b->mode == 2 ? nsteps / 2 + nsteps % 2 : nsteps; }
+int chain_launches(const cdf_batch *b, int nsteps) {
+    return b->mode == 2 || b->fused ? nsteps / 2 + nsteps % 2 : nsteps;
+}
+
+// Enqueue n steps of all instances as launches of two steps each on the batch
+// stream; an odd n ends with one step of the persistent kernel's code.
+cdf_status enqueue_fused(cdf_batch *b, int nsteps, bool moments_last, int parity0) {
+    int par = parity0;
+    for (int done = 0; done < nsteps; par ^= 1) {
+        const bool two = nsteps - done >= 2;
+        done += two ? 2 : 1;
+        const bool last = moments_last && done == nsteps;
+        if (two) {
+            BCK(launch_step2_batch(b->m, b->kind, b->d_inst, b->d_pair_inst, b->pair_tiles, b->buf[par], b->buf[par ^ 1],
+                                   sprev_of(b, par), sprev_of(b, par ^ 1), last ? b->mom : nullptr, b->s));
+        } else {
+            const cdf_status st = enqueue_batch(b, 1, last, par, sprev_of(b, par), sprev_of(b, par ^ 1));
+            if (st != CDF_OK) return st;
+        }
+    }
+    return CDF_OK;
+}
 
 // Enqueue n steps of every instance as chains of single-lattice step kernels on
 // the stream pool (fork from and join back to the batch stream).
 cdf_status enqueue_chains(cdf_batch *b, int nsteps, bool moments_last, int parity0) {
+    if (b->fused) return enqueue_fused(b, nsteps, moments_last, parity0);
     BCK(cudaEventRecord(b->ev_fork, b->s));
     for (cudaStream_t ps : b->pool) BCK(cudaStreamWaitEvent(ps, b->ev_fork, 0));
     const int launches = chain_launches(b, nsteps);
@@ -364,6 +436,15 @@ bool chain_pair_fits(const cdf_batch *b, dim3 blk, int th) {
     return true;
 }
 
+// Two steps of all instances per launch: wherever every instance has a tiling (not with
+// the barrier's test hook), it is faster than the persistent kernel, which moves twice the bytes.
+bool fused_fits(const cdf_batch *b) {
+    int tw, th;
+    for (const LbParams &p : b->params)
+        if (!pair_tile(p, &tw, &th)) return false;
+    return !b->extra_arrivals;
+}
+
 cdf_status check_err(cdf_batch *b) {
     if (*b->h_err) {
         char m[256];
@@ -397,6 +478,7 @@ cdf_status bautotune(cdf_batch *b) {
                 b->chain_th = it->second.th;
                 return setup_tiles(b, dim3(64, 4));
             }
+            b->fused = fused_fits(b);
             return setup_tiles(b, it->second.shape);
         }
     }
@@ -416,16 +498,26 @@ cdf_status bautotune(cdf_batch *b) {
         cudaEventElapsedTime(&ms, e0, e1);
         return ms;
     };
-    const dim3 tiles[] = {dim3(32, 4), dim3(32, 8), dim3(64, 2), dim3(64, 4), dim3(128, 1), dim3(128, 2),
+    const dim3 tiles[] = {dim3(64, 4), dim3(32, 4), dim3(32, 8), dim3(64, 2), dim3(128, 1), dim3(128, 2),
                           dim3(256, 1)};
+    b->mode = 0;
+    b->fused = fused_fits(b);
     for (const dim3 &c : tiles) {
         cdf_status st = setup_tiles(b, c);
         if (st != CDF_OK) return st;
-        float ms = time_it([&](int n) { return launch_batch(b, n, false); }, steps);
-        if (ms < 0) return bfail(CDF_ECUDA, "autotuning the persistent kernel failed");
-        ms *= (float)kChainGraphSteps / steps;  // per 32 steps, comparable with the chains
+        float ms;
+        if (b->fused) {
+            ms = time_it([&](int n) { return run_chains(b, n, false); }, kChainGraphSteps);
+        } else {
+            ms = time_it([&](int n) { return launch_batch(b, n, false); }, steps);
+            if (ms >= 0) ms *= (float)kChainGraphSteps / steps;  // per 32 steps, comparable with the chains
+        }
+        if (ms < 0) return bfail(CDF_ECUDA, "autotuning the whole-batch kernels failed");
         if (ms < best) { best = ms; choice = {0, c, 0}; }
+        if (b->fused) break;  // the tile shape matters to the persistent kernel only
     }
+    b->fused = false;
+    set_chain_block(b, b->chain_block);  // drops the captured launches
     const dim3 blocks[] = {dim3(128, 1), dim3(128, 2), dim3(256, 1), dim3(64, 4), dim3(32, 8), dim3(128, 0),
                            dim3(256, 0)};  // y == 0: flat launch
     b->mode = 1;
@@ -457,11 +549,12 @@ cdf_status bautotune(cdf_batch *b) {
         g_bmode[key] = choice;
     }
     b->mode = choice.mode;
+    set_chain_block(b, b->mode >= 1 ? choice.shape : b->chain_block);
     if (b->mode >= 1) {
-        set_chain_block(b, choice.shape);
         b->chain_th = choice.th;
         return setup_tiles(b, dim3(64, 4));
     }
+    b->fused = fused_fits(b);
     return setup_tiles(b, choice.shape);
 }
 
@@ -509,13 +602,16 @@ cdf_status cdf_batch_create(int count, const cdf_grid *grids, int m, const cdf_d
         b->pop_off.push_back(b->pop_total);
         b->sp_off.push_back(b->sp_total);
         b->mom_off.push_back(b->mom_total);
+        b->node_off.push_back(b->nodes);
         const long long plane = b->params[k].plane;
         b->pop_total += (long long)(9 + 5 * m) * plane;
         b->sp_total += plane;
         b->mom_total += (long long)(m + 3) * plane;
         b->nodes += (long long)grids[k].nx * grids[k].ny;
         b->stage_floats = std::max(b->stage_floats, (size_t)(m + 3) * grids[k].nx * grids[k].ny);
+        b->max_nodes = std::max(b->max_nodes, (long long)grids[k].nx * grids[k].ny);
     }
+    b->kind = batch_closure_kind(b->params.data(), count);
     b->sprev_planes = sprev_planes;
     b->steps_per_launch = opt->steps_per_launch > 0 ? opt->steps_per_launch : 32;
     b->timeout_ns = opt->barrier_timeout_s > 0 ? (unsigned long long)(opt->barrier_timeout_s * 1e9) : 1000000000ull;
@@ -579,7 +675,10 @@ cdf_status cdf_batch_create(int count, const cdf_grid *grids, int m, const cdf_d
     }
     cdf_status st;
     if (opt->mode >= 1 && opt->tile_x > 0) st = setup_tiles(b, dim3(64, 4));
-    else if (opt->tile_x > 0) st = setup_tiles(b, dim3(opt->tile_x, opt->tile_y));
+    else if (opt->tile_x > 0) {
+        b->fused = fused_fits(b);
+        st = setup_tiles(b, dim3(opt->tile_x, opt->tile_y));
+    }
     else if (b->extra_arrivals) st = setup_tiles(b, dim3(64, 4));
     else st = bautotune(b);
     if (st == CDF_OK && cudaStreamSynchronize(b->s) != cudaSuccess) st = bfail(CDF_ECUDA, "set-up failed");
@@ -623,8 +722,8 @@ cdf_status cdf_batch_step(cdf_batch *b, long long n) {
     BCK(cudaEventRecord(b->ev_in, b->user));
     BCK(cudaStreamWaitEvent(b->s, b->ev_in, 0));
     while (n > 0) {
-        const int k = (int)std::min<long long>(n, b->mode >= 1 ? kChainGraphSteps : b->steps_per_launch);
-        cdf_status st = b->mode >= 1 ? run_chains(b, k, n == k) : launch_batch(b, k, n == k);
+        const int k = (int)std::min<long long>(n, in_launches(b) ? kChainGraphSteps : b->steps_per_launch);
+        cdf_status st = in_launches(b) ? run_chains(b, k, n == k) : launch_batch(b, k, n == k);
         if (st != CDF_OK) return st;
         n -= k;
     }
@@ -656,6 +755,11 @@ cdf_status cdf_batch_init_moments_device(cdf_batch *b, int k, const float *dev_f
     BCK(cudaEventRecord(b->ev_in, b->user));
     BCK(cudaStreamWaitEvent(b->s, b->ev_in, 0));
     const float *src = dev_fields;
+    if (k == -1 && b->count <= 65535) {
+        BCK(launch_init_batch(b->m, b->d_inst, b->count, b->max_nodes, dev_fields, b->buf[b->cur], sprev_of(b, b->cur),
+                              b->mom, b->s));
+        k0 = k1;
+    }
     for (int j = k0; j < k1; ++j) {
         const LbParams &P = b->params[j];
         BCK(launch_init(P, kFP32, src, P.nx, b->buf[b->cur] + b->pop_off[j], sprev_of(b, b->cur) + b->sp_off[j],
@@ -673,6 +777,10 @@ cdf_status cdf_batch_moments_device(cdf_batch *b, int k, float *dev_out) {
     BCK(cudaEventRecord(b->ev_in, b->user));
     BCK(cudaStreamWaitEvent(b->s, b->ev_in, 0));
     float *dst = dev_out;
+    if (k == -1 && b->count <= 65535) {
+        BCK(launch_pack_batch(b->m, b->d_inst, b->count, b->max_nodes, b->mom, dev_out, b->s));
+        k0 = k1;
+    }
     for (int j = k0; j < k1; ++j) {
         const LbParams &P = b->params[j];
         BCK(launch_pack_moments(P, b->mom + b->mom_off[j], dst, b->s));

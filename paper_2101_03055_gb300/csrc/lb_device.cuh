@@ -460,8 +460,8 @@ __device__ __forceinline__ void collide(const LbParams &p, V (&f)[M][5], V (&h)[
         V fm = splat<V>(p.Fbase);
 #pragma unroll
         for (int a = 0; a < M; ++a) fm = vfma(p.beta[a], s.phi[a], fm);
-        Fx = p.g[0] * fm;
-        Fy = p.g[1] * fm;
+        Fx = vmul(p.g[0], fm);
+        Fy = vmul(p.g[1], fm);
     }
 
     // Eq. sum-u and Eq. sum-p (varphi = 0):

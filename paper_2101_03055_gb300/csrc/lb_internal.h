@@ -125,6 +125,38 @@ cudaError_t launch_export_mr(const LbParams &p, int storage, const void *in, con
 cudaError_t launch_pack_moments(const LbParams &p, const float *moments, float *dense,
                                 cudaStream_t s);
 
+// One instance of a batch (lb_batch.cu): its parameters and where its planes, its moments and
+// its part of a dense stack of all instances begin (floats; node_off in nodes), and its
+// tiles in the two tilings.
+struct BatchInst {
+    LbParams p;
+    long long pop_off;   // planes in a population buffer
+    long long sp_off;    // S(t - 1) plane
+    long long mom_off;   // moment planes
+    long long node_off;  // nodes of the instances before it
+    int tile_base;       // first tile and tiles per row, persistent kernel
+    int tiles_x;
+    int pair_base;       // the same for the two-step launches, tiles of tw x th
+    int pair_x;
+    int tw, th;
+    unsigned inv_w1, inv_tw;  // ceil(2^20 / (tw + 2)), ceil(2^20 / tw)
+};
+// Nodes of a tile and the ring around it that step2_batch_kernel holds in shared memory: 51 KB
+// for two scalars, four CTAs of 256 threads an SM.
+constexpr int kBatchRegion = 640;
+// The closure kind (lb_device.cuh) that can run all `count` lattices.
+int batch_closure_kind(const LbParams *p, int count);
+// Two steps of every instance in one launch of `tiles` CTAs; tile_inst names each tile's
+// instance.  On a periodic axis the lattice must be at least tw + 2 (th + 2) nodes long.
+cudaError_t launch_step2_batch(int m, int kind, const BatchInst *inst, const int *tile_inst, int tiles, const float *in,
+                               float *out, const float *sp_in, float *sp_out, float *moments, cudaStream_t s);
+// Initialisation from, and packing into, the dense moment stacks of all instances back to back
+// (count <= 65535 instances of at most max_nodes nodes).
+cudaError_t launch_init_batch(int m, const BatchInst *inst, int count, long long max_nodes, const float *fields,
+                              float *out, float *sprev, float *moments, cudaStream_t s);
+cudaError_t launch_pack_batch(int m, const BatchInst *inst, int count, long long max_nodes, const float *moments,
+                              float *dense, cudaStream_t s);
+
 // Tile-resident persistent step (lb_resident.cu), FP32 storage.  The lattice
 // is cut into tiles_x x tiles_y tiles of tw x th nodes (the last row and column
 // of tiles may be smaller), one co-resident CTA of `threads` threads and

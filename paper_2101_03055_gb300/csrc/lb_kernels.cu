@@ -115,13 +115,13 @@ cudaError_t for_model(const LbParams &p, const F &f) {
 struct SmemOptIn {
     std::atomic<bool> done[64];
     template <typename... KArgs>
-    cudaError_t operator()(void (*kern)(KArgs...)) {
+    cudaError_t operator()(void (*kern)(KArgs...), int bytes = kStep2MaxSmem) {
         int dev = 0;
         cudaError_t e = cudaGetDevice(&dev);
         if (e != cudaSuccess) return e;
         if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
         if (done[dev].load()) return cudaSuccess;
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kStep2MaxSmem);
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
         if (e == cudaSuccess) done[dev].store(true);
         return e;
     }
@@ -352,6 +352,123 @@ __global__ void __launch_bounds__(FW ? FW * FY : step2_max_threads(M), FW ? step
             for (int i = 0; i < 5; ++i) pl.out[9 + 5 * a + i][o0] = f[a][i];
         if (consume) sp_out[o0] = o.s1;
         if (moments) write_moments<M>(moments, P, o0, o);
+    }
+}
+
+// The same for all instances of a batch in one launch: CTA b works on tile b of the
+// batch (instance tile_inst[b]); the instance's parameters are staged in shared
+// memory.  Every instance has output tiles of its own size tw x th, as even a division
+// of its lattice as fits (pair_tile in lb_batch.cu): a 64 x 64 lattice is eight tiles of
+// 32 x 16, where 30 x 14 tiles would be fifteen, 65 % full.  So the nodes of R1 and of the
+// tile are walked in row order, 256 at a time, whatever the width; the shared-memory
+// plane stride is the constant kBatchRegion.  512 cavities of 64 x 64, 64 steps with
+// initialisation and moments: 8.7 ms on the persistent kernel, 4.3 with tiles of 30 x 14 for
+// all, 3.9 now (118 us a launch).  On larger lattices the chains of step2_kernel per instance,
+// which read the parameters as constant operands, stay ahead (64 plumes of 128-512 x 64-256);
+// the autotuner times both.  Bound by instruction issue (563 a warp update with walls in
+// nearly every warp, issue active 56 %).
+// q / d for 0 <= q < 1024, 3 <= d <= 1024, with inv = ceil(2^20 / d).
+__device__ __forceinline__ int small_div(int q, unsigned inv) { return (int)(((unsigned)q * inv) >> 20); }
+
+template <int M, int K>
+__global__ void __launch_bounds__(256, step2_max_threads(M) / 256)
+    step2_batch_kernel(const BatchInst *__restrict__ inst, const int *__restrict__ tile_inst, const float *in,
+                       float *out, const float *sp_in, float *sp_out, float *moments) {
+    constexpr int NP = 9 + 5 * M, SP = kBatchRegion;
+    extern __shared__ float sm[];
+    __shared__ BatchInst me;
+    const int tid = threadIdx.x, lane = tid & 31, warp0 = tid - lane;
+    {
+        // (the tables do not change: read before the wait for the previous launch)
+        const int *const src = reinterpret_cast<const int *>(inst + __ldg(tile_inst + blockIdx.x));
+        for (int w = tid; w < (int)(sizeof(BatchInst) / sizeof(int)); w += 256)
+            reinterpret_cast<int *>(&me)[w] = __ldg(src + w);
+    }
+    __syncthreads();
+    pdl_wait_and_release();
+    const LbParams &p = me.p;
+    const int TW = me.tw, TH = me.th, W1 = TW + 2, H1 = TH + 2;
+    const int lt = blockIdx.x - me.pair_base, ty = lt / me.pair_x;
+    const int X0 = (lt - ty * me.pair_x) * TW, Y0 = ty * TH;
+    const float *const i0 = in + me.pop_off;
+    float *const out0 = out + me.pop_off;
+    const long long P = p.plane;
+    const int pitch = p.pitch, nx = p.nx, ny = p.ny;
+    const int xend = min(X0 + TW, nx), yend = min(Y0 + TH, ny);
+    const bool consume = M >= 2 && closure_has<K>(kConsume, p.skind == 2);
+    const float *const s_in = sp_in + me.sp_off;
+    float *const s_out = sp_out + me.sp_off;
+
+    // ---- step 1: R1 from global memory into shared memory
+    {
+        const auto mk = [pitch](int sx, int sy) { return sy * pitch + sx; };
+        const auto ld = [i0, &p, P](int plane, int off) { return __ldg(i0 + plane * P + CDF_CHK(p, off, P, 1)); };
+        const unsigned inv = me.inv_w1;
+        for (int base = warp0; base < W1 * H1; base += 256) {
+            const int l = base + lane, ly = small_div(l, inv), lx = l - ly * W1;
+            const int xu = X0 - 1 + lx, yu = Y0 - 1 + ly;
+            const bool ok = l < W1 * H1 && xu <= xend && yu <= yend && (p.periodic_x || (xu >= 0 && xu < nx)) &&
+                            (p.periodic_y || (yu >= 0 && yu < ny));
+            const int gx = xu < 0 ? xu + nx : (xu >= nx ? xu - nx : xu);
+            const int gy = yu < 0 ? yu + ny : (yu >= ny ? yu - ny : yu);
+            const bool general = ok && !inner_node(p, gx, gy);
+            float h[9], f[M][5];
+            if (!__any_sync(0xffffffffu, general)) {
+                if (!ok) continue;
+                pull_node<M, true, K>(p, gx, gy, mk, ld, f, h);
+            } else {
+                if (!ok) continue;
+                pull_node<M, false, K>(p, gx, gy, mk, ld, f, h);
+            }
+            const int o0 = CDF_CHK(p, gy * pitch + gx, P, 2), l0 = CDF_CHK(p, l, SP, 3);
+            NodeOut<M> o;
+            collide<M, K>(p, f, h, node_pref<K>(p, gx, gy), consume ? s_in[o0] : 0.f, false, o);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) sm[i * SP + l0] = h[i];
+#pragma unroll
+            for (int a = 0; a < M; ++a)
+#pragma unroll
+                for (int i = 0; i < 5; ++i) sm[(9 + 5 * a + i) * SP + l0] = f[a][i];
+            if (consume) sm[NP * SP + l0] = o.s1;
+        }
+    }
+    __syncthreads();
+
+    // ---- step 2: the tile from shared memory into global memory
+    const auto lds = [&p](int plane, int off) { return sm[plane * SP + CDF_CHK(p, off, SP, 4)]; };
+    const auto mk_in = [W1, X0, Y0](int sx, int sy) { return (sy - Y0 + 1) * W1 + (sx - X0 + 1); };
+    const auto mk_gen = [W1, H1, X0, Y0, nx, ny](int sx, int sy) {
+        int a = sx - X0 + 1, b = sy - Y0 + 1;
+        a = a < 0 ? a + nx : (a >= W1 ? a - nx : a);
+        b = b < 0 ? b + ny : (b >= H1 ? b - ny : b);
+        return b * W1 + a;
+    };
+    float *const mom = moments ? moments + me.mom_off : nullptr;
+    const unsigned inv = me.inv_tw;
+    for (int base = warp0; base < TW * TH; base += 256) {
+        const int q = base + lane, oy = small_div(q, inv), x = X0 + q - oy * TW, y = Y0 + oy;
+        const bool ok = q < TW * TH && x < nx && y < ny;
+        const bool general = ok && !inner_node(p, x, y);
+        float h[9], f[M][5];
+        if (!__any_sync(0xffffffffu, general)) {
+            if (!ok) continue;
+            pull_node<M, true, K>(p, x, y, mk_in, lds, f, h);
+        } else {
+            if (!ok) continue;
+            pull_node<M, false, K>(p, x, y, mk_gen, lds, f, h);
+        }
+        const int o0 = CDF_CHK(p, y * pitch + x, P, 2);
+        NodeOut<M> o;
+        collide<M, K>(p, f, h, node_pref<K>(p, x, y),
+                      consume ? sm[NP * SP + CDF_CHK(p, (oy + 1) * W1 + x - X0 + 1, SP, 4)] : 0.f, false, o);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) out0[i * P + o0] = h[i];
+#pragma unroll
+        for (int a = 0; a < M; ++a)
+#pragma unroll
+            for (int i = 0; i < 5; ++i) out0[(9 + 5 * a + i) * P + o0] = f[a][i];
+        if (consume) s_out[o0] = o.s1;
+        if (mom) write_moments<M>(mom, P, o0, o);
     }
 }
 
@@ -645,12 +762,9 @@ __global__ void init_kernel_case1(const LbParams p, const float *__restrict__ fi
 
 // ---- initialisation from moments (collide-only pass at t = 0) ------------------
 template <int M, typename T>
-__global__ void init_kernel(const LbParams p, const float *__restrict__ fields, int fpitch,
-                            T *__restrict__ out, float *__restrict__ sprev,
-                            float *__restrict__ moments) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    if (x >= p.nx || y >= p.ny) return;
+__device__ __forceinline__ void init_node(const LbParams &p, int x, int y, const float *__restrict__ fields, int fpitch,
+                                          T *__restrict__ out, float *__restrict__ sprev,
+                                          float *__restrict__ moments) {
     const long long P = p.plane, FP = (long long)fpitch * p.ny;
     const long long o0 = (long long)y * p.pitch + x, i0 = (long long)y * fpitch + x;
     float phi[M], phid[M];
@@ -665,7 +779,7 @@ __global__ void init_kernel(const LbParams p, const float *__restrict__ fields, 
     float fm = p.Fbase;
 #pragma unroll
     for (int a = 0; a < M; ++a) fm = fmaf(p.beta[a], phi[a], fm);
-    const float Fx = p.g[0] * fm, Fy = p.g[1] * fm;
+    const float Fx = __fmul_rn(p.g[0], fm), Fy = __fmul_rn(p.g[1], fm);
     // f = f^eq(phi, u); h = h^eq(u, p) - F_i / 2 (moments then return the inputs)
     float f[M][5], h[9];
     const float usq = usq_of(ux, uy);
@@ -682,6 +796,43 @@ __global__ void init_kernel(const LbParams p, const float *__restrict__ fields, 
     store_node<M, T>(out, P, o0, f, h);
     if (M >= 2 && p.skind == 2) sprev[o0] = o.s1;
     write_moments<M>(moments, P, o0, o);
+}
+
+template <int M, typename T>
+__global__ void init_kernel(const LbParams p, const float *__restrict__ fields, int fpitch,
+                            T *__restrict__ out, float *__restrict__ sprev,
+                            float *__restrict__ moments) {
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    if (x < p.nx && y < p.ny) init_node<M, T>(p, x, y, fields, fpitch, out, sprev, moments);
+}
+
+// Initialisation and moment packing of all instances of a batch in one launch each
+// (instance blockIdx.y, its nodes in row order): one launch per instance cost the
+// host about 2.2 us each, 1.1 ms for the 512 instances of a training set.
+template <int M>
+__global__ void init_batch_kernel(const BatchInst *__restrict__ inst, const float *__restrict__ fields,
+                                  float *__restrict__ out, float *__restrict__ sprev, float *__restrict__ moments) {
+    __shared__ LbParams p;
+    const BatchInst *const me = inst + blockIdx.y;
+    if ((long long)blockIdx.x * blockDim.x >= (long long)me->p.nx * me->p.ny) return;
+    for (int w = threadIdx.x; w < (int)(sizeof(LbParams) / sizeof(int)); w += blockDim.x)
+        reinterpret_cast<int *>(&p)[w] = reinterpret_cast<const int *>(&me->p)[w];
+    __syncthreads();
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x, y = idx / p.nx, x = idx - y * p.nx;
+    if (y < p.ny)
+        init_node<M, float>(p, x, y, fields + (M + 3) * me->node_off, p.nx, out + me->pop_off, sprev + me->sp_off,
+                            moments + me->mom_off);
+}
+__global__ void pack_batch_kernel(const BatchInst *__restrict__ inst, int nf, const float *__restrict__ mom,
+                                  float *__restrict__ dense) {
+    const BatchInst *const me = inst + blockIdx.y;
+    const int nx = me->p.nx, n = nx * me->p.ny, idx = blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= n) return;
+    const int y = idx / nx, x = idx - y * nx;
+    const float *const m = mom + me->mom_off + (long long)y * me->p.pitch + x;
+    float *const d = dense + nf * me->node_off + idx;
+    for (int k = 0; k < nf; ++k) d[(long long)k * n] = m[k * me->p.plane];
 }
 
 // Post-collision populations (full values) as dense FP32 planes [9 + 5m][ny][nx].
@@ -998,7 +1149,7 @@ __global__ void init_kernel_mr(const LbParams p, const float *__restrict__ field
     float fm = p.Fbase;
 #pragma unroll
     for (int a = 0; a < M; ++a) fm = fmaf(p.beta[a], phi[a], fm);
-    const float Fx = p.g[0] * fm, Fy = p.g[1] * fm;
+    const float Fx = __fmul_rn(p.g[0], fm), Fy = __fmul_rn(p.g[1], fm);
     float f[M][5], h[9];
     const float uF = fmaf(ux, Fx, __fmul_rn(uy, Fy));
     scalar_equilibrium<M>(phi, phi, ux, uy, f);
@@ -1255,6 +1406,57 @@ cudaError_t step2_mr_dispatch(const LbParams &p, const void *in, const float *mi
         return fixed ? run(step2_kernel_mr<M, T, K, 32, 8, 14>, opt_in_fixed) : run(step2_kernel_mr<M, T, K>, opt_in);
     });
     return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+int batch_closure_kind(const LbParams *p, int count) {
+    int kind = closure_kind(p[0]);
+    for (int k = 1; k < count; ++k) {
+        const int other = closure_kind(p[k]);
+        if (other == kind) continue;
+        const bool both = (kind == kKindForced || kind == kKindPlain) && (other == kKindForced || other == kKindPlain);
+        kind = both ? kKindForced : kAnyClosure;  // the forced kind has every term of the plain one
+    }
+    return kind;
+}
+
+cudaError_t launch_step2_batch(int m, int kind, const BatchInst *inst, const int *tile_inst, int tiles, const float *in,
+                               float *out, const float *sp_in, float *sp_out, float *moments, cudaStream_t s) {
+    const size_t smem = (size_t)(9 + 5 * m + 1) * kBatchRegion * sizeof(float);
+    const auto run = [&](auto *kern, SmemOptIn &opt_in) {
+        const cudaError_t e = opt_in(kern, (int)smem);
+        if (e != cudaSuccess) return e;
+        return launch_pdl_smem(kern, dim3(tiles), dim3(256), smem, s, inst, tile_inst, in, out, sp_in, sp_out, moments);
+    };
+    static SmemOptIn o1, o2[4], o3, o4;
+    cudaError_t e = cudaErrorInvalidValue;
+    if (m == 1) e = run(step2_batch_kernel<1, kAnyClosure>, o1);
+    if (m == 2 && kind == kKindPlume) e = run(step2_batch_kernel<2, kKindPlume>, o2[0]);
+    else if (m == 2 && kind == kKindForced) e = run(step2_batch_kernel<2, kKindForced>, o2[1]);
+    else if (m == 2 && kind == kKindPlain) e = run(step2_batch_kernel<2, kKindPlain>, o2[2]);
+    else if (m == 2) e = run(step2_batch_kernel<2, kAnyClosure>, o2[3]);
+    if (m == 3) e = run(step2_batch_kernel<3, kAnyClosure>, o3);
+    if (m == 4) e = run(step2_batch_kernel<4, kAnyClosure>, o4);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+cudaError_t launch_init_batch(int m, const BatchInst *inst, int count, long long max_nodes, const float *fields,
+                              float *out, float *sprev, float *moments, cudaStream_t s) {
+    const dim3 grid((unsigned)((max_nodes + 255) / 256), (unsigned)count);
+    switch (m) {
+        case 1: init_batch_kernel<1><<<grid, 256, 0, s>>>(inst, fields, out, sprev, moments); break;
+        case 2: init_batch_kernel<2><<<grid, 256, 0, s>>>(inst, fields, out, sprev, moments); break;
+        case 3: init_batch_kernel<3><<<grid, 256, 0, s>>>(inst, fields, out, sprev, moments); break;
+        case 4: init_batch_kernel<4><<<grid, 256, 0, s>>>(inst, fields, out, sprev, moments); break;
+        default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
+}
+
+cudaError_t launch_pack_batch(int m, const BatchInst *inst, int count, long long max_nodes, const float *moments,
+                              float *dense, cudaStream_t s) {
+    pack_batch_kernel<<<dim3((unsigned)((max_nodes + 255) / 256), (unsigned)count), 256, 0, s>>>(inst, m + 3, moments,
+                                                                                                  dense);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_step2_mr(const LbParams &p, int storage, const void *in, const float *moments_in, void *out,
