@@ -14,6 +14,8 @@
 #include <atomic>
 #include <cmath>
 #include <cstdint>
+#include <initializer_list>
+#include <type_traits>
 #include <utility>
 
 #include "../../include/cdf_nn.h"
@@ -994,149 +996,270 @@ __global__ void bias_grad_kernel(const __nv_bfloat16 *__restrict__ dy, float *__
     if (threadIdx.x < 8) atomicAdd(db + c0 + threadIdx.x, red[threadIdx.x][0]);
 }
 
-__global__ void relu_bwd_kernel(__nv_bfloat16 *__restrict__ d, const __nv_bfloat16 *__restrict__ y, long long n) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n && !(__bfloat162float(y[i]) > 0.f)) d[i] = __float2bfloat16_rn(0.f);
+// The layers between the convolutions move each element once or twice and compute
+// next to nothing, so they are bound by memory accesses: a thread takes V = 8
+// channels, one 16-byte access each, wherever the channel counts and slices are multiples
+// of 8 and the pointers lie on 16 bytes, else one (2-byte accesses reached a tenth of
+// the copy bandwidth: 32 x 64 x 64 x 64 channels upsampled in 45 us, with 16 bytes in 7).
+// Indexes are 32-bit where the element count allows (I = int).
+template <int V>
+struct alignas(2 * V) Chan {  // V consecutive BF16 values
+    __nv_bfloat16 e[V];
+};
+template <int V>
+__device__ __forceinline__ Chan<V> load_chan(const __nv_bfloat16 *p) {
+    Chan<V> r;
+    if constexpr (V == 8) {
+        const uint4 q = *reinterpret_cast<const uint4 *>(p);
+        *reinterpret_cast<uint4 *>(r.e) = q;
+    } else {
+        r.e[0] = *p;
+    }
+    return r;
+}
+template <int V>
+__device__ __forceinline__ void store_chan(__nv_bfloat16 *p, const Chan<V> &r) {
+    if constexpr (V == 8) *reinterpret_cast<uint4 *>(p) = *reinterpret_cast<const uint4 *>(r.e);
+    else *p = r.e[0];
 }
 
+template <int V>
+__global__ void relu_bwd_kernel(__nv_bfloat16 *__restrict__ d, const __nv_bfloat16 *__restrict__ y, long long n) {
+    const long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * V;
+    if (i >= n) return;
+    const Chan<V> yv = load_chan<V>(y + i);
+    Chan<V> dv = load_chan<V>(d + i);
+#pragma unroll
+    for (int k = 0; k < V; ++k)
+        if (!(__bfloat162float(yv.e[k]) > 0.f)) dv.e[k] = __float2bfloat16_rn(0.f);
+    store_chan<V>(d + i, dv);
+}
+
+template <int V, class I>
 __global__ void avgpool2_fwd_kernel(const __nv_bfloat16 *__restrict__ x, __nv_bfloat16 *__restrict__ y, int N, int H,
                                     int W, int C) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const I i = (I)blockIdx.x * blockDim.x + threadIdx.x, G = C / V;
     const int Ho = H / 2, Wo = W / 2;
-    const long long n_out = (long long)N * Ho * Wo * C;
-    if (i >= n_out) return;
-    const int c = (int)(i % C);
-    long long q = i / C;
+    if (i >= (I)N * Ho * Wo * G) return;
+    const int c = (int)(i % G) * V;
+    I q = i / G;
     const int xo = (int)(q % Wo);
     q /= Wo;
     const int yo = (int)(q % Ho);
-    const int n = (int)(q / Ho);
-    float s = 0.f;
+    const long long n = q / Ho;
+    float s[V];
+#pragma unroll
+    for (int k = 0; k < V; ++k) s[k] = 0.f;
 #pragma unroll
     for (int a = 0; a < 2; ++a)
 #pragma unroll
-        for (int b = 0; b < 2; ++b)
-            s += __bfloat162float(x[(((long long)n * H + 2 * yo + a) * W + 2 * xo + b) * C + c]);
-    y[i] = __float2bfloat16_rn(0.25f * s);
+        for (int b = 0; b < 2; ++b) {
+            const Chan<V> v = load_chan<V>(x + ((n * H + 2 * yo + a) * W + 2 * xo + b) * C + c);
+#pragma unroll
+            for (int k = 0; k < V; ++k) s[k] += __bfloat162float(v.e[k]);
+        }
+    Chan<V> o;
+#pragma unroll
+    for (int k = 0; k < V; ++k) o.e[k] = __float2bfloat16_rn(0.25f * s[k]);
+    store_chan<V>(y + (long long)i * V, o);
 }
 
+// One thread per dy element: the four pixels of its window get the same value.
+template <int V, class I>
 __global__ void avgpool2_bwd_kernel(const __nv_bfloat16 *__restrict__ dy, __nv_bfloat16 *__restrict__ dx, int N, int H,
                                     int W, int C) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;  // over dx
-    const long long n_in = (long long)N * H * W * C;
-    if (i >= n_in) return;
-    const int c = (int)(i % C);
-    long long q = i / C;
-    const int xx = (int)(q % W);
-    q /= W;
-    const int yy = (int)(q % H);
-    const int n = (int)(q / H);
-    const float g = __bfloat162float(dy[(((long long)n * (H / 2) + yy / 2) * (W / 2) + xx / 2) * C + c]);
-    dx[i] = __float2bfloat16_rn(0.25f * g);
+    const I i = (I)blockIdx.x * blockDim.x + threadIdx.x, G = C / V;
+    const int Ho = H / 2, Wo = W / 2;
+    if (i >= (I)N * Ho * Wo * G) return;
+    const int c = (int)(i % G) * V;
+    I q = i / G;
+    const int xo = (int)(q % Wo);
+    q /= Wo;
+    const int yo = (int)(q % Ho);
+    const long long n = q / Ho;
+    Chan<V> g = load_chan<V>(dy + (long long)i * V);
+#pragma unroll
+    for (int k = 0; k < V; ++k) g.e[k] = __float2bfloat16_rn(0.25f * __bfloat162float(g.e[k]));
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int b = 0; b < 2; ++b) store_chan<V>(dx + ((n * H + 2 * yo + a) * W + 2 * xo + b) * C + c, g);
 }
 
-// Nearest 2x upsampling of x [N, H, W, C] into channels [coff, coff + C) of y [N, 2H, 2W, Cy].
+// Nearest 2x upsampling of x [N, H, W, C] into channels [coff, coff + C) of y [N, 2H, 2W, Cy];
+// one thread per x element.
+template <int V, class I>
 __global__ void upsample2_fwd_kernel(const __nv_bfloat16 *__restrict__ x, __nv_bfloat16 *__restrict__ y, int N, int H,
                                      int W, int C, int Cy, int coff) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;  // over y's selected channels
-    const long long n_out = (long long)N * 2 * H * 2 * W * C;
-    if (i >= n_out) return;
-    const int c = (int)(i % C);
-    long long q = i / C;
-    const int xo = (int)(q % (2 * W));
-    q /= 2 * W;
-    const int yo = (int)(q % (2 * H));
-    const int n = (int)(q / (2 * H));
-    y[(((long long)n * 2 * H + yo) * 2 * W + xo) * Cy + coff + c] = x[(((long long)n * H + yo / 2) * W + xo / 2) * C + c];
+    const I i = (I)blockIdx.x * blockDim.x + threadIdx.x, G = C / V;
+    if (i >= (I)N * H * W * G) return;
+    const int c = (int)(i % G) * V;
+    I q = i / G;
+    const int xx = (int)(q % W);
+    const long long row = q / W;  // n H + y
+    const Chan<V> v = load_chan<V>(x + (long long)i * V);
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int b = 0; b < 2; ++b) store_chan<V>(y + ((2 * row + a) * 2 * W + 2 * xx + b) * Cy + coff + c, v);
 }
 
 // Backward of the above: dx[n][y][x][c] = sum of the 4 covering dy values (channels coff..coff+C of dy).
+template <int V, class I>
 __global__ void upsample2_bwd_kernel(const __nv_bfloat16 *__restrict__ dy, __nv_bfloat16 *__restrict__ dx, int N, int H,
                                      int W, int C, int Cy, int coff) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long n_in = (long long)N * H * W * C;
-    if (i >= n_in) return;
-    const int c = (int)(i % C);
-    long long q = i / C;
+    const I i = (I)blockIdx.x * blockDim.x + threadIdx.x, G = C / V;
+    if (i >= (I)N * H * W * G) return;
+    const int c = (int)(i % G) * V;
+    I q = i / G;
     const int xx = (int)(q % W);
-    q /= W;
-    const int yy = (int)(q % H);
-    const int n = (int)(q / H);
-    float s = 0.f;
+    const long long row = q / W;
+    float s[V];
+#pragma unroll
+    for (int k = 0; k < V; ++k) s[k] = 0.f;
 #pragma unroll
     for (int a = 0; a < 2; ++a)
 #pragma unroll
-        for (int b = 0; b < 2; ++b)
-            s += __bfloat162float(dy[(((long long)n * 2 * H + 2 * yy + a) * 2 * W + 2 * xx + b) * Cy + coff + c]);
-    dx[i] = __float2bfloat16_rn(s);
+        for (int b = 0; b < 2; ++b) {
+            const Chan<V> v = load_chan<V>(dy + ((2 * row + a) * 2 * W + 2 * xx + b) * Cy + coff + c);
+#pragma unroll
+            for (int k = 0; k < V; ++k) s[k] += __bfloat162float(v.e[k]);
+        }
+    Chan<V> o;
+#pragma unroll
+    for (int k = 0; k < V; ++k) o.e[k] = __float2bfloat16_rn(s[k]);
+    store_chan<V>(dx + (long long)i * V, o);
 }
 
 // y[:, :, :, dst_off + c] = x[:, :, :, src_off + c] for c < count (skip concat / split).
+template <int V, class I>
 __global__ void copy_channels_kernel(const __nv_bfloat16 *__restrict__ x, __nv_bfloat16 *__restrict__ y, long long P,
                                      int Cx, int Cy, int src_off, int dst_off, int count, int accumulate) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= P * count) return;
-    const long long p = i / count;
-    const int c = (int)(i - p * count);
-    const float v = __bfloat162float(x[p * Cx + src_off + c]);
-    __nv_bfloat16 *d = y + p * Cy + dst_off + c;
-    *d = __float2bfloat16_rn(accumulate ? v + __bfloat162float(*d) : v);
+    const I i = (I)blockIdx.x * blockDim.x + threadIdx.x, G = count / V;
+    const long long p = i / G;
+    if (p >= P) return;
+    const int c = (int)(i % G) * V;
+    Chan<V> v = load_chan<V>(x + p * Cx + src_off + c);
+    __nv_bfloat16 *const d = y + p * Cy + dst_off + c;
+    const Chan<V> old = accumulate ? load_chan<V>(d) : v;
+#pragma unroll
+    for (int k = 0; k < V; ++k) {
+        const float f = __bfloat162float(v.e[k]);
+        v.e[k] = __float2bfloat16_rn(accumulate ? f + __bfloat162float(old.e[k]) : f);
+    }
+    store_chan<V>(d, v);
 }
 
-// 1x1 output head in FP32 arithmetic: out[p][o] = sum_c x[p][c] w[o][c] + b[o].
+// 1x1 output head in FP32 arithmetic: out[p][o] = sum_c x[p][c] w[o][c] + b[o]; one thread per
+// pixel and up to four outputs.
+template <int V>
 __global__ void head_fwd_kernel(const __nv_bfloat16 *__restrict__ x, const float *__restrict__ w,
                                 const float *__restrict__ b, float *__restrict__ out, long long P, int C, int O) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= P * O) return;
-    const long long p = i / O;
-    const int o = (int)(i - p * O);
-    float s = b[o];
-    for (int c = 0; c < C; ++c) s = fmaf(__bfloat162float(x[p * C + c]), w[o * C + c], s);
-    out[i] = s;
+    const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int o0 = blockIdx.y * 4, no = min(4, O - o0);
+    if (p >= P) return;
+    float s[4];
+#pragma unroll
+    for (int o = 0; o < 4; ++o) s[o] = o < no ? b[o0 + o] : 0.f;
+    for (int c = 0; c < C; c += V) {
+        const Chan<V> v = load_chan<V>(x + p * C + c);
+#pragma unroll
+        for (int k = 0; k < V; ++k)
+#pragma unroll
+            for (int o = 0; o < 4; ++o)
+                if (o < no) s[o] = fmaf(__bfloat162float(v.e[k]), __ldg(w + (o0 + o) * C + c + k), s[o]);
+    }
+#pragma unroll
+    for (int o = 0; o < 4; ++o)
+        if (o < no) out[p * O + o0 + o] = s[o];
 }
 
 // dx[p][c] = sum_o dout[p][o] w[o][c]
+template <int V, class I>
 __global__ void head_bwd_data_kernel(const float *__restrict__ dout, const float *__restrict__ w,
                                      __nv_bfloat16 *__restrict__ dx, long long P, int C, int O) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= P * C) return;
-    const long long p = i / C;
-    const int c = (int)(i - p * C);
-    float s = 0.f;
-    for (int o = 0; o < O; ++o) s = fmaf(dout[p * O + o], w[o * C + c], s);
-    dx[i] = __float2bfloat16_rn(s);
-}
-
-// dw[o][c] += sum_p dout[p][o] x[p][c]; db[o] += sum_p dout[p][o]  (one block per (o, c-chunk) pair, grid-stride)
-__global__ void head_bwd_weight_kernel(const __nv_bfloat16 *__restrict__ x, const float *__restrict__ dout,
-                                       float *__restrict__ dw, float *__restrict__ db, long long P, int C, int O) {
-    const int o = blockIdx.x / (C + 1), c = blockIdx.x % (C + 1);  // c == C: bias
-    float s = 0.f;
-    for (long long p = (long long)blockIdx.y * blockDim.x + threadIdx.x; p < P; p += (long long)gridDim.y * blockDim.x)
-        s += dout[p * O + o] * (c < C ? __bfloat162float(x[p * C + c]) : 1.f);
-    __shared__ float red[256];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int st = blockDim.x / 2; st > 0; st >>= 1) {
-        if ((int)threadIdx.x < st) red[threadIdx.x] += red[threadIdx.x + st];
-        __syncthreads();
+    const I i = (I)blockIdx.x * blockDim.x + threadIdx.x, G = C / V;
+    const long long p = i / G;
+    if (p >= P) return;
+    const int c = (int)(i % G) * V;
+    float s[V];
+#pragma unroll
+    for (int k = 0; k < V; ++k) s[k] = 0.f;
+    for (int o = 0; o < O; ++o) {
+        const float d = dout[p * O + o];
+#pragma unroll
+        for (int k = 0; k < V; ++k) s[k] = fmaf(d, __ldg(w + o * C + c + k), s[k]);
     }
-    if (threadIdx.x == 0) atomicAdd(c < C ? dw + o * C + c : db + o, red[0]);
+    Chan<V> r;
+#pragma unroll
+    for (int k = 0; k < V; ++k) r.e[k] = __float2bfloat16_rn(s[k]);
+    store_chan<V>(dx + (long long)i * V, r);
 }
 
-// Mean squared error over n values; loss (FP32 sum, atomically added) and its gradient 2 (pred - target) / n.
-__global__ void mse_kernel(const float *__restrict__ pred, const float *__restrict__ target, float *__restrict__ grad,
-                           float *__restrict__ loss, long long n) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+// dw[o][c] += sum_p dout[p][o] x[p][c]; db[o] += sum_p dout[p][o].  A warp takes 64
+// consecutive pixels (lane = channel, four outputs at a time), the block's eight
+// warps are added in shared memory, one atomic addition per block and weight.
+constexpr int kHeadRun = 64;
+__global__ void __launch_bounds__(256) head_bwd_weight_kernel(const __nv_bfloat16 *__restrict__ x,
+                                                              const float *__restrict__ dout,
+                                                              float *__restrict__ dw, float *__restrict__ db,
+                                                              long long P, int C, int O) {
+    __shared__ float red[8][5][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const long long p0 = ((long long)blockIdx.x * 8 + warp) * kHeadRun, p1 = min(P, p0 + kHeadRun);
+    for (int o0 = 0; o0 < O; o0 += 4)
+        for (int c0 = 0; c0 < C; c0 += 32) {
+            const int c = c0 + lane;
+            const bool bias = c0 == 0 && lane < min(4, O - o0);  // these lanes also add up dout
+            float s[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+            for (long long p = p0; p < p1; ++p) {
+                const float xv = c < C ? __bfloat162float(x[p * C + c]) : 0.f;
+#pragma unroll
+                for (int o = 0; o < 4; ++o)
+                    if (o0 + o < O) s[o] += dout[p * O + o0 + o] * xv;
+                if (bias) s[4] += dout[p * O + o0 + lane];
+            }
+            __syncthreads();
+#pragma unroll
+            for (int o = 0; o < 5; ++o) red[warp][o][lane] = s[o];
+            __syncthreads();
+            if (warp < 5) {
+                float t = 0.f;
+#pragma unroll
+                for (int k = 0; k < 8; ++k) t += red[k][warp][lane];
+                if (warp < 4 && o0 + warp < O && c < C) atomicAdd(dw + (o0 + warp) * C + c, t);
+                if (warp == 4 && bias) atomicAdd(db + o0 + lane, t);
+            }
+        }
+}
+
+// Mean squared error over n values; loss (FP32 sum, one atomic addition per block of 2048 values) and
+// its gradient 2 (pred - target) / n.
+__global__ void __launch_bounds__(256) mse_kernel(const float *__restrict__ pred, const float *__restrict__ target,
+                                                  float *__restrict__ grad, float *__restrict__ loss, long long n) {
+    const long long i0 = (long long)blockIdx.x * 2048 + threadIdx.x;
     float e = 0.f;
-    if (i < n) {
-        const float d = pred[i] - target[i];
-        grad[i] = 2.f * d / (float)n;
-        e = d * d / (float)n;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const long long i = i0 + 256 * k;
+        if (i < n) {
+            const float d = pred[i] - target[i];
+            grad[i] = 2.f * d / (float)n;
+            e += d * d / (float)n;
+        }
     }
+    __shared__ float red[8];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) e += __shfl_down_sync(0xffffffffu, e, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(loss, e);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = e;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float t = 0.f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) t += red[k];
+        atomicAdd(loss, t);
+    }
 }
 
 // Adam on FP32 master weights; refreshes the BF16 copy when one is given.
@@ -1156,6 +1279,25 @@ __global__ void adam_kernel(float *__restrict__ w, const float *__restrict__ g, 
 }
 
 inline unsigned blocks_for(long long n, int t = 256) { return (unsigned)((n + t - 1) / t); }
+
+// May a kernel take 8 channels a thread: all counts and offsets multiples of 8, all pointers on
+// 16 bytes?
+bool by_eight(std::initializer_list<long long> counts, std::initializer_list<const void *> pointers) {
+    for (long long c : counts)
+        if (c % 8) return false;
+    for (const void *p : pointers)
+        if (reinterpret_cast<uintptr_t>(p) & 15) return false;
+    return true;
+}
+// f(Int<V>, index type) for n elements: 8 a thread and 32-bit indexes where possible.
+template <int N>
+using Int = std::integral_constant<int, N>;
+template <class F>
+void with_width(bool eight, long long n, const F &f) {
+    if (eight && n < (1ll << 30)) f(Int<8>{}, 0);
+    else if (eight) f(Int<8>{}, 0ll);
+    else f(Int<1>{}, 0ll);
+}
 
 thread_local char g_nn_err[256] = "";
 cdf_nn_status nn_fail(const char *m) {
@@ -1268,40 +1410,56 @@ cdf_nn_status cdf_nn_conv3x3_bwd_weight(const void *x, const void *dy, float *dw
 
 cdf_nn_status cdf_nn_relu_bwd(void *d, const void *y, long long n, void *stream) {
     if (!d || !y || n < 0) return nn_fail("relu_bwd: bad arguments");
-    if (n) relu_bwd_kernel<<<blocks_for(n), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        static_cast<__nv_bfloat16 *>(d), static_cast<const __nv_bfloat16 *>(y), n);
+    if (n)
+        with_width(by_eight({n}, {d, y}), n, [&](auto v, auto) {
+            constexpr int V = decltype(v)::value;
+            relu_bwd_kernel<V><<<blocks_for(n / V), 256, 0, static_cast<cudaStream_t>(stream)>>>(
+                static_cast<__nv_bfloat16 *>(d), static_cast<const __nv_bfloat16 *>(y), n);
+        });
     return launched();
 }
 
 cdf_nn_status cdf_nn_avgpool2_fwd(const void *x, void *y, int N, int H, int W, int C, void *stream) {
     if (!x || !y || H % 2 || W % 2) return nn_fail("avgpool2: H and W must be even");
     const long long n = (long long)N * (H / 2) * (W / 2) * C;
-    avgpool2_fwd_kernel<<<blocks_for(n), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        static_cast<const __nv_bfloat16 *>(x), static_cast<__nv_bfloat16 *>(y), N, H, W, C);
+    with_width(by_eight({C}, {x, y}), n, [&](auto v, auto index) {
+        constexpr int V = decltype(v)::value;
+        avgpool2_fwd_kernel<V, decltype(index)><<<blocks_for(n / V), 256, 0, static_cast<cudaStream_t>(stream)>>>(
+            static_cast<const __nv_bfloat16 *>(x), static_cast<__nv_bfloat16 *>(y), N, H, W, C);
+    });
     return launched();
 }
 
 cdf_nn_status cdf_nn_avgpool2_bwd(const void *dy, void *dx, int N, int H, int W, int C, void *stream) {
     if (!dy || !dx || H % 2 || W % 2) return nn_fail("avgpool2: H and W must be even");
-    const long long n = (long long)N * H * W * C;
-    avgpool2_bwd_kernel<<<blocks_for(n), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        static_cast<const __nv_bfloat16 *>(dy), static_cast<__nv_bfloat16 *>(dx), N, H, W, C);
+    const long long n = (long long)N * (H / 2) * (W / 2) * C;
+    with_width(by_eight({C}, {dy, dx}), 4 * n, [&](auto v, auto index) {
+        constexpr int V = decltype(v)::value;
+        avgpool2_bwd_kernel<V, decltype(index)><<<blocks_for(n / V), 256, 0, static_cast<cudaStream_t>(stream)>>>(
+            static_cast<const __nv_bfloat16 *>(dy), static_cast<__nv_bfloat16 *>(dx), N, H, W, C);
+    });
     return launched();
 }
 
 cdf_nn_status cdf_nn_upsample2_fwd(const void *x, void *y, int N, int H, int W, int C, int Cy, int coff, void *stream) {
     if (!x || !y || coff < 0 || coff + C > Cy) return nn_fail("upsample2: bad channel slice");
-    const long long n = (long long)N * 4 * H * W * C;
-    upsample2_fwd_kernel<<<blocks_for(n), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        static_cast<const __nv_bfloat16 *>(x), static_cast<__nv_bfloat16 *>(y), N, H, W, C, Cy, coff);
+    const long long n = (long long)N * H * W * C;
+    with_width(by_eight({C, Cy, coff}, {x, y}), 4 * n, [&](auto v, auto index) {
+        constexpr int V = decltype(v)::value;
+        upsample2_fwd_kernel<V, decltype(index)><<<blocks_for(n / V), 256, 0, static_cast<cudaStream_t>(stream)>>>(
+            static_cast<const __nv_bfloat16 *>(x), static_cast<__nv_bfloat16 *>(y), N, H, W, C, Cy, coff);
+    });
     return launched();
 }
 
 cdf_nn_status cdf_nn_upsample2_bwd(const void *dy, void *dx, int N, int H, int W, int C, int Cy, int coff, void *stream) {
     if (!dy || !dx || coff < 0 || coff + C > Cy) return nn_fail("upsample2: bad channel slice");
     const long long n = (long long)N * H * W * C;
-    upsample2_bwd_kernel<<<blocks_for(n), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        static_cast<const __nv_bfloat16 *>(dy), static_cast<__nv_bfloat16 *>(dx), N, H, W, C, Cy, coff);
+    with_width(by_eight({C, Cy, coff}, {dy, dx}), n, [&](auto v, auto index) {
+        constexpr int V = decltype(v)::value;
+        upsample2_bwd_kernel<V, decltype(index)><<<blocks_for(n / V), 256, 0, static_cast<cudaStream_t>(stream)>>>(
+            static_cast<const __nv_bfloat16 *>(dy), static_cast<__nv_bfloat16 *>(dx), N, H, W, C, Cy, coff);
+    });
     return launched();
 }
 
@@ -1309,17 +1467,24 @@ cdf_nn_status cdf_nn_copy_channels(const void *x, void *y, long long P, int Cx, 
                                    int count, int accumulate, void *stream) {
     if (!x || !y || src_off + count > Cx || dst_off + count > Cy || count < 0) return nn_fail("copy_channels: bad slice");
     const long long n = P * count;
-    if (n) copy_channels_kernel<<<blocks_for(n), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        static_cast<const __nv_bfloat16 *>(x), static_cast<__nv_bfloat16 *>(y), P, Cx, Cy, src_off, dst_off, count,
-        accumulate);
+    if (n)
+        with_width(by_eight({Cx, Cy, src_off, dst_off, count}, {x, y}), n, [&](auto v, auto index) {
+            constexpr int V = decltype(v)::value;
+            copy_channels_kernel<V, decltype(index)><<<blocks_for(n / V), 256, 0, static_cast<cudaStream_t>(stream)>>>(
+                static_cast<const __nv_bfloat16 *>(x), static_cast<__nv_bfloat16 *>(y), P, Cx, Cy, src_off, dst_off,
+                count, accumulate);
+        });
     return launched();
 }
 
 cdf_nn_status cdf_nn_head_fwd(const void *x, const float *w, const float *b, float *out, long long P, int C, int O,
                               void *stream) {
     if (!x || !w || !b || !out) return nn_fail("head_fwd: NULL argument");
-    head_fwd_kernel<<<blocks_for(P * O), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        static_cast<const __nv_bfloat16 *>(x), w, b, out, P, C, O);
+    with_width(by_eight({C}, {x}), P * C, [&](auto v, auto) {
+        constexpr int V = decltype(v)::value;
+        head_fwd_kernel<V><<<dim3(blocks_for(P), (unsigned)((O + 3) / 4)), 256, 0, static_cast<cudaStream_t>(stream)>>>(
+            static_cast<const __nv_bfloat16 *>(x), w, b, out, P, C, O);
+    });
     return launched();
 }
 
@@ -1327,15 +1492,19 @@ cdf_nn_status cdf_nn_head_bwd(const void *x, const float *w, const float *dout, 
                               long long P, int C, int O, void *stream) {
     if (!x || !w || !dout || !dx || !dw || !db) return nn_fail("head_bwd: NULL argument");
     auto s = static_cast<cudaStream_t>(stream);
-    head_bwd_data_kernel<<<blocks_for(P * C), 256, 0, s>>>(dout, w, static_cast<__nv_bfloat16 *>(dx), P, C, O);
-    dim3 g((unsigned)(O * (C + 1)), (unsigned)((P + 256 * 32 - 1) / (256 * 32)));
-    head_bwd_weight_kernel<<<g, 256, 0, s>>>(static_cast<const __nv_bfloat16 *>(x), dout, dw, db, P, C, O);
+    with_width(by_eight({C}, {dx}), P * C, [&](auto v, auto index) {
+        constexpr int V = decltype(v)::value;
+        head_bwd_data_kernel<V, decltype(index)><<<blocks_for(P * C / V), 256, 0, s>>>(
+            dout, w, static_cast<__nv_bfloat16 *>(dx), P, C, O);
+    });
+    head_bwd_weight_kernel<<<blocks_for(P, 8 * kHeadRun), 256, 0, s>>>(static_cast<const __nv_bfloat16 *>(x), dout, dw,
+                                                                       db, P, C, O);
     return launched();
 }
 
 cdf_nn_status cdf_nn_mse(const float *pred, const float *target, float *grad, float *loss, long long n, void *stream) {
     if (!pred || !target || !grad || !loss) return nn_fail("mse: NULL argument");
-    mse_kernel<<<blocks_for(n), 256, 0, static_cast<cudaStream_t>(stream)>>>(pred, target, grad, loss, n);
+    mse_kernel<<<blocks_for(n, 2048), 256, 0, static_cast<cudaStream_t>(stream)>>>(pred, target, grad, loss, n);
     return launched();
 }
 
