@@ -63,6 +63,24 @@ cdf_nn_status cdf_nn_head_fwd(const void *x, const float *w, const float *b, flo
                               void *stream);
 cdf_nn_status cdf_nn_head_bwd(const void *x, const float *w, const float *dout, void *dx, float *dw, float *db,
                               long long P, int C, int O, void *stream);
+/* The same layers fused as the network's two passes use them; the same bits as the calls they
+ * stand for.  ReLU outputs y mask a gradient: it is 0 where y <= 0.
+ * conv3x3_bwd_data, then relu_bwd through the layer's input y [N][H][W][Cin]; */
+cdf_nn_status cdf_nn_conv3x3_bwd_data_relu(const void *dy, const void *w, const void *y, void *dx, int N, int H, int W,
+                                           int Cin, int Cout, void *stream);
+/* upsample2_fwd of x into channels [0, C) of y [N][2H][2W][C + Cs] and skip [N][2H][2W][Cs] into the rest; */
+cdf_nn_status cdf_nn_upsample2_concat(const void *x, const void *skip, void *y, int N, int H, int W, int C, int Cs,
+                                      void *stream);
+/* upsample2_bwd of channels [0, C) of dy [N][2H][2W][Cy], then relu_bwd through y [N][H][W][C]; */
+cdf_nn_status cdf_nn_upsample2_bwd_relu(const void *dy, const void *y, void *dx, int N, int H, int W, int C, int Cy,
+                                        void *stream);
+/* avgpool2_bwd of dp [N][H/2][W/2][C], plus channels [coff, coff + C) of dcat [N][H][W][Cy], then relu_bwd
+ * through y [N][H][W][C]; */
+cdf_nn_status cdf_nn_pool_skip_bwd_relu(const void *dp, const void *dcat, const void *y, void *dx, int N, int H, int W,
+                                        int C, int Cy, int coff, void *stream);
+/* head_bwd, then relu_bwd of dx through the head's input x. */
+cdf_nn_status cdf_nn_head_bwd_relu(const void *x, const float *w, const float *dout, void *dx, float *dw, float *db,
+                                   long long P, int C, int O, void *stream);
 /* Mean squared error over n values: *loss += mean((pred - target)^2) (zero it first),
  * grad = 2 (pred - target) / n. */
 cdf_nn_status cdf_nn_mse(const float *pred, const float *target, float *grad, float *loss, long long n, void *stream);

@@ -116,7 +116,8 @@ __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.
 //               gradient: W[co][8 - tap][ci] as it lies, N-major), once where all of
 //               them fit in the ring, else again for every item;
 //   warp 12     issues the MMAs;
-//   warps 0-3   read the accumulators, add the bias, apply the ReLU and store BF16.
+//   warps 0-3   read the accumulators, add the bias, apply the ReLU (gradient: zero where
+//               `mask`, the ReLU output that fed the layer, is not positive) and store BF16.
 // With nbuf = 2 the next item's copies, this one's MMAs and the last one's stores
 // overlap inside a CTA, with nbuf = 1 (less shared memory) between the CTAs of an SM.
 // K runs tap by tap, 16 channels at a time, as in conv3x3_tc_kernel: the same sums in
@@ -211,6 +212,7 @@ template <bool kBwd, int BN>
 __global__ void __launch_bounds__(kLinThreads) conv3x3_lin_kernel(const __grid_constant__ CUtensorMap wmap,
                                                                   const __nv_bfloat16 *__restrict__ in,
                                                                   const float *__restrict__ bias,
+                                                                  const __nv_bfloat16 *__restrict__ mask,
                                                                   __nv_bfloat16 *__restrict__ out, const LinConv g) {
     extern __shared__ __align__(1024) unsigned char lin_raw[];
     unsigned char *const lin_smem = lin_raw + ((1024u - (smem_u32(lin_raw) & 1023u)) & 1023u);
@@ -417,6 +419,13 @@ __global__ void __launch_bounds__(kLinThreads) conv3x3_lin_kernel(const __grid_c
                             if (bias) v += bv[q];
                             if (g.relu) v = fmaxf(v, 0.f);
                             o[q] = __float2bfloat16_rn(v);
+                        }
+                        if (kBwd && mask) {
+                            const uint4 mv = __ldg(reinterpret_cast<const uint4 *>(mask + (long long)px * g.Cout + n0 + c0) + k);
+                            const __nv_bfloat16 *m = reinterpret_cast<const __nv_bfloat16 *>(&mv);
+#pragma unroll
+                            for (int q = 0; q < 8; ++q)
+                                if (!(__bfloat162float(m[q]) > 0.f)) o[q] = __float2bfloat16_rn(0.f);
                         }
                         *reinterpret_cast<uint4 *>(dst + c0 + 8 * k) = *reinterpret_cast<const uint4 *>(o);
                     }
@@ -691,6 +700,30 @@ inline DeviceShape device_shape() {
 
 constexpr int kMaxSmemCta = 222 * 1024;  // dynamic; the static arrays take the rest of 227 KB
 
+// The plans of the last shapes this thread used, one per slot: choosing one takes a few microseconds
+// of host time, as much as the launch.  A plan is a function of its key alone.
+template <class Plan>
+struct PlanCache {
+    struct Entry {
+        long long key[6];
+        Plan plan;
+        bool used = false;
+    };
+    Entry entry[64];
+    template <class Make>
+    const Plan &get(const long long (&key)[6], const Make &make) {
+        unsigned long long h = 0;
+        for (long long k : key) h = (h ^ (unsigned long long)k) * 0x9E3779B97F4A7C15ull;
+        Entry &e = entry[h >> 58];
+        if (!e.used || !std::equal(key, key + 6, e.key)) {
+            e.plan = make();
+            std::copy(key, key + 6, e.key);
+            e.used = true;
+        }
+        return e.plan;
+    }
+};
+
 // The item shape of conv3x3_lin_kernel for one layer: BN output channels, T tiles of 128
 // positions and one or two slabs, chosen to make the busiest SM's time least.  The
 // estimate, in SM cycles: an item's staging (about 16 bytes a cycle of a CTA's copies and their
@@ -739,8 +772,8 @@ inline LinPlan lin_plan(const LinImage &im, int Cin, int Cout, const DeviceShape
 }
 
 template <bool kBwd, int BN>
-cudaError_t launch_conv_lin(const CUtensorMap &map, const __nv_bfloat16 *in, const float *bias, __nv_bfloat16 *out,
-                            const LinConv &g, const LinPlan &pl, int sms, cudaStream_t s) {
+cudaError_t launch_conv_lin(const CUtensorMap &map, const __nv_bfloat16 *in, const float *bias,
+                            const __nv_bfloat16 *mask, __nv_bfloat16 *out, const LinConv &g, const LinPlan &pl, int sms, cudaStream_t s) {
     static std::atomic<bool> set[64];
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -755,7 +788,7 @@ cudaError_t launch_conv_lin(const CUtensorMap &map, const __nv_bfloat16 *in, con
     }
     const int tiles_n = g.Cout / BN;
     const dim3 grid((unsigned)std::min(g.items, std::max(1, sms * pl.occ / tiles_n)), (unsigned)tiles_n);
-    conv3x3_lin_kernel<kBwd, BN><<<grid, kLinThreads, pl.smem, s>>>(map, in, bias, out, g);
+    conv3x3_lin_kernel<kBwd, BN><<<grid, kLinThreads, pl.smem, s>>>(map, in, bias, mask, out, g);
     return cudaGetLastError();
 }
 
@@ -764,8 +797,8 @@ cudaError_t launch_conv_lin(const CUtensorMap &map, const __nv_bfloat16 *in, con
 // (wide images with many channels, e.g. 384 channels from W = 114 on), for 2^30 positions and
 // more, and for weights off a 16-byte boundary (TMA); the staged im2col kernels take those.
 template <bool kBwd>
-cudaError_t conv_lin(const __nv_bfloat16 *in, const __nv_bfloat16 *w, const float *bias, __nv_bfloat16 *out, int N,
-                     int H, int W, int Cin, int Cout, int relu, cudaStream_t s, bool *ran) {
+cudaError_t conv_lin(const __nv_bfloat16 *in, const __nv_bfloat16 *w, const float *bias,
+                     const __nv_bfloat16 *mask, __nv_bfloat16 *out, int N, int H, int W, int Cin, int Cout, int relu, cudaStream_t s, bool *ran) {
     *ran = false;
     LinConv g{};
     const DeviceShape d = device_shape();
@@ -776,7 +809,8 @@ cudaError_t conv_lin(const __nv_bfloat16 *in, const __nv_bfloat16 *w, const floa
     g.dg = fast_div((uint32_t)Cin / 8);
     g.boxk = Cin % 64 ? 32 : 64;
     g.relu = relu;
-    const LinPlan pl = lin_plan(g.im, Cin, Cout, d);
+    thread_local PlanCache<LinPlan> plans;
+    const LinPlan pl = plans.get({g.im.L, W, Cin, Cout, d.sms, d.smem_sm}, [&] { return lin_plan(g.im, Cin, Cout, d); });
     if (!pl.bn) return cudaSuccess;
     g.dc = fast_div((uint32_t)Cin);
     g.T = pl.t;
@@ -807,11 +841,11 @@ cudaError_t conv_lin(const __nv_bfloat16 *in, const __nv_bfloat16 *w, const floa
     if (r != CUDA_SUCCESS) return cudaSuccess;
     *ran = true;
     switch (pl.bn) {
-        case 256: return launch_conv_lin<kBwd, 256>(map, in, bias, out, g, pl, d.sms, s);
-        case 128: return launch_conv_lin<kBwd, 128>(map, in, bias, out, g, pl, d.sms, s);
-        case 64: return launch_conv_lin<kBwd, 64>(map, in, bias, out, g, pl, d.sms, s);
-        case 32: return launch_conv_lin<kBwd, 32>(map, in, bias, out, g, pl, d.sms, s);
-        default: return launch_conv_lin<kBwd, 16>(map, in, bias, out, g, pl, d.sms, s);
+        case 256: return launch_conv_lin<kBwd, 256>(map, in, bias, mask, out, g, pl, d.sms, s);
+        case 128: return launch_conv_lin<kBwd, 128>(map, in, bias, mask, out, g, pl, d.sms, s);
+        case 64: return launch_conv_lin<kBwd, 64>(map, in, bias, mask, out, g, pl, d.sms, s);
+        case 32: return launch_conv_lin<kBwd, 32>(map, in, bias, mask, out, g, pl, d.sms, s);
+        default: return launch_conv_lin<kBwd, 16>(map, in, bias, mask, out, g, pl, d.sms, s);
     }
 }
 
@@ -831,7 +865,7 @@ inline size_t wgrad_smem(int bn, int co_tile) {
     const int gy = co_tile / 8, gx = bn / 8, spy = lin_stride(kWgK, gy), spx = lin_stride(kWgK + 2, gx);
     return std::max<size_t>(16ull * (kWgStages * (gy * spy + gx * spx) + (16 - gy) * spy), 8 * 256 * sizeof(float));
 }
-inline WgLinPlan wgrad_lin_plan(long long L, long long P, int Cin, int Cout) {
+inline WgLinPlan make_wgrad_lin_plan(long long L, long long P, int Cin, int Cout) {
     constexpr int kSms = 152;  // (the workspace query has no device to ask)
     WgLinPlan w;
     w.co_tile = Cout % 128 == 0 ? 128 : (Cout % 64 == 0 ? 64 : 32);
@@ -862,6 +896,11 @@ inline WgLinPlan wgrad_lin_plan(long long L, long long P, int Cin, int Cout) {
     w.bias_per = (P + bs - 1) / bs;
     w.bias_splits = (int)((P + w.bias_per - 1) / w.bias_per);
     return w;
+}
+
+inline WgLinPlan wgrad_lin_plan(long long L, long long P, int Cin, int Cout) {
+    thread_local PlanCache<WgLinPlan> plans;
+    return plans.get({L, P, Cin, Cout, 0, 0}, [&] { return make_wgrad_lin_plan(L, P, Cin, Cout); });
 }
 
 template <int BN>

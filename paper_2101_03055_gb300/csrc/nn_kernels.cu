@@ -817,7 +817,7 @@ cudaError_t conv_dispatch(const __nv_bfloat16 *in, const __nv_bfloat16 *w, const
     const int BN = Cout_g % 128 == 0 ? 128 : (Cout_g % 64 == 0 ? 64 : (Cout_g % 32 == 0 ? 32 : 16));
     if (g_path == 1 || g_path == 4) {
         bool ran = false;
-        const cudaError_t e = conv_lin<kBwdData>(in, w, bias, out, N, H, W, Cin_g, Cout_g, relu, s, &ran);
+        const cudaError_t e = conv_lin<kBwdData>(in, w, bias, nullptr, out, N, H, W, Cin_g, Cout_g, relu, s, &ran);
         if (ran) return e;
     }
     if (g_path == 3 && !kBwdData) {  // forward: the persistent warp-specialised kernel
@@ -1150,6 +1150,101 @@ __global__ void copy_channels_kernel(const __nv_bfloat16 *__restrict__ x, __nv_b
     store_chan<V>(d, v);
 }
 
+// ---- the same layers fused as the network's passes use them ----------------------
+// (a launch and one pass over the activations less each; the intermediate values are
+// rounded to BF16 where the separate layers store them, so the results are the same bits)
+
+// y[n][yy][xx] = (upsampled x, skip): the first C channels from x [N, H, W, C] by nearest 2x
+// upsampling, the next Cs from skip [N, 2H, 2W, Cs]; one thread per 8 (V) channels of a coarse
+// pixel or of a skip pixel.
+template <int V, class I>
+__global__ void upsample2_concat_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__restrict__ skip,
+                                        __nv_bfloat16 *__restrict__ y, int N, int H, int W, int C, int Cs) {
+    I i = (I)blockIdx.x * blockDim.x + threadIdx.x;
+    const I G = C / V, Gs = Cs / V, nx = (I)N * H * W * G;
+    const int Cy = C + Cs;
+    if (i < nx) {
+        const int c = (int)(i % G) * V;
+        const I q = i / G;
+        const int xx = (int)(q % W);
+        const long long row = q / W;  // n H + y
+        const Chan<V> v = load_chan<V>(x + (long long)i * V);
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+#pragma unroll
+            for (int b = 0; b < 2; ++b) store_chan<V>(y + ((2 * row + a) * 2 * W + 2 * xx + b) * Cy + c, v);
+        return;
+    }
+    i -= nx;
+    if (i >= (I)N * 4 * H * W * Gs) return;
+    const long long p = i / Gs;
+    store_chan<V>(y + p * Cy + C + (int)(i % Gs) * V, load_chan<V>(skip + (long long)i * V));
+}
+
+// Gradient of a ReLU's output y [N, H, W, C] that was upsampled into the first C of dy's Cy
+// channels: dx = sum of the four covering dy values where y > 0, else 0.
+template <int V, class I>
+__global__ void upsample2_bwd_relu_kernel(const __nv_bfloat16 *__restrict__ dy, const __nv_bfloat16 *__restrict__ y,
+                                          __nv_bfloat16 *__restrict__ dx, int N, int H, int W, int C, int Cy) {
+    const I i = (I)blockIdx.x * blockDim.x + threadIdx.x, G = C / V;
+    if (i >= (I)N * H * W * G) return;
+    const int c = (int)(i % G) * V;
+    const I q = i / G;
+    const int xx = (int)(q % W);
+    const long long row = q / W;
+    float s[V];
+#pragma unroll
+    for (int k = 0; k < V; ++k) s[k] = 0.f;
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            const Chan<V> v = load_chan<V>(dy + ((2 * row + a) * 2 * W + 2 * xx + b) * Cy + c);
+#pragma unroll
+            for (int k = 0; k < V; ++k) s[k] += __bfloat162float(v.e[k]);
+        }
+    const Chan<V> m = load_chan<V>(y + (long long)i * V);
+    Chan<V> o;
+#pragma unroll
+    for (int k = 0; k < V; ++k) o.e[k] = __float2bfloat16_rn(__bfloat162float(m.e[k]) > 0.f ? s[k] : 0.f);
+    store_chan<V>(dx + (long long)i * V, o);
+}
+
+// Gradient of a ReLU's output y [N, H, W, C] that was pooled (gradient dp [N, H/2, W/2, C]) and
+// copied into channels [coff, coff + C) of a concatenation (gradient dcat, Cy channels): dx =
+// dp / 4 (BF16) + dcat, where y > 0, else 0.  One thread per pooled element.
+template <int V, class I>
+__global__ void pool_skip_bwd_relu_kernel(const __nv_bfloat16 *__restrict__ dp, const __nv_bfloat16 *__restrict__ dcat,
+                                          const __nv_bfloat16 *__restrict__ y, __nv_bfloat16 *__restrict__ dx, int N,
+                                          int H, int W, int C, int Cy, int coff) {
+    const I i = (I)blockIdx.x * blockDim.x + threadIdx.x, G = C / V;
+    const int Ho = H / 2, Wo = W / 2;
+    if (i >= (I)N * Ho * Wo * G) return;
+    const int c = (int)(i % G) * V;
+    I q = i / G;
+    const int xo = (int)(q % Wo);
+    q /= Wo;
+    const int yo = (int)(q % Ho);
+    const long long n = q / Ho;
+    Chan<V> g = load_chan<V>(dp + (long long)i * V);
+#pragma unroll
+    for (int k = 0; k < V; ++k) g.e[k] = __float2bfloat16_rn(0.25f * __bfloat162float(g.e[k]));
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            const long long p = (n * H + 2 * yo + a) * W + 2 * xo + b;
+            const Chan<V> sk = load_chan<V>(dcat + p * Cy + coff + c), m = load_chan<V>(y + p * C + c);
+            Chan<V> o;
+#pragma unroll
+            for (int k = 0; k < V; ++k) {
+                const float f = __bfloat162float(sk.e[k]) + __bfloat162float(g.e[k]);
+                o.e[k] = __float2bfloat16_rn(__bfloat162float(m.e[k]) > 0.f ? f : 0.f);
+            }
+            store_chan<V>(dx + p * C + c, o);
+        }
+}
+
 // 1x1 output head in FP32 arithmetic: out[p][o] = sum_c x[p][c] w[o][c] + b[o]; one thread per
 // pixel and up to four outputs.
 template <int V>
@@ -1174,10 +1269,11 @@ __global__ void head_fwd_kernel(const __nv_bfloat16 *__restrict__ x, const float
         if (o < no) out[p * O + o0 + o] = s[o];
 }
 
-// dx[p][c] = sum_o dout[p][o] w[o][c]
+// dx[p][c] = sum_o dout[p][o] w[o][c], zero where `mask` (the ReLU output x, or NULL) is not positive
 template <int V, class I>
 __global__ void head_bwd_data_kernel(const float *__restrict__ dout, const float *__restrict__ w,
-                                     __nv_bfloat16 *__restrict__ dx, long long P, int C, int O) {
+                                     const __nv_bfloat16 *__restrict__ mask, __nv_bfloat16 *__restrict__ dx,
+                                     long long P, int C, int O) {
     const I i = (I)blockIdx.x * blockDim.x + threadIdx.x, G = C / V;
     const long long p = i / G;
     if (p >= P) return;
@@ -1191,8 +1287,10 @@ __global__ void head_bwd_data_kernel(const float *__restrict__ dout, const float
         for (int k = 0; k < V; ++k) s[k] = fmaf(d, __ldg(w + o * C + c + k), s[k]);
     }
     Chan<V> r;
+    const Chan<V> m = mask ? load_chan<V>(mask + (long long)i * V) : Chan<V>{};
 #pragma unroll
-    for (int k = 0; k < V; ++k) r.e[k] = __float2bfloat16_rn(s[k]);
+    for (int k = 0; k < V; ++k)
+        r.e[k] = __float2bfloat16_rn(!mask || __bfloat162float(m.e[k]) > 0.f ? s[k] : 0.f);
     store_chan<V>(dx + (long long)i * V, r);
 }
 
@@ -1488,17 +1586,84 @@ cdf_nn_status cdf_nn_head_fwd(const void *x, const float *w, const float *b, flo
     return launched();
 }
 
-cdf_nn_status cdf_nn_head_bwd(const void *x, const float *w, const float *dout, void *dx, float *dw, float *db,
-                              long long P, int C, int O, void *stream) {
+static cdf_nn_status head_bwd(const void *x, const float *w, const float *dout, void *dx, float *dw, float *db,
+                              long long P, int C, int O, bool relu, void *stream) {
     if (!x || !w || !dout || !dx || !dw || !db) return nn_fail("head_bwd: NULL argument");
     auto s = static_cast<cudaStream_t>(stream);
-    with_width(by_eight({C}, {dx}), P * C, [&](auto v, auto index) {
+    const auto *xb = static_cast<const __nv_bfloat16 *>(x);
+    with_width(by_eight({C}, {dx, x}), P * C, [&](auto v, auto index) {
         constexpr int V = decltype(v)::value;
         head_bwd_data_kernel<V, decltype(index)><<<blocks_for(P * C / V), 256, 0, s>>>(
-            dout, w, static_cast<__nv_bfloat16 *>(dx), P, C, O);
+            dout, w, relu ? xb : nullptr, static_cast<__nv_bfloat16 *>(dx), P, C, O);
     });
-    head_bwd_weight_kernel<<<blocks_for(P, 8 * kHeadRun), 256, 0, s>>>(static_cast<const __nv_bfloat16 *>(x), dout, dw,
-                                                                       db, P, C, O);
+    head_bwd_weight_kernel<<<blocks_for(P, 8 * kHeadRun), 256, 0, s>>>(xb, dout, dw, db, P, C, O);
+    return launched();
+}
+
+cdf_nn_status cdf_nn_head_bwd(const void *x, const float *w, const float *dout, void *dx, float *dw, float *db,
+                              long long P, int C, int O, void *stream) {
+    return head_bwd(x, w, dout, dx, dw, db, P, C, O, false, stream);
+}
+
+cdf_nn_status cdf_nn_head_bwd_relu(const void *x, const float *w, const float *dout, void *dx, float *dw, float *db,
+                                   long long P, int C, int O, void *stream) {
+    return head_bwd(x, w, dout, dx, dw, db, P, C, O, true, stream);
+}
+
+cdf_nn_status cdf_nn_conv3x3_bwd_data_relu(const void *dy, const void *w, const void *y, void *dx, int N, int H, int W,
+                                           int Cin, int Cout, void *stream) {
+    if (!dy || !w || !y || !dx || N < 1 || H < 1 || W < 1 || Cin % 16 || Cout % 32)
+        return nn_fail("conv3x3_bwd_data_relu: bad arguments (Cin % 16, Cout % 32)");
+    const auto s = static_cast<cudaStream_t>(stream);
+    if ((g_path == 1 || g_path == 4) && !(reinterpret_cast<uintptr_t>(y) & 15)) {
+        bool ran = false;
+        const cudaError_t e = conv_lin<true>(static_cast<const __nv_bfloat16 *>(dy), static_cast<const __nv_bfloat16 *>(w),
+                                             nullptr, static_cast<const __nv_bfloat16 *>(y),
+                                             static_cast<__nv_bfloat16 *>(dx), N, H, W, Cout, Cin, 0, s, &ran);
+        if (e != cudaSuccess) { cudaGetLastError(); return nn_fail(cudaGetErrorString(e)); }
+        if (ran) return launched();
+    }
+    const cdf_nn_status st = cdf_nn_conv3x3_bwd_data(dy, w, dx, N, H, W, Cin, Cout, stream);
+    return st != CDF_NN_OK ? st : cdf_nn_relu_bwd(dx, y, (long long)N * H * W * Cin, stream);
+}
+
+cdf_nn_status cdf_nn_upsample2_concat(const void *x, const void *skip, void *y, int N, int H, int W, int C, int Cs,
+                                      void *stream) {
+    if (!x || !skip || !y || N < 1 || H < 1 || W < 1 || C < 1 || Cs < 1) return nn_fail("upsample2_concat: bad arguments");
+    const long long n = (long long)N * H * W * (C + 4ll * Cs);
+    with_width(by_eight({C, Cs}, {x, skip, y}), 4 * n, [&](auto v, auto index) {
+        constexpr int V = decltype(v)::value;
+        upsample2_concat_kernel<V, decltype(index)><<<blocks_for(n / V), 256, 0, static_cast<cudaStream_t>(stream)>>>(
+            static_cast<const __nv_bfloat16 *>(x), static_cast<const __nv_bfloat16 *>(skip),
+            static_cast<__nv_bfloat16 *>(y), N, H, W, C, Cs);
+    });
+    return launched();
+}
+
+cdf_nn_status cdf_nn_upsample2_bwd_relu(const void *dy, const void *y, void *dx, int N, int H, int W, int C, int Cy,
+                                        void *stream) {
+    if (!dy || !y || !dx || N < 1 || H < 1 || W < 1 || C < 1 || C > Cy) return nn_fail("upsample2_bwd_relu: bad arguments");
+    const long long n = (long long)N * H * W * C;
+    with_width(by_eight({C, Cy}, {dy, y, dx}), n, [&](auto v, auto index) {
+        constexpr int V = decltype(v)::value;
+        upsample2_bwd_relu_kernel<V, decltype(index)><<<blocks_for(n / V), 256, 0, static_cast<cudaStream_t>(stream)>>>(
+            static_cast<const __nv_bfloat16 *>(dy), static_cast<const __nv_bfloat16 *>(y),
+            static_cast<__nv_bfloat16 *>(dx), N, H, W, C, Cy);
+    });
+    return launched();
+}
+
+cdf_nn_status cdf_nn_pool_skip_bwd_relu(const void *dp, const void *dcat, const void *y, void *dx, int N, int H, int W,
+                                        int C, int Cy, int coff, void *stream) {
+    if (!dp || !dcat || !y || !dx || N < 1 || H < 2 || W < 2 || H % 2 || W % 2 || C < 1 || coff < 0 || coff + C > Cy)
+        return nn_fail("pool_skip_bwd_relu: bad arguments (H and W even, coff + C <= Cy)");
+    const long long n = (long long)N * (H / 2) * (W / 2) * C;
+    with_width(by_eight({C, Cy, coff}, {dp, dcat, y, dx}), 4 * n, [&](auto v, auto index) {
+        constexpr int V = decltype(v)::value;
+        pool_skip_bwd_relu_kernel<V, decltype(index)><<<blocks_for(n / V), 256, 0, static_cast<cudaStream_t>(stream)>>>(
+            static_cast<const __nv_bfloat16 *>(dp), static_cast<const __nv_bfloat16 *>(dcat),
+            static_cast<const __nv_bfloat16 *>(y), static_cast<__nv_bfloat16 *>(dx), N, H, W, C, Cy, coff);
+    });
     return launched();
 }
 

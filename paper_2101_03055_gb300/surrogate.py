@@ -13,6 +13,7 @@ convergence as for a start from rest.
 from __future__ import annotations
 
 import ctypes
+import functools
 import math
 import os
 
@@ -34,6 +35,11 @@ NN_SIGNATURES = {
     "cdf_nn_copy_channels": [ctypes.c_void_p] * 2 + [ctypes.c_longlong] + [ctypes.c_int] * 6 + [ctypes.c_void_p],
     "cdf_nn_head_fwd": [ctypes.c_void_p] * 4 + [ctypes.c_longlong, ctypes.c_int, ctypes.c_int, ctypes.c_void_p],
     "cdf_nn_head_bwd": [ctypes.c_void_p] * 6 + [ctypes.c_longlong, ctypes.c_int, ctypes.c_int, ctypes.c_void_p],
+    "cdf_nn_conv3x3_bwd_data_relu": [ctypes.c_void_p] * 4 + [ctypes.c_int] * 5 + [ctypes.c_void_p],
+    "cdf_nn_upsample2_concat": [ctypes.c_void_p] * 3 + [ctypes.c_int] * 5 + [ctypes.c_void_p],
+    "cdf_nn_upsample2_bwd_relu": [ctypes.c_void_p] * 3 + [ctypes.c_int] * 5 + [ctypes.c_void_p],
+    "cdf_nn_pool_skip_bwd_relu": [ctypes.c_void_p] * 4 + [ctypes.c_int] * 6 + [ctypes.c_void_p],
+    "cdf_nn_head_bwd_relu": [ctypes.c_void_p] * 6 + [ctypes.c_longlong, ctypes.c_int, ctypes.c_int, ctypes.c_void_p],
     "cdf_nn_mse": [ctypes.c_void_p] * 4 + [ctypes.c_longlong, ctypes.c_void_p],
     "cdf_nn_adam": [ctypes.c_void_p] * 5 + [ctypes.c_longlong] + [ctypes.c_float] * 4 + [ctypes.c_longlong,
                                                                                          ctypes.c_void_p],
@@ -74,18 +80,20 @@ def tensor_error_flag() -> int:
 
 
 def _call(name, *args):
-    st = getattr(nn_lib(), name)(*args)
-    if st != 0:
+    if getattr(nn_lib(), name)(*args) != 0:
         raise RuntimeError(f"{name}: {nn_lib().cdf_nn_last_error().decode()}")
 
 
+# Pointers and streams go to ctypes as plain integers (the signatures make them void *), and
+# the current stream's handle comes without a Stream object: a pass of the U-Net is about
+# sixty such calls, and 12 us each for the object alone kept the GPU waiting.
 def _p(t):
-    return ctypes.c_void_p(t.data_ptr()) if t is not None else None
+    return t.data_ptr() if t is not None else None
 
 
 def _stream():
     import torch
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream or None)
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()) or None
 
 
 # ---- thin same-name wrappers of include/cdf_nn.h ----------------------------------------
@@ -93,7 +101,7 @@ def conv3x3_fwd(x, w, b, relu):
     import torch
     N, H, W, Cin = x.shape
     Cout = w.shape[0]
-    y = torch.empty((N, H, W, Cout), dtype=torch.bfloat16, device=x.device)
+    y = x.new_empty((N, H, W, Cout), dtype=torch.bfloat16)
     _call("cdf_nn_conv3x3_fwd", _p(x), _p(w), _p(b), _p(y), N, H, W, Cin, Cout, int(relu), _stream())
     return y
 
@@ -106,7 +114,21 @@ def conv3x3_bwd_data(dy, w, Cin):
     return dx
 
 
+def conv3x3_bwd_data_relu(dy, w, y):
+    """conv3x3_bwd_data, zero where the layer's input y (a ReLU output) is not positive."""
+    import torch
+    N, H, W, Cout = dy.shape
+    dx = torch.empty_like(y)
+    _call("cdf_nn_conv3x3_bwd_data_relu", _p(dy), _p(w), _p(y), _p(dx), N, H, W, y.shape[3], Cout, _stream())
+    return dx
+
+
 _workspace = {}
+
+
+@functools.lru_cache(maxsize=None)
+def _weight_workspace(N, H, W, Cin, Cout):
+    return int(nn_lib().cdf_nn_conv3x3_bwd_weight_workspace(N, H, W, Cin, Cout))
 
 
 def conv3x3_bwd_weight(x, dy, dw, db):
@@ -115,7 +137,7 @@ def conv3x3_bwd_weight(x, dy, dw, db):
     import torch
     N, H, W, Cin = x.shape
     Cout = dy.shape[3]
-    need = int(nn_lib().cdf_nn_conv3x3_bwd_weight_workspace(N, H, W, Cin, Cout))
+    need = _weight_workspace(N, H, W, Cin, Cout)
     ws = _workspace.get(x.device)
     if ws is None or ws.numel() * 4 < need:
         ws = torch.empty((max(need, 4) + 3) // 4, dtype=torch.float32, device=x.device)
@@ -157,6 +179,34 @@ def upsample2_bwd_from(dy, C, coff):
     return dx
 
 
+def upsample2_concat(x, skip):
+    """x upsampled 2x (nearest) with skip behind it in the channels."""
+    N, H, W, C = x.shape
+    Cs = skip.shape[3]
+    y = x.new_empty((N, 2 * H, 2 * W, C + Cs))
+    _call("cdf_nn_upsample2_concat", _p(x), _p(skip), _p(y), N, H, W, C, Cs, _stream())
+    return y
+
+
+def upsample2_bwd_relu(dcat, y):
+    """Gradient of y (a ReLU output), upsampled into the first channels of a concatenation."""
+    import torch
+    N, H, W, C = y.shape
+    dx = torch.empty_like(y)
+    _call("cdf_nn_upsample2_bwd_relu", _p(dcat), _p(y), _p(dx), N, H, W, C, dcat.shape[3], _stream())
+    return dx
+
+
+def pool_skip_bwd_relu(dpool, dcat, y):
+    """Gradient of y (a ReLU output) that was pooled and concatenated (its channels are dcat's last)."""
+    import torch
+    N, H, W, C = y.shape
+    dx = torch.empty_like(y)
+    _call("cdf_nn_pool_skip_bwd_relu", _p(dpool), _p(dcat), _p(y), _p(dx), N, H, W, C, dcat.shape[3],
+          dcat.shape[3] - C, _stream())
+    return dx
+
+
 def copy_channels(x, y, src_off, dst_off, count, accumulate=False):
     P = x.numel() // x.shape[-1]
     _call("cdf_nn_copy_channels", _p(x), _p(y), P, x.shape[-1], y.shape[-1], src_off, dst_off, count,
@@ -178,6 +228,15 @@ def head_bwd(x, w, dout, dw, db):
     O = w.shape[0]
     dx = torch.empty((N, H, W, C), dtype=torch.bfloat16, device=x.device)
     _call("cdf_nn_head_bwd", _p(x), _p(w), _p(dout), _p(dx), _p(dw), _p(db), N * H * W, C, O, _stream())
+    return dx
+
+
+def head_bwd_relu(x, w, dout, dw, db):
+    """head_bwd with dx zero where the head's input x (a ReLU output) is not positive."""
+    import torch
+    N, H, W, C = x.shape
+    dx = torch.empty_like(x)
+    _call("cdf_nn_head_bwd_relu", _p(x), _p(w), _p(dout), _p(dx), _p(dw), _p(db), N * H * W, C, w.shape[0], _stream())
     return dx
 
 
@@ -247,12 +306,8 @@ class UNet:
             acts[f"e{L}a"], acts[f"e{L}b"] = h1, h2
             skips.append(h2)
             h = h2
-        import torch
         for L in range(self.levels - 2, -1, -1):
-            N, Hh, Ww, C = h.shape
-            cat = torch.empty((N, 2 * Hh, 2 * Ww, C + self.ch[L]), dtype=torch.bfloat16, device=h.device)
-            upsample2_into(h, cat, 0)
-            copy_channels(skips[L], cat, 0, C, self.ch[L])
+            cat = upsample2_concat(h, skips[L])
             acts[f"d{L}.cat"] = cat
             h1 = conv3x3_fwd(cat, self.bf16[f"d{L}a.w"], self.master[f"d{L}a.b"], True)
             h2 = conv3x3_fwd(h1, self.bf16[f"d{L}b.w"], self.master[f"d{L}b.b"], True)
@@ -261,37 +316,36 @@ class UNet:
         acts["head.in"] = h
         return head_fwd(h, self.master["head.w"], self.master["head.b"]), acts
 
-    def backward(self, acts, dout):
+    def _zero_grads(self):
+        """FP32 zeros for every parameter: views of one buffer, each on 16 bytes."""
         import torch
-        grads = {k: torch.zeros_like(t) for k, t in self.master.items()}
-        dh = head_bwd(acts["head.in"], self.master["head.w"], dout, grads["head.w"], grads["head.b"])
-        dskip = [None] * self.levels
+        sizes = [-(-t.numel() // 4) * 4 for t in self.master.values()]
+        flat = torch.zeros(sum(sizes), dtype=torch.float32, device=self.master["head.b"].device)
+        return {k: part[:t.numel()].view(t.shape)
+                for (k, t), part in zip(self.master.items(), flat.split(sizes))}
+
+    def backward(self, acts, dout):
+        grads = self._zero_grads()
+        # dh: gradient of a block's output before its ReLU; dcat[L]: of the concatenation at level L
+        dh = head_bwd_relu(acts["head.in"], self.master["head.w"], dout, grads["head.w"], grads["head.b"])
+        dcat = [None] * self.levels
         for L in range(0, self.levels - 1):
-            dh, dskip[L] = self._block_bwd(f"d{L}", acts[f"d{L}.cat"], acts, dh, grads, split=self.ch[L])
+            dcat[L] = self._block_bwd(f"d{L}", acts[f"d{L}.cat"], acts, dh, grads)
+            below = f"d{L + 1}b" if L + 2 < self.levels else f"e{L + 1}b"
+            dh = upsample2_bwd_relu(dcat[L], acts[below])
         for L in range(self.levels - 1, -1, -1):
-            if dskip[L] is not None:
-                copy_channels(dskip[L], dh, 0, 0, self.ch[L], accumulate=True)
-            dx, _ = self._block_bwd(f"e{L}", acts[f"e{L}.in"], acts, dh, grads, split=None)
+            dx = self._block_bwd(f"e{L}", acts[f"e{L}.in"], acts, dh, grads, need_dx=L > 0)
             if L > 0:
-                N, H, W, C = acts[f"e{L - 1}b"].shape
-                dh = avgpool2_bwd(dx, H, W)
+                dh = pool_skip_bwd_relu(dx, dcat[L - 1], acts[f"e{L - 1}b"])
         return grads
 
-    def _block_bwd(self, name, x_in, acts, dh, grads, split):
-        # second conv
-        relu_bwd(dh, acts[f"{name}b"])
-        conv3x3_bwd_weight(acts[f"{name}a"], dh, grads[f"{name}b.w"], grads[f"{name}b.b"])
-        d1 = conv3x3_bwd_data(dh, self.bf16[f"{name}b.w"], acts[f"{name}a"].shape[3])
-        relu_bwd(d1, acts[f"{name}a"])
+    def _block_bwd(self, name, x_in, acts, dh, grads, need_dx=True):
+        """Weight gradients of a block's two convolutions and, if asked for, its input's gradient."""
+        mid = acts[f"{name}a"]
+        conv3x3_bwd_weight(mid, dh, grads[f"{name}b.w"], grads[f"{name}b.b"])
+        d1 = conv3x3_bwd_data_relu(dh, self.bf16[f"{name}b.w"], mid)
         conv3x3_bwd_weight(x_in, d1, grads[f"{name}a.w"], grads[f"{name}a.b"])
-        dx = conv3x3_bwd_data(d1, self.bf16[f"{name}a.w"], x_in.shape[3])
-        if split is None:
-            return dx, None
-        cup = x_in.shape[3] - split
-        import torch
-        dskip = torch.empty((*dx.shape[:3], split), dtype=torch.bfloat16, device=dx.device)
-        copy_channels(dx, dskip, cup, 0, split)
-        return upsample2_bwd_from(dx, cup, 0), dskip
+        return conv3x3_bwd_data(d1, self.bf16[f"{name}a.w"], x_in.shape[3]) if need_dx else None
 
     def adam_step(self, grads, lr):
         self.step_count += 1
