@@ -513,6 +513,28 @@ __device__ __forceinline__ void bias_partial(const __nv_bfloat16 *__restrict__ d
         g.bpart[(long long)split * g.Cout + gb * g.gw * 8 + i] = red[(i & 7) * 256 + (i >> 3)];
 }
 
+// One warp copies positions q .. q + n - 1 (n <= 32) with G channel groups from src, whose
+// pixels are `stride` channels apart, to dst[(group sp + position) 16 bytes], channel group fastest:
+// lane l finds the pixel of position l once, the copies get it by shuffle; positions from `valid`
+// on are zeros.  (For the stages of a weight gradient, each a few copies per thread: 192 -> 64
+// channels at 32 x 32 x 32 44 -> 39 us.  The slabs of conv3x3_lin_kernel, many copies per
+// thread, are faster with the pixel found for every copy and 256 threads abreast: 53 against 63 us
+// at 16 x 256 x 256, 32 -> 32; plain loads and stores instead of cp.async 62-67 us.)
+__device__ __forceinline__ void stage_run(const LinImage &im, int q, int n, int lane,
+                                          const __nv_bfloat16 *__restrict__ src, int stride, int G, FastDiv dg,
+                                          unsigned char *dst, int sp, int valid = 32) {
+    const int mine = lane < min(n, valid) ? lin_pixel(im, q + lane) : -1;
+    const int total = n * G;
+#pragma unroll 4
+    for (int base = 0; base < total; base += 32) {
+        const int e = base + lane, pos = div_by(e, dg), grp = e - pos * G;
+        const int px = __shfl_sync(0xffffffffu, mine, pos & 31);
+        if (e < total)
+            cp_async16(dst + (grp * sp + pos) * 16, px >= 0 ? src + (long long)px * stride + grp * 8 : src,
+                       px >= 0 ? 16 : 0);
+    }
+}
+
 template <int BN, bool kFirst>
 __device__ __forceinline__ void wgrad_slices(uint32_t tmem, uint64_t ad, uint64_t bd, uint32_t idesc, uint32_t lead) {
 #pragma unroll
@@ -580,21 +602,12 @@ __global__ void __launch_bounds__(kWgThreads) conv3x3_wgrad_lin_kernel(const __n
             if (!ok) break;
             unsigned char *Y = wg_smem + (s % kWgStages) * (ybytes + xbytes), *X = Y + ybytes;
             const int q = qbeg + s * kWgK;
-#pragma unroll 4
-            for (int e = tid; e < kWgK * Gy; e += kWgStagers) {
-                const int pos = div_by(e, g.dgy), grp = e - pos * Gy;
-                const int px = q + pos < qend ? lin_pixel(g.im, q + pos) : -1;
-                cp_async16(Y + (grp * g.spy + pos) * 16, px >= 0 ? dy + (long long)px * g.Cout + co0 + grp * 8 : dy,
-                           px >= 0 ? 16 : 0);
-            }
-            const int qx = q + (ky - 1) * g.im.Wp - 1;  // X from one position before to one after, row ky
-#pragma unroll 3
-            for (int e = tid; e < (kWgK + 2) * Gx; e += kWgStagers) {
-                const int pos = div_by(e, g.dgx), grp = e - pos * Gx;
-                const int px = lin_pixel(g.im, qx + pos);
-                cp_async16(X + (grp * g.spx + pos) * 16, px >= 0 ? x + (long long)px * g.Cin + ci0 + grp * 8 : x,
-                           px >= 0 ? 16 : 0);
-            }
+            // each warp an eighth of the positions: 8 of dY, 9 (the last one fewer) of X, which run from one
+            // position before the stage's to one after, in row ky
+            const int qy = q + 8 * warp, ny = max(0, min(8, qend - qy));
+            stage_run(g.im, qy, 8, lane, dy + co0, g.Cout, Gy, g.dgy, Y + 8 * warp * 16, g.spy, ny);
+            stage_run(g.im, q + (ky - 1) * g.im.Wp - 1 + 9 * warp, min(9, kWgK + 2 - 9 * warp), lane, x + ci0, g.Cin, Gx,
+                      g.dgx, X + 9 * warp * 16, g.spx, 9);
             cp_async_commit();
             if (s >= kWgLag) {
                 cp_async_wait<kWgLag>();
