@@ -136,20 +136,27 @@ struct BatchInst {
     long long node_off;  // nodes of the instances before it
     int tile_base;       // first tile and tiles per row, persistent kernel
     int tiles_x;
-    int pair_base;       // the same for the two-step launches, tiles of tw x th
+    int pair_tiles;      // the same for the two-step launches: tiles of tw x th
     int pair_x;
     int tw, th;
     unsigned inv_w1, inv_tw;  // ceil(2^20 / (tw + 2)), ceil(2^20 / tw)
 };
-// Nodes of a tile and the ring around it that step2_batch_kernel holds in shared memory: 51 KB
-// for two scalars, four CTAs of 256 threads an SM.
-constexpr int kBatchRegion = 640;
+// The instances of one two-step launch, as a kernel parameter (at most 32,764 bytes in all).
+constexpr int kBatchGroup = 64;
+struct BatchPack {
+    BatchInst inst[kBatchGroup];
+};
+static_assert(sizeof(BatchPack) <= 32000, "a kernel's parameters");
+// The largest tile of step2_batch_kernel, 32 x 16 nodes, and the pitch of a row of it with its ring: 49 KB
+// of shared memory for two scalars with consumption, four CTAs on an SM.
+constexpr int kBatchTileX = 32, kBatchTileY = 16, kBatchPitch = kBatchTileX + 2;
 // The closure kind (lb_device.cuh) that can run all `count` lattices.
 int batch_closure_kind(const LbParams *p, int count);
-// Two steps of every instance in one launch of `tiles` CTAs; tile_inst names each tile's
-// instance.  On a periodic axis the lattice must be at least tw + 2 (th + 2) nodes long.
-cudaError_t launch_step2_batch(int m, int kind, const BatchInst *inst, const int *tile_inst, int tiles, const float *in,
-                               float *out, const float *sp_in, float *sp_out, float *moments, cudaStream_t s);
+// Two steps of `count` <= kBatchGroup instances (host copies).  On a periodic axis a lattice must
+// be at least tw + 2 (th + 2) nodes long, and an instance's planes together hold fewer than
+// 2^31 values.
+cudaError_t launch_step2_batch(int m, int kind, const BatchInst *inst, int count, const float *in, float *out,
+                               const float *sp_in, float *sp_out, float *moments, cudaStream_t s);
 // Initialisation from, and packing into, the dense moment stacks of all instances back to back
 // (count <= 65535 instances of at most max_nodes nodes).
 cudaError_t launch_init_batch(int m, const BatchInst *inst, int count, long long max_nodes, const float *fields,

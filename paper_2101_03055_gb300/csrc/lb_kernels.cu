@@ -15,7 +15,9 @@
 // addresses, and the overlap between neighbouring warps is served from L1/L2.
 #include "lb_device.cuh"
 
+#include <algorithm>
 #include <atomic>
+#include <cstring>
 #include <type_traits>
 
 namespace cdflb {
@@ -27,7 +29,7 @@ using namespace dev;
 // finishes, and waits inside for that kernel's results.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl_smem(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                            Args... args) {
+                            const Args &...args) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = block;
@@ -355,45 +357,99 @@ __global__ void __launch_bounds__(FW ? FW * FY : step2_max_threads(M), FW ? step
     }
 }
 
-// The same for all instances of a batch in one launch: CTA b works on tile b of the
-// batch (instance tile_inst[b]); the instance's parameters are staged in shared
-// memory.  Every instance has output tiles of its own size tw x th, as even a division
+// The same for up to kBatchGroup instances of a batch in one launch: CTA (t, k) works on tile
+// t of instance k of `pack`, whose parameters lie in the constant bank.
+// Every instance has output tiles of its own size tw x th, as even a division
 // of its lattice as fits (pair_tile in lb_batch.cu): a 64 x 64 lattice is eight tiles of
 // 32 x 16, where 30 x 14 tiles would be fifteen, 65 % full.  So the nodes of R1 and of the
-// tile are walked in row order, 256 at a time, whatever the width; the shared-memory
-// plane stride is the constant kBatchRegion.  512 cavities of 64 x 64, 64 steps with
-// initialisation and moments: 8.7 ms on the persistent kernel, 4.3 with tiles of 30 x 14 for
-// all, 3.9 now (118 us a launch).  On larger lattices the chains of step2_kernel per instance,
-// which read the parameters as constant operands, stay ahead (64 plumes of 128-512 x 64-256);
-// the autotuner times both.  Bound by instruction issue (563 a warp update with walls in
-// nearly every warp, issue active 56 %).
-// q / d for 0 <= q < 1024, 3 <= d <= 1024, with inv = ceil(2^20 / d).
-__device__ __forceinline__ int small_div(int q, unsigned inv) { return (int)(((unsigned)q * inv) >> 20); }
+// tile are walked as lists (NodeWalk), whatever the width; the row pitch and the plane
+// stride in shared memory are constants.
+// Bound by instruction issue and the latency of a CTA's few rounds (issue active 63 %, four
+// CTAs of 256 threads an SM).  512 cavities of 64 x 64, 64 steps with initialisation and moments: 8.7 ms
+// on the persistent kernel; 3.9 with the parameters staged in shared memory, a
+// runtime pitch and a row-order walk; 3.2 with the parameters in the constant bank (no
+// spills, uniform operands) and constant strides; 2.7 with the inner nodes first; 2.5 with
+// the groups of lattices that run side by side held in L2 (lb_batch.cu).  Chains of step2_kernel per
+// instance: 72.5 us a step for these against 36.9, and 67.6 against 65.8 for 64 plumes of 128-512 x
+// 64-256, but 6.5 against 7.8 for 8 lattices of 300 x 200; the autotuner times both.
+// A rectangle [xa, xb) x [ya, yb) of nodes walked by a CTA, 32 a round: first its part away from
+// the lattice's edges, in row order, then the strips along the edges (at most two nodes wide,
+// left, right, lower, upper), so that a round runs either the pull without boundary
+// rules or the one with them as a whole.  On a 64 x 64 lattice a row-order walk has a node at
+// an edge in nearly every round (22 % fewer instructions with this one).
+struct NodeWalk {
+    int xa, xb, ya, yb;      // all nodes
+    int ixa, ixb, iya, iyb;  // the inner ones (empty: ixa = ixb, iya = iyb)
+    int inner, edge, inner_rounds, rounds;
+    unsigned inv;            // ceil(2^20 / (ixb - ixa))
+    __device__ __forceinline__ NodeWalk(int xa_, int xb_, int ya_, int yb_, int nx, int ny)
+        : xa(xa_), xb(xb_), ya(ya_), yb(yb_) {
+        ixa = max(xa, 1);
+        ixb = min(xb, nx - 1);
+        iya = max(ya, 1);
+        iyb = min(yb, ny - 1);
+        if (ixa >= ixb || iya >= iyb) {
+            ixa = ixb = xb;  // everything is the left strip
+            iya = iyb = yb;
+        }
+        const int w = ixb - ixa;
+        inner = w * (iyb - iya);
+        edge = (xb - xa) * (yb - ya) - inner;
+        inner_rounds = (inner + 31) >> 5;
+        rounds = inner_rounds + ((edge + 31) >> 5);
+        inv = w > 0 ? ((1u << 20) + w - 1) / w : 0u;
+    }
+    // Node `lane` of round r; false: none.
+    __device__ __forceinline__ bool node(int r, int lane, int &x, int &y) const {
+        if (r < inner_rounds) {
+            const int q = r * 32 + lane, row = (int)(((unsigned)q * inv) >> 20);  // q < 1024
+            x = ixa + q - row * (ixb - ixa);
+            y = iya + row;
+            return q < inner;
+        }
+        int q = (r - inner_rounds) * 32 + lane;
+        if (q >= edge) return false;
+        const int h = yb - ya, wl = ixa - xa, wr = xb - ixb, w = ixb - ixa;
+        if (q < wl * h) {  // (wl is at most 2 where there are inner nodes)
+            const int row = q / wl;
+            x = xa + q - row * wl;
+            y = ya + row;
+            return true;
+        }
+        q -= wl * h;
+        if (q < wr * h) {
+            const int row = wr == 1 ? q : q / wr;
+            x = ixb + q - row * wr;
+            y = ya + row;
+            return true;
+        }
+        q -= wr * h;
+        const int low = (iya - ya) * w, row = q < low ? q / w : (q - low) / w;
+        x = ixa + (q < low ? q : q - low) - row * w;
+        y = (q < low ? ya : iyb) + row;
+        return true;
+    }
+};
 
 template <int M, int K>
 __global__ void __launch_bounds__(256, step2_max_threads(M) / 256)
-    step2_batch_kernel(const BatchInst *__restrict__ inst, const int *__restrict__ tile_inst, const float *in,
-                       float *out, const float *sp_in, float *sp_out, float *moments) {
-    constexpr int NP = 9 + 5 * M, SP = kBatchRegion;
+    step2_batch_kernel(const __grid_constant__ BatchPack pack, const float *in, float *out, const float *sp_in,
+                       float *sp_out, float *moments) {
+    constexpr int NP = 9 + 5 * M, SP = kBatchPitch * (kBatchTileY + 2), PT = kBatchPitch;
     extern __shared__ float sm[];
-    __shared__ BatchInst me;
-    const int tid = threadIdx.x, lane = tid & 31, warp0 = tid - lane;
-    {
-        // (the tables do not change: read before the wait for the previous launch)
-        const int *const src = reinterpret_cast<const int *>(inst + __ldg(tile_inst + blockIdx.x));
-        for (int w = tid; w < (int)(sizeof(BatchInst) / sizeof(int)); w += 256)
-            reinterpret_cast<int *>(&me)[w] = __ldg(src + w);
-    }
-    __syncthreads();
+    const BatchInst &me = pack.inst[blockIdx.y];
+    const int lt = blockIdx.x;
     pdl_wait_and_release();
+    if (lt >= me.pair_tiles) return;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const LbParams &p = me.p;
     const int TW = me.tw, TH = me.th, W1 = TW + 2, H1 = TH + 2;
-    const int lt = blockIdx.x - me.pair_base, ty = lt / me.pair_x;
+    const int ty = lt / me.pair_x;
     const int X0 = (lt - ty * me.pair_x) * TW, Y0 = ty * TH;
     const float *const i0 = in + me.pop_off;
     float *const out0 = out + me.pop_off;
-    const long long P = p.plane;
-    const int pitch = p.pitch, nx = p.nx, ny = p.ny;
+    // element offsets within an instance's planes fit in 32 bits (checked by fused_fits)
+    const int P = (int)p.plane, pitch = p.pitch, nx = p.nx, ny = p.ny;
     const int xend = min(X0 + TW, nx), yend = min(Y0 + TH, ny);
     const bool consume = M >= 2 && closure_has<K>(kConsume, p.skind == 2);
     const float *const s_in = sp_in + me.sp_off;
@@ -402,25 +458,19 @@ __global__ void __launch_bounds__(256, step2_max_threads(M) / 256)
     // ---- step 1: R1 from global memory into shared memory
     {
         const auto mk = [pitch](int sx, int sy) { return sy * pitch + sx; };
-        const auto ld = [i0, &p, P](int plane, int off) { return __ldg(i0 + plane * P + CDF_CHK(p, off, P, 1)); };
-        const unsigned inv = me.inv_w1;
-        for (int base = warp0; base < W1 * H1; base += 256) {
-            const int l = base + lane, ly = small_div(l, inv), lx = l - ly * W1;
-            const int xu = X0 - 1 + lx, yu = Y0 - 1 + ly;
-            const bool ok = l < W1 * H1 && xu <= xend && yu <= yend && (p.periodic_x || (xu >= 0 && xu < nx)) &&
-                            (p.periodic_y || (yu >= 0 && yu < ny));
+        const auto ld = [i0, &p, P](int plane, int off) { return __ldg(i0 + (size_t)(plane * P) + CDF_CHK(p, off, P, 1)); };
+        const NodeWalk walk(p.periodic_x ? X0 - 1 : max(X0 - 1, 0), p.periodic_x ? xend + 1 : min(xend + 1, nx),
+                            p.periodic_y ? Y0 - 1 : max(Y0 - 1, 0), p.periodic_y ? yend + 1 : min(yend + 1, ny), nx, ny);
+        for (int r = warp; r < walk.rounds; r += 8) {
+            int xu, yu;
+            if (!walk.node(r, lane, xu, yu)) continue;
             const int gx = xu < 0 ? xu + nx : (xu >= nx ? xu - nx : xu);
             const int gy = yu < 0 ? yu + ny : (yu >= ny ? yu - ny : yu);
-            const bool general = ok && !inner_node(p, gx, gy);
             float h[9], f[M][5];
-            if (!__any_sync(0xffffffffu, general)) {
-                if (!ok) continue;
-                pull_node<M, true, K>(p, gx, gy, mk, ld, f, h);
-            } else {
-                if (!ok) continue;
-                pull_node<M, false, K>(p, gx, gy, mk, ld, f, h);
-            }
-            const int o0 = CDF_CHK(p, gy * pitch + gx, P, 2), l0 = CDF_CHK(p, l, SP, 3);
+            if (r < walk.inner_rounds) pull_node<M, true, K>(p, gx, gy, mk, ld, f, h);
+            else pull_node<M, false, K>(p, gx, gy, mk, ld, f, h);
+            const int o0 = CDF_CHK(p, gy * pitch + gx, P, 2);
+            const int l0 = CDF_CHK(p, (yu - Y0 + 1) * PT + (xu - X0 + 1), SP, 3);
             NodeOut<M> o;
             collide<M, K>(p, f, h, node_pref<K>(p, gx, gy), consume ? s_in[o0] : 0.f, false, o);
 #pragma unroll
@@ -436,37 +486,31 @@ __global__ void __launch_bounds__(256, step2_max_threads(M) / 256)
 
     // ---- step 2: the tile from shared memory into global memory
     const auto lds = [&p](int plane, int off) { return sm[plane * SP + CDF_CHK(p, off, SP, 4)]; };
-    const auto mk_in = [W1, X0, Y0](int sx, int sy) { return (sy - Y0 + 1) * W1 + (sx - X0 + 1); };
+    const auto mk_in = [X0, Y0](int sx, int sy) { return (sy - Y0 + 1) * PT + (sx - X0 + 1); };
     const auto mk_gen = [W1, H1, X0, Y0, nx, ny](int sx, int sy) {
         int a = sx - X0 + 1, b = sy - Y0 + 1;
         a = a < 0 ? a + nx : (a >= W1 ? a - nx : a);
         b = b < 0 ? b + ny : (b >= H1 ? b - ny : b);
-        return b * W1 + a;
+        return b * PT + a;
     };
     float *const mom = moments ? moments + me.mom_off : nullptr;
-    const unsigned inv = me.inv_tw;
-    for (int base = warp0; base < TW * TH; base += 256) {
-        const int q = base + lane, oy = small_div(q, inv), x = X0 + q - oy * TW, y = Y0 + oy;
-        const bool ok = q < TW * TH && x < nx && y < ny;
-        const bool general = ok && !inner_node(p, x, y);
+    const NodeWalk walk(X0, xend, Y0, yend, nx, ny);
+    for (int r = warp; r < walk.rounds; r += 8) {
+        int x, y;
+        if (!walk.node(r, lane, x, y)) continue;
         float h[9], f[M][5];
-        if (!__any_sync(0xffffffffu, general)) {
-            if (!ok) continue;
-            pull_node<M, true, K>(p, x, y, mk_in, lds, f, h);
-        } else {
-            if (!ok) continue;
-            pull_node<M, false, K>(p, x, y, mk_gen, lds, f, h);
-        }
+        if (r < walk.inner_rounds) pull_node<M, true, K>(p, x, y, mk_in, lds, f, h);
+        else pull_node<M, false, K>(p, x, y, mk_gen, lds, f, h);
         const int o0 = CDF_CHK(p, y * pitch + x, P, 2);
         NodeOut<M> o;
-        collide<M, K>(p, f, h, node_pref<K>(p, x, y),
-                      consume ? sm[NP * SP + CDF_CHK(p, (oy + 1) * W1 + x - X0 + 1, SP, 4)] : 0.f, false, o);
+        collide<M, K>(p, f, h, node_pref<K>(p, x, y), consume ? sm[NP * SP + CDF_CHK(p, mk_in(x, y), SP, 4)] : 0.f, false,
+                      o);
 #pragma unroll
-        for (int i = 0; i < 9; ++i) out0[i * P + o0] = h[i];
+        for (int i = 0; i < 9; ++i) out0[(size_t)(i * P) + o0] = h[i];
 #pragma unroll
         for (int a = 0; a < M; ++a)
 #pragma unroll
-            for (int i = 0; i < 5; ++i) out0[(9 + 5 * a + i) * P + o0] = f[a][i];
+            for (int i = 0; i < 5; ++i) out0[(size_t)((9 + 5 * a + i) * P) + o0] = f[a][i];
         if (consume) s_out[o0] = o.s1;
         if (mom) write_moments<M>(mom, P, o0, o);
     }
@@ -1419,13 +1463,18 @@ int batch_closure_kind(const LbParams *p, int count) {
     return kind;
 }
 
-cudaError_t launch_step2_batch(int m, int kind, const BatchInst *inst, const int *tile_inst, int tiles, const float *in,
-                               float *out, const float *sp_in, float *sp_out, float *moments, cudaStream_t s) {
-    const size_t smem = (size_t)(9 + 5 * m + 1) * kBatchRegion * sizeof(float);
+cudaError_t launch_step2_batch(int m, int kind, const BatchInst *inst, int count, const float *in, float *out,
+                               const float *sp_in, float *sp_out, float *moments, cudaStream_t s) {
+    if (count < 1 || count > kBatchGroup) return cudaErrorInvalidValue;
+    BatchPack pack;
+    std::memcpy(pack.inst, inst, count * sizeof(BatchInst));
+    int tiles = 0;
+    for (int k = 0; k < count; ++k) tiles = std::max(tiles, inst[k].pair_tiles);
+    const size_t smem = (size_t)(9 + 5 * m + 1) * kBatchPitch * (kBatchTileY + 2) * sizeof(float);
     const auto run = [&](auto *kern, SmemOptIn &opt_in) {
         const cudaError_t e = opt_in(kern, (int)smem);
         if (e != cudaSuccess) return e;
-        return launch_pdl_smem(kern, dim3(tiles), dim3(256), smem, s, inst, tile_inst, in, out, sp_in, sp_out, moments);
+        return launch_pdl_smem(kern, dim3(tiles, count), dim3(256), smem, s, pack, in, out, sp_in, sp_out, moments);
     };
     static SmemOptIn o1, o2[4], o3, o4;
     cudaError_t e = cudaErrorInvalidValue;

@@ -49,3 +49,10 @@ def test_small_walled_lattices(cdf):
 
 def test_short_periodic_axis_runs_on_the_persistent_kernel(cdf):
     check(cdf, [_rand_problem(nx, ny, 2, 8, "periodic", "noslip_noflux") for nx, ny in [(5, 20), (40, 12)]])
+
+
+def test_several_groups(cdf):
+    """More instances than one launch takes, enough nodes for the largest tiles, uneven groups."""
+    sizes = [(33, 17), (64, 64), (70, 50), (6, 90), (130, 40)]
+    check(cdf, [_rand_problem(*sizes[k % 5], 2, k, "mixed", "noslip_noflux") for k in range(70)], steps=(2, 33, 1))
+    check(cdf, [_rand_problem(16, 16, 1, k, "periodic", "mixed") for k in range(300)], steps=(34,))
