@@ -17,9 +17,9 @@
 //
 // Measured on GB300 (launches in a CUDA graph; before: the im2col kernels, forward rows of
 // whole 128-pixel tiles without im2col), forward / input gradient / weight and bias gradient:
-//   16 x 256 x 256, 32 -> 32     91 / 286 / 451 us before,  53 / 56 / 189 us now
-//   16 x 32 x 32, 256 -> 256    116 / 206 / 163 us before,  26 / 29 / 79 us now (740 TFLOP/s forward)
-//   the U-Net's first eleven layer shapes at 32 x 64 x 64, summed: 741 / 1050 / 1123 us before, 129 / 138 / 313 us now
+//   16 x 256 x 256, 32 -> 32     91 / 286 / 451 us before,  53 / 55 / 115 us now
+//   16 x 32 x 32, 256 -> 256    116 / 206 / 163 us before,  26 / 28 / 59 us now (750 TFLOP/s forward)
+//   the U-Net's first eleven layer shapes at 32 x 64 x 64, summed: 741 / 1050 / 1123 us before, 128 / 138 / 228 us now
 
 // Division of 0 <= x < 2^31 by a constant d >= 1: (umulhi(x, mul) + x) >> shift
 // (Granlund & Montgomery, PLDI 1994, the round-up multiplier of 33 bits).
@@ -448,31 +448,31 @@ __global__ void __launch_bounds__(kLinThreads) conv3x3_lin_kernel(const __grid_c
 
 // ---------------------------------------------------------------------------
 // Weight gradient dW[co][t][ci] = sum_q dY[q][co] X[q + shift(t)][ci] over the
-// padded positions (a padding position has dY = 0).  GEMM per tap: M = output
-// channels (tile 128), N = input channels (tile BN), K = positions.  Both operands
-// are staged as [channel group][position][16 bytes], which read with channels as
-// M / N and positions as K is the MN-major core-matrix layout: no transposition,
-// and the three taps of one row ky are the same staged X seen 16 bytes apart.  A
-// CTA owns the three taps of one ky (3 BN columns of TMEM), one channel tile of
-// each side and one contiguous run of positions; it writes its FP32 partial sums
-// to part[split][co][9 ci], the layout of dW, and weight_sum_kernel adds the splits
-// in a fixed order.  K runs in stages of 64 positions through a ring of four buffers
-// (two CTAs an SM, more with few channels): warps 0-7 stage by cp.async, two stages
-// behind the newest copies they announce the ones that landed; warp 8 issues the
-// twelve MMAs of a stage.  Bound: at 64 columns the MMA's reads of both operands
-// (48 cycles a slice, 32 of them arithmetic).  With one barrier of all threads a stage
-// and their waits for the MMAs in between, the same tiles took 113 us at 16 x 32 x 32,
-// 256 -> 256.
+// padded positions (a padding position has dY = 0).  GEMM: M = (row ky, input
+// channel of a tile of CI), 96 rows of 128 for CI = 32, N = output channels (tile BN),
+// K = positions.  Both operands are staged as [channel group][position][16 bytes], which
+// read with channels as M / N and positions as K is the MN-major core-matrix layout: no
+// transposition, and the three taps of a row are the same staged X seen 16 bytes apart:
+// three MMAs per 16 positions for nine taps.  A CTA owns one channel tile of each side (3 BN columns of
+// TMEM) and one contiguous run of positions; it writes its FP32 partial
+// sums to part[split][co][9 ci], the layout of dW, and weight_sum_kernel adds the splits
+// in a fixed order.  K runs in stages of 64 positions through a ring of four buffers: warps 0-7 stage
+// by cp.async, two stages behind the newest copies they announce the ones that landed; warp 8
+// issues the twelve MMAs of a stage.  Bound: the latency of a CTA's stages (issue active 31-48 %, tensor pipe
+// 11-23 %) and L2 (three copies of X).  With M = output channels and one row ky per CTA, 32 output channels
+// filled a quarter of each MMA, every CTA staged dY once per row and the copies' instructions
+// bound (issue active 66-71 %).  Kernel and sum of the splits, before and now: 16 x 256 x 256, 32 -> 32 193 and 115 us;
+// 32 x 64 x 64, 96 -> 32 61 and 36; 32 x 32 x 32, 192 -> 64 39 and 28; 32 x 16 x 16, 384 -> 128 39 and 29;
+// 16 x 32 x 32, 256 -> 256 79 and 59.  Two warps filling a whole buffer each instead of all eight
+// filling every one: 111, 37, 31, 38 and 73.
 // ---------------------------------------------------------------------------
 constexpr int kWgK = 64, kWgStages = 4, kWgStagers = 256, kWgThreads = 288, kWgLag = 2;
 
 struct LinWgrad {
     LinImage im;
-    int Cin, Cout, co_tile;     // co_tile: output channels staged per CTA (at most 128)
-    FastDiv dgx, dgy;           // by BN / 8 and co_tile / 8
+    int Cin, Cout;
     int spx, spy;               // positions per staged group
     int per, splits;            // positions per split
-    bool wide;                  // part on a 32-byte boundary
     // bias gradient: blocks behind the splits' (bias_blocks = 0: none), gw groups of 8 channels
     // and bias_per pixels each
     int bias_blocks, gw;
@@ -513,25 +513,37 @@ __device__ __forceinline__ void bias_partial(const __nv_bfloat16 *__restrict__ d
         g.bpart[(long long)split * g.Cout + gb * g.gw * 8 + i] = red[(i & 7) * 256 + (i >> 3)];
 }
 
-// One warp copies positions q .. q + n - 1 (n <= 32) with G channel groups from src, whose
-// pixels are `stride` channels apart, to dst[(group sp + position) 16 bytes], channel group fastest:
-// lane l finds the pixel of position l once, the copies get it by shuffle; positions from `valid`
-// on are zeros.  (For the stages of a weight gradient, each a few copies per thread: 192 -> 64
-// channels at 32 x 32 x 32 44 -> 39 us.  The slabs of conv3x3_lin_kernel, many copies per
+// One warp's eighth of a stage: positions 9 warp .. 9 warp + 8 of the 66 of X, which run from one before the
+// stage's to one after, in the rows above, at and below, and of dY those of the middle row.  Lane 9 r + j finds
+// the pixel of position j of row r once, the copies get it by shuffle, channel group fastest.  dY
+// is zero from position `valid` on.  (192 -> 64 channels at 32 x 32 x 32, one row per CTA: 44 -> 39 us against
+// finding the pixel for every copy.  The slabs of conv3x3_lin_kernel, many copies per
 // thread, are faster with the pixel found for every copy and 256 threads abreast: 53 against 63 us
 // at 16 x 256 x 256, 32 -> 32; plain loads and stores instead of cp.async 62-67 us.)
-__device__ __forceinline__ void stage_run(const LinImage &im, int q, int n, int lane,
-                                          const __nv_bfloat16 *__restrict__ src, int stride, int G, FastDiv dg,
-                                          unsigned char *dst, int sp, int valid = 32) {
-    const int mine = lane < min(n, valid) ? lin_pixel(im, q + lane) : -1;
-    const int total = n * G;
-#pragma unroll 4
-    for (int base = 0; base < total; base += 32) {
-        const int e = base + lane, pos = div_by(e, dg), grp = e - pos * G;
-        const int px = __shfl_sync(0xffffffffu, mine, pos & 31);
-        if (e < total)
-            cp_async16(dst + (grp * sp + pos) * 16, px >= 0 ? src + (long long)px * stride + grp * 8 : src,
+template <int CI, int BN>
+__device__ __forceinline__ void wgrad_stage(const LinWgrad &g, int q, int warp, int lane, int valid,
+                                            const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__restrict__ dy,
+                                            unsigned char *X, unsigned char *Y) {
+    constexpr int Gx = CI / 8, Gy = BN / 8;
+    const int j0 = 9 * warp, nj = min(9, kWgK + 2 - j0);
+    const int row = lane / 9, j = lane - 9 * row;
+    const int mine = row < 3 && j < nj ? lin_pixel(g.im, q + (row - 1) * g.im.Wp - 1 + j0 + j) : -1;
+#pragma unroll
+    for (int base = 0; base < 27 * Gx; base += 32) {
+        const int e = base + lane, i = e / Gx, grp = e % Gx, r = i / 9, pos = i - 9 * r;
+        const int px = __shfl_sync(0xffffffffu, mine, i & 31);
+        if (i < 27 && pos < nj)
+            cp_async16(X + ((r * Gx + grp) * g.spx + j0 + pos) * 16, px >= 0 ? x + (long long)px * g.Cin + grp * 8 : x,
                        px >= 0 ? 16 : 0);
+    }
+#pragma unroll
+    for (int base = 0; base < 9 * Gy; base += 32) {
+        const int e = base + lane, i = e / Gy, grp = e % Gy, pos = j0 + i - 1;
+        const int px = __shfl_sync(0xffffffffu, mine, (9 + i) & 31);
+        if (i < nj && pos >= 0 && pos < kWgK)
+            cp_async16(Y + (grp * g.spy + pos) * 16,
+                       px >= 0 && pos < valid ? dy + (long long)px * g.Cout + grp * 8 : dy,
+                       px >= 0 && pos < valid ? 16 : 0);
     }
 }
 
@@ -541,15 +553,15 @@ __device__ __forceinline__ void wgrad_slices(uint32_t tmem, uint64_t ad, uint64_
     for (int j = 0; j < kWgK / 16; ++j)
 #pragma unroll
         for (int kx = 0; kx < 3; ++kx)
-            mma_f16(tmem + (uint32_t)(kx * BN), ad + j * 16, bd + j * 16 + kx, idesc, kFirst && j == 0 ? 0u : 1u, lead);
+            mma_f16(tmem + (uint32_t)(kx * BN), ad + j * 16 + kx, bd + j * 16, idesc, kFirst && j == 0 ? 0u : 1u, lead);
 }
 
-template <int BN>
+template <int CI, int BN>
 __global__ void __launch_bounds__(kWgThreads) conv3x3_wgrad_lin_kernel(const __nv_bfloat16 *__restrict__ x,
                                                                        const __nv_bfloat16 *__restrict__ dy,
                                                                        float *__restrict__ part, const LinWgrad g) {
     constexpr int kNeed = 3 * BN;
-    constexpr uint32_t kCols = kNeed <= 64 ? 64u : (kNeed <= 128 ? 128u : (kNeed <= 256 ? 256u : 512u));
+    constexpr uint32_t kCols = kNeed <= 128 ? 128u : (kNeed <= 256 ? 256u : 512u);
     extern __shared__ __align__(128) unsigned char wg_smem[];
     __shared__ __align__(8) uint64_t full[kWgStages], empty[kWgStages], done;
     __shared__ uint32_t tmem_slot;
@@ -560,14 +572,13 @@ __global__ void __launch_bounds__(kWgThreads) conv3x3_wgrad_lin_kernel(const __n
         return;
     }
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
-    const int ci_tiles = g.Cin / BN;
-    const int ky = blockIdx.x % 3, ci0 = (blockIdx.x / 3 % ci_tiles) * BN, co0 = (blockIdx.x / 3 / ci_tiles) * g.co_tile;
+    const int ci_tiles = g.Cin / CI;
+    const int ci0 = (blockIdx.x % ci_tiles) * CI, co0 = (blockIdx.x / ci_tiles) * BN;
     const int qbeg = blockIdx.y * g.per, qend = min(g.im.L, qbeg + g.per);
     const int nst = (qend - qbeg + kWgK - 1) / kWgK;  // >= 1: no split is empty
-    const int Gx = BN / 8, Gy = g.co_tile >> 3;
-    // the MMA reads 16 groups of dY; with fewer staged ones the rest is whatever lies
-    // behind them, in rows whose sums are not used (the launch leaves room for them after the last buffer)
-    const uint32_t ybytes = (uint32_t)(Gy * g.spy) * 16u, xbytes = (uint32_t)(Gx * g.spx) * 16u;
+    // the MMA reads 16 groups of X; behind the staged ones (3 CI / 8) it reads whatever lies
+    // there, for rows whose sums are not used (wgrad_smem leaves room behind the last buffer)
+    const uint32_t xbytes = (uint32_t)(3 * CI / 8 * g.spx) * 16u, ybytes = (uint32_t)(BN / 8 * g.spy) * 16u;
 
     if (warp == 8) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
@@ -600,14 +611,9 @@ __global__ void __launch_bounds__(kWgThreads) conv3x3_wgrad_lin_kernel(const __n
             if (s >= kWgStages)
                 ok = warp_wait(&empty[s % kWgStages], (uint32_t)((s / kWgStages - 1) & 1), lane, &abort_flag);
             if (!ok) break;
-            unsigned char *Y = wg_smem + (s % kWgStages) * (ybytes + xbytes), *X = Y + ybytes;
+            unsigned char *X = wg_smem + (s % kWgStages) * (xbytes + ybytes);
             const int q = qbeg + s * kWgK;
-            // each warp an eighth of the positions: 8 of dY, 9 (the last one fewer) of X, which run from one
-            // position before the stage's to one after, in row ky
-            const int qy = q + 8 * warp, ny = max(0, min(8, qend - qy));
-            stage_run(g.im, qy, 8, lane, dy + co0, g.Cout, Gy, g.dgy, Y + 8 * warp * 16, g.spy, ny);
-            stage_run(g.im, q + (ky - 1) * g.im.Wp - 1 + 9 * warp, min(9, kWgK + 2 - 9 * warp), lane, x + ci0, g.Cin, Gx,
-                      g.dgx, X + 9 * warp * 16, g.spx, 9);
+            wgrad_stage<CI, BN>(g, q, warp, lane, qend - q, x + ci0, dy + co0, X, X + xbytes);
             cp_async_commit();
             if (s >= kWgLag) {
                 cp_async_wait<kWgLag>();
@@ -620,9 +626,9 @@ __global__ void __launch_bounds__(kWgThreads) conv3x3_wgrad_lin_kernel(const __n
     } else {
         const uint32_t lead = elect_lane();
         constexpr uint32_t idesc = mma_idesc(128, BN) | (1u << 15) | (1u << 16);  // both operands MN-major
-        const uint32_t stage = (ybytes + xbytes) >> 4;
-        const uint64_t ad = smem_desc(smem_u32(wg_smem), 128, (uint32_t)g.spy * 16);
-        const uint64_t bd = smem_desc(smem_u32(wg_smem) + ybytes, 128, (uint32_t)g.spx * 16);
+        const uint32_t stage = (xbytes + ybytes) >> 4;
+        const uint64_t ad = smem_desc(smem_u32(wg_smem), 128, (uint32_t)g.spx * 16);
+        const uint64_t bd = smem_desc(smem_u32(wg_smem) + xbytes, 128, (uint32_t)g.spy * 16);
         for (int s = 0; s < nst; ++s) {
             const int b = s % kWgStages;
             ok = ws_wait(smem_u32(&full[b]), (uint32_t)((s / kWgStages) & 1), &abort_flag);
@@ -639,31 +645,20 @@ __global__ void __launch_bounds__(kWgThreads) conv3x3_wgrad_lin_kernel(const __n
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (warp < 8 && abort_flag == 0) {
-        // TMEM lane = row = output channel; warps w and w + 4 share the lanes of quarter w & 3
-        const int quarter = warp & 3, r0 = quarter * 32 + lane;
-        float *const row = part + ((long long)blockIdx.y * g.Cout + co0 + r0) * (9 * g.Cin) + 3 * ky * g.Cin + ci0;
+    const int quarter = warp & 3, r0 = quarter * 32 + lane, ky = r0 / CI;
+    if (warp < 8 && quarter * 32 < 3 * CI && abort_flag == 0) {
+        // TMEM lane = row = (ky, input channel): a column's lanes are consecutive floats of dW;
+        // warps w and w + 4 share the lanes of quarter w & 3
+        float *const col = part + ((long long)blockIdx.y * g.Cout + co0) * (9 * g.Cin) + 3 * ky * g.Cin + ci0 + r0 % CI;
 #pragma unroll 2
         for (int c = (warp >> 2) * 16; c < 3 * BN; c += 32) {
             uint32_t r[16];
             tmem_load<16>(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c, r);
             tmem_wait_ld();
-            if (r0 < g.co_tile) {
-                float *const d = row + (c / BN) * g.Cin + c % BN;
-                // whole 32-byte sectors: a warp's rows lie 36 Cin bytes apart
-                if (g.wide) {
+            float *const d = col + (long long)(c % BN) * (9 * g.Cin) + (c / BN) * g.Cin;
+            if (ky < 3)
 #pragma unroll
-                    for (int q = 0; q < 2; ++q)
-                        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(d + 8 * q),
-                                     "r"(r[8 * q]), "r"(r[8 * q + 1]), "r"(r[8 * q + 2]), "r"(r[8 * q + 3]),
-                                     "r"(r[8 * q + 4]), "r"(r[8 * q + 5]), "r"(r[8 * q + 6]), "r"(r[8 * q + 7])
-                                     : "memory");
-                } else {
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        reinterpret_cast<uint4 *>(d)[q] = make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
-                }
-            }
+                for (int k = 0; k < 16; ++k) d[(long long)k * (9 * g.Cin)] = __uint_as_float(r[k]);
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -862,43 +857,44 @@ cudaError_t conv_lin(const __nv_bfloat16 *in, const __nv_bfloat16 *w, const floa
     }
 }
 
-// The weight gradient's tiling: BN input channels per CTA and the positions per split, a
+// The weight gradient's tiling: BN output channels per CTA and the positions per split, a
 // multiple of 64 and at most 1024 (the FP32 sums of one split stay as short as they were with
 // 16 stages of 64 pixels), for the least estimated time in SM cycles: the busiest SM's MMAs or
 // its CTAs' stages one after the other (about 900 cycles each), and the partial sums, written
 // once and read once at about 20 bytes a cycle and SM.  Then the bias gradient's blocks, at
 // most about two per SM, with at least 16 pixels a thread.
 struct WgLinPlan {
-    int bn = 0, co_tile = 0, splits = 0, per = 0;
+    int ci = 0, bn = 0, splits = 0, per = 0;
     int gw = 0, bias_splits = 0;
     long long bias_per = 0;
     size_t smem = 0;
 };
-inline size_t wgrad_smem(int bn, int co_tile) {
-    const int gy = co_tile / 8, gx = bn / 8, spy = lin_stride(kWgK, gy), spx = lin_stride(kWgK + 2, gx);
-    return std::max<size_t>(16ull * (kWgStages * (gy * spy + gx * spx) + (16 - gy) * spy), 8 * 256 * sizeof(float));
+inline size_t wgrad_smem(int ci, int bn) {
+    const int spx = lin_stride(kWgK + 2, ci / 8), spy = lin_stride(kWgK, bn / 8), x = 3 * ci / 8 * spx, y = bn / 8 * spy;
+    return std::max<size_t>(16ull * (kWgStages * (x + y) + std::max(0, 16 * spx - x - y)), 8 * 256 * sizeof(float));
 }
 inline WgLinPlan make_wgrad_lin_plan(long long L, long long P, int Cin, int Cout) {
     constexpr int kSms = 152;  // (the workspace query has no device to ask)
     WgLinPlan w;
-    w.co_tile = Cout % 128 == 0 ? 128 : (Cout % 64 == 0 ? 64 : 32);
+    w.ci = Cin % 32 ? 16 : 32;
     double least = 1e30;
-    for (int bn : {64, 32, 16}) {
-        if (Cin % bn) continue;
-        const long long tiles = 3ll * (Cin / bn) * (Cout / w.co_tile);
-        const int cols = 3 * bn <= 64 ? 64 : (3 * bn <= 128 ? 128 : 256);
-        const int occ = (int)std::max<size_t>(1, std::min<size_t>({228 * 1024 / (wgrad_smem(bn, w.co_tile) + 2048), 512u / cols, 7u}));
+    for (int bn : {128, 64, 32}) {
+        if (Cout % bn) continue;
+        const long long tiles = (long long)(Cin / w.ci) * (Cout / bn);
+        const int cols = 3 * bn <= 128 ? 128 : (3 * bn <= 256 ? 256 : 512);
+        const int occ = (int)std::max<size_t>(1, std::min<size_t>({228 * 1024 / (wgrad_smem(w.ci, bn) + 2048), 512u / cols, 7u}));
         for (int per : {1024, 896, 768, 640, 512, 384, 256, 192, 128}) {
             const long long s = (L + per - 1) / per, ctas = tiles * s;
             const double n = (double)((ctas + kSms - 1) / kSms), nst = std::min<double>(per, (double)L) / kWgK;
-            const double mma = n * nst * 12 * (32 + bn / 4.0), chain = std::ceil(n / occ) * (nst * 900 + 3000);
+            const double slice = bn == 128 ? 64 : (bn == 64 ? 48 : 45);
+            const double mma = n * nst * 12 * slice, chain = std::ceil(n / occ) * (nst * 900 + 3000);
             const double time = std::max(mma, chain) + 2.0 * s * 36 * Cin * Cout / (kSms * 20.0);
             if (time < least) {
                 least = time;
                 w.bn = bn;
                 w.per = per;
                 w.splits = (int)s;
-                w.smem = wgrad_smem(bn, w.co_tile);
+                w.smem = wgrad_smem(w.ci, bn);
             }
         }
     }
@@ -916,7 +912,7 @@ inline WgLinPlan wgrad_lin_plan(long long L, long long P, int Cin, int Cout) {
     return plans.get({L, P, Cin, Cout, 0, 0}, [&] { return make_wgrad_lin_plan(L, P, Cin, Cout); });
 }
 
-template <int BN>
+template <int CI, int BN>
 cudaError_t launch_wgrad_lin(const __nv_bfloat16 *x, const __nv_bfloat16 *dy, float *part, const LinWgrad &g,
                              size_t smem, cudaStream_t s) {
     static std::atomic<bool> set[64];
@@ -924,16 +920,16 @@ cudaError_t launch_wgrad_lin(const __nv_bfloat16 *x, const __nv_bfloat16 *dy, fl
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev >= 64 || !set[dev].load()) {
-        e = cudaFuncSetAttribute(conv3x3_wgrad_lin_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmemCta);
+        e = cudaFuncSetAttribute(conv3x3_wgrad_lin_kernel<CI, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmemCta);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(conv3x3_wgrad_lin_kernel<BN>, cudaFuncAttributePreferredSharedMemoryCarveout,
+            e = cudaFuncSetAttribute(conv3x3_wgrad_lin_kernel<CI, BN>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                      (int)cudaSharedmemCarveoutMaxShared);
         if (e != cudaSuccess) return e;
         if (dev < 64) set[dev].store(true);
     }
-    const int tiles = 3 * (g.Cin / BN) * (g.Cout / g.co_tile);
+    const int tiles = (g.Cin / CI) * (g.Cout / BN);
     const dim3 grid((unsigned)tiles, (unsigned)(g.splits + (g.bias_blocks + tiles - 1) / tiles));
-    conv3x3_wgrad_lin_kernel<BN><<<grid, kWgThreads, smem, s>>>(x, dy, part, g);
+    conv3x3_wgrad_lin_kernel<CI, BN><<<grid, kWgThreads, smem, s>>>(x, dy, part, g);
     return cudaGetLastError();
 }
 
@@ -943,22 +939,19 @@ inline cudaError_t wgrad_lin(const __nv_bfloat16 *x, const __nv_bfloat16 *dy, fl
     g.im = im;
     g.Cin = Cin;
     g.Cout = Cout;
-    g.co_tile = w.co_tile;
-    g.dgx = fast_div((uint32_t)w.bn / 8);
-    g.dgy = fast_div((uint32_t)w.co_tile / 8);
-    g.spx = lin_stride(kWgK + 2, w.bn / 8);
-    g.spy = lin_stride(kWgK, w.co_tile / 8);
+    g.spx = lin_stride(kWgK + 2, w.ci / 8);
+    g.spy = lin_stride(kWgK, w.bn / 8);
     g.per = w.per;
     g.splits = w.splits;
-    g.wide = (reinterpret_cast<uintptr_t>(part) & 31) == 0;
     g.bias_blocks = bpart ? w.bias_splits * (Cout / 8 / w.gw) : 0;
     g.gw = w.gw;
     g.P = P;
     g.bias_per = w.bias_per;
     g.bpart = bpart;
+    const bool c32 = w.ci == 32;
     switch (w.bn) {
-        case 64: return launch_wgrad_lin<64>(x, dy, part, g, w.smem, s);
-        case 32: return launch_wgrad_lin<32>(x, dy, part, g, w.smem, s);
-        default: return launch_wgrad_lin<16>(x, dy, part, g, w.smem, s);
+        case 128: return c32 ? launch_wgrad_lin<32, 128>(x, dy, part, g, w.smem, s) : launch_wgrad_lin<16, 128>(x, dy, part, g, w.smem, s);
+        case 64: return c32 ? launch_wgrad_lin<32, 64>(x, dy, part, g, w.smem, s) : launch_wgrad_lin<16, 64>(x, dy, part, g, w.smem, s);
+        default: return c32 ? launch_wgrad_lin<32, 32>(x, dy, part, g, w.smem, s) : launch_wgrad_lin<16, 32>(x, dy, part, g, w.smem, s);
     }
 }
