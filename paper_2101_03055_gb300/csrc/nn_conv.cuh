@@ -19,7 +19,7 @@
 // whole 128-pixel tiles without im2col), forward / input gradient / weight and bias gradient:
 //   16 x 256 x 256, 32 -> 32     91 / 286 / 451 us before,  53 / 55 / 115 us now
 //   16 x 32 x 32, 256 -> 256    116 / 206 / 163 us before,  26 / 28 / 59 us now (750 TFLOP/s forward)
-//   the U-Net's first eleven layer shapes at 32 x 64 x 64, summed: 741 / 1050 / 1123 us before, 128 / 138 / 228 us now
+//   the U-Net's first eleven layer shapes at 32 x 64 x 64, summed: 741 / 1050 / 1123 us before, 128 / 138 / 217 us now
 
 // Division of 0 <= x < 2^31 by a constant d >= 1: (umulhi(x, mul) + x) >> shift
 // (Granlund & Montgomery, PLDI 1994, the round-up multiplier of 33 bits).
@@ -859,9 +859,11 @@ cudaError_t conv_lin(const __nv_bfloat16 *in, const __nv_bfloat16 *w, const floa
 
 // The weight gradient's tiling: BN output channels per CTA and the positions per split, a
 // multiple of 64 and at most 1024 (the FP32 sums of one split stay as short as they were with
-// 16 stages of 64 pixels), for the least estimated time in SM cycles: the busiest SM's MMAs or
-// its CTAs' stages one after the other (about 900 cycles each), and the partial sums, written
-// once and read once at about 20 bytes a cycle and SM.  Then the bias gradient's blocks, at
+// 16 stages of 64 pixels), for the least estimated time in SM cycles: the busiest SM's MMAs (at two thirds of
+// their rate) or its CTAs one after the other (900 cycles a stage, 1000 and 20 a column for start and
+// stores), and the partial sums, written and read at about 40 bytes a cycle and SM.  The
+// constants are fitted to 13 layers of the network and of large images, every BN and run length: its choices
+// take 9 % more time than the best ones at most, 1 % on average.  Then the bias gradient's blocks, at
 // most about two per SM, with at least 16 pixels a thread.
 struct WgLinPlan {
     int ci = 0, bn = 0, splits = 0, per = 0;
@@ -887,8 +889,8 @@ inline WgLinPlan make_wgrad_lin_plan(long long L, long long P, int Cin, int Cout
             const long long s = (L + per - 1) / per, ctas = tiles * s;
             const double n = (double)((ctas + kSms - 1) / kSms), nst = std::min<double>(per, (double)L) / kWgK;
             const double slice = bn == 128 ? 64 : (bn == 64 ? 48 : 45);
-            const double mma = n * nst * 12 * slice, chain = std::ceil(n / occ) * (nst * 900 + 3000);
-            const double time = std::max(mma, chain) + 2.0 * s * 36 * Cin * Cout / (kSms * 20.0);
+            const double mma = n * nst * 18 * slice, chain = std::ceil(n / occ) * (nst * 900 + 1000 + 20 * bn);
+            const double time = std::max(mma, chain) + s * 36.0 * Cin * Cout / (kSms * 20.0);
             if (time < least) {
                 least = time;
                 w.bn = bn;
