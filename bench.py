@@ -110,7 +110,7 @@ def describe(name: str) -> str:
         "cde_cellular_2048": "Case 1 cellular flow at 2048x2048 (profiling size above L2)",
         "batched_plume_sweep_64": "64 chemotaxis-plume instances of the 256-instance sweep (profiling size)",
         "batched_plume_sweep_256": "256 chemotaxis-plume instances, W~U{128..512} x H~U{64..256} (13.2 M nodes), "
-                                   "per-instance chi, D_c, gravity; execution mode (persistent kernel or graph of per-instance "
+                                   "per-instance chi, D_c, gravity; execution mode (whole-batch launches or graph of per-instance "
                                    "chains of one- or two-step launches) and tiles picked by the autotuner",
     }[name]
 
@@ -361,28 +361,38 @@ class _Batch:
                            f"CTAs of {info.chain_block_x}x{info.chain_block_y}, output tiles "
                            f"{info.chain_block_x - 2}x{info.chain_tile_y}; graph of 32 steps over a 32-stream pool)")
         else:
-            self.kernel = (f"batch_kernel<{self.m}> (persistent, {info.grid_blocks} CTAs, "
-                           f"{info.steps_per_launch} steps/launch)")
+            # instances in the groups of one launch: a multiple of four groups of about 20 MiB of populations
+            # (both buffers), at most 64 instances each
+            size = [8 * (9 + 5 * pb.m + (info.bytes_per_lup > 8 * (9 + 5 * pb.m))) * ((pb.nx + 31) // 32 * 32) * pb.ny
+                    for pb in pbs]
+            want = (sum(size) // (20 << 20) + 4) // 4 * 4
+            before, last, run, self.groups = 0, 0, 0, 1
+            for k, b in enumerate(size):
+                g = int((before + 0.5 * b) / sum(size) * want)
+                if k and (g != last or run == 64):
+                    self.groups, run = self.groups + 1, 0
+                before, last, run = before + b, g, run + 1
+            self.kernel = (f"step2_batch_kernel<{self.m}> (two time steps of a group of instances per launch, "
+                           f"{self.groups} groups; graph of 32 steps over 4 streams)")
         self.mode = info.mode
         self.count = info.count
-        self.spl = info.steps_per_launch
 
     def steps_per_launch(self, n):
-        """Lattice steps per launch of the dominant kernel inside step(n) (chains:
-        one or two lattice steps of one instance, counted here per whole sweep step)."""
-        return {1: 1, 2: 2 if n >= 2 else 1}.get(self.mode, min(n, self.spl))
+        """Lattice steps per launch of the dominant kernel inside step(n) (of one instance
+        or one group of them, counted here per whole sweep step)."""
+        return 1 if self.mode == 1 or n < 2 else 2
 
     def updates_per_pass(self, n):
-        """Updates per read + write of the state: the persistent kernel passes over
-        global memory every step; chains of two-step launches once per two steps."""
-        return 2 if (self.mode == 2 and n >= 2) else 1
+        """Updates per read + write of the state: launches of two steps pass over
+        global memory once per two steps."""
+        return 2 if (self.mode != 1 and n >= 2) else 1
 
     def launches(self, n):
         if self.mode == 1:
             return n * self.count
         if self.mode == 2:
             return (n // 2 + n % 2) * self.count
-        return -(-n // self.spl)
+        return n // 2 * self.groups + n % 2
 
     stream = property(lambda self: self.s.stream)
 
@@ -487,10 +497,7 @@ def conv_line(N, H, W, Cin, Cout, reps, device, peak_tflops, peak_gbs):
     return {"description": f"3x3 convolution forward (bias + ReLU), N={N} {H}x{W}, {Cin}->{Cout} channels, BF16 "
                            f"operands, FP32 accumulation in tensor memory",
             "value": tf, "unit": "TFLOP/s", "launch_us": us, "flops_per_launch": flops,
-            "kernel": (f"conv3x3_slab_kernel<{min(Cout, 128 if Cin < 64 else 64)},{Cin // 8}> (no im2col copy, "
-                       f"persistent)" if W % 128 == 0 and Cin in (16, 32, 64) else
-                       f"conv3x3_tc_pipe_kernel<false,{Cout if Cout <= 128 else 128}>" if Cin >= 128 else
-                       f"conv3x3_tc_kernel<false,{Cout if Cout <= 128 else 128}>"), "gpu_launches": 2 * reps,
+            "kernel": "conv3x3_lin_kernel<false> (no im2col copy, persistent)", "gpu_launches": 2 * reps,
             "synchronous_staging": {"kernel": f"conv3x3_tc_kernel<false,{Cout if Cout <= 128 else 128}>",
                                     "launch_us": us_sync, "value": flops / us_sync / 1e6},
             "roofline": {"bound": "tensor" if flops / nbytes > peak_tflops * 1e12 / (peak_gbs * 1e9) else "hbm",
@@ -526,11 +533,11 @@ def wgrad_line(N, H, W, Cin, Cout, reps, device, peak_tflops, peak_gbs):
     flops = 2.0 * N * H * W * 9 * Cin * Cout
     nbytes = 2.0 * N * H * W * (Cin + Cout) + 4.0 * 9 * Cin * Cout
     tf = flops / us / 1e6
-    bn = 256 if Cout % 256 == 0 else (128 if Cout % 128 == 0 else (64 if Cout % 64 == 0 else 32))
     return {"description": f"3x3 convolution weight + bias gradient, N={N} {H}x{W}, {Cin}->{Cout} channels, BF16 "
                            f"operands, FP32 accumulation in tensor memory, pixel splits summed in a fixed order",
             "value": tf, "unit": "TFLOP/s", "launch_us": us, "flops_per_launch": flops,
-            "kernel": f"conv3x3_wgrad_tc_kernel<{bn}>", "gpu_launches": 4 * reps,
+            "kernel": "conv3x3_wgrad_lin_kernel (bias gradient in the same launch) and weight_sum_kernel",
+            "gpu_launches": 2 * reps,
             "roofline": {"bound": "tensor" if flops / nbytes > peak_tflops * 1e12 / (peak_gbs * 1e9) else "hbm",
                          "achieved": tf, "peak": peak_tflops, "unit": "TFLOP/s", "frac": tf / peak_tflops,
                          "traffic": None, "peak_source": "measured BF16 GEMM burst (MEASURED_PEAKS.json bf16_tflops)",
@@ -853,7 +860,7 @@ def main():
                     help="slab: one single lattice split along y over the ranks, halo exchange through NCCL "
                          "after every step (strong scaling); none: every rank its own instance (weak scaling)")
     ap.add_argument("--batch-mode", type=int, default=0, choices=[0, 1, 2],
-                    help="with --batch-tile: the batched solver's mode (0 persistent, 1 chains, 2 two-step chains)")
+                    help="with --batch-tile: the batched solver's mode (0 whole batch, 1 chains, 2 two-step chains)")
     ap.add_argument("--batch-tile", default=None,
                     help="'X,Y': tile (mode 0) or CTA shape (modes 1, 2) of the batched solver, 'X,Y,TH,LANES' in "
                          "mode 2 (tile height, nodes per thread); default: autotuned")
