@@ -1463,8 +1463,14 @@ long long cdf_nn_conv3x3_bwd_weight_workspace(int N, int H, int W, int Cin, int 
     if (N < 1 || H < 1 || W < 1 || Cin < 16 || Cin % 16 || Cout < 32 || Cout % 32) return -1;
     const int images = wgrad_images(N, H, W);
     if (images == 0) return 4;  // the warp-level kernel adds to dw directly
-    const WgLinPlan w = wgrad_lin_plan((long long)images * (H + 1) * (W + 1), (long long)images * H * W, Cin, Cout);
-    return ((long long)w.splits * 9 * Cin + w.bias_splits) * Cout * (long long)sizeof(float);
+    // the largest of the launches: all images, or runs of `images` and a remainder with a tiling of its own
+    long long most = 0;
+    for (int n : {images, N % images})
+        if (n > 0) {
+            const WgLinPlan w = wgrad_lin_plan((long long)n * (H + 1) * (W + 1), (long long)n * H * W, Cin, Cout);
+            most = std::max(most, ((long long)w.splits * 9 * Cin + w.bias_splits) * Cout * (long long)sizeof(float));
+        }
+    return most;
 }
 
 cdf_nn_status cdf_nn_conv3x3_bwd_weight(const void *x, const void *dy, float *dw, float *db, int N, int H, int W,

@@ -126,7 +126,7 @@ def conv3x3_bwd_data_relu(dy, w, y):
 _workspace = {}
 
 
-@functools.lru_cache(maxsize=None)
+@functools.lru_cache(maxsize=256)
 def _weight_workspace(N, H, W, Cin, Cout):
     return int(nn_lib().cdf_nn_conv3x3_bwd_weight_workspace(N, H, W, Cin, Cout))
 
