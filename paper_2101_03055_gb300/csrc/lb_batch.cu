@@ -276,8 +276,6 @@ cdf_status setup_tiles(cdf_batch *b, dim3 tile) {
         inst[k].pair_tiles = inst[k].pair_x * ((p.ny + th - 1) / th);
         inst[k].tw = tw;
         inst[k].th = th;
-        inst[k].inv_w1 = ((1u << 20) + tw + 1) / (tw + 2);
-        inst[k].inv_tw = ((1u << 20) + tw - 1) / tw;
     }
     const auto bytes = [b](int k) { return 8ll * (9 + 5 * b->m + b->sprev_planes) * b->params[k].plane; };
     long long total = 0, before = 0, last = 0;

@@ -139,7 +139,6 @@ struct BatchInst {
     int pair_tiles;      // the same for the two-step launches: tiles of tw x th
     int pair_x;
     int tw, th;
-    unsigned inv_w1, inv_tw;  // ceil(2^20 / (tw + 2)), ceil(2^20 / tw)
 };
 // The instances of one two-step launch, as a kernel parameter (at most 32,764 bytes in all).
 constexpr int kBatchGroup = 64;
