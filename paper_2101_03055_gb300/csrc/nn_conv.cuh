@@ -456,7 +456,8 @@ __global__ void __launch_bounds__(kLinThreads) conv3x3_lin_kernel(const __grid_c
 // three MMAs per 16 positions for nine taps.  A CTA owns one channel tile of each side (3 BN columns of
 // TMEM) and one contiguous run of positions; it writes its FP32 partial
 // sums to part[split][co][9 ci], the layout of dW, and weight_sum_kernel adds the splits
-// in a fixed order.  K runs in stages of 64 positions through a ring of four buffers: warps 0-7 stage
+// in a fixed order; a launch takes as many splits as keep their partial sums within kWgPartBytes,
+// and the next launch adds its own to dW.  K runs in stages of 64 positions through a ring of four buffers: warps 0-7 stage
 // by cp.async, two stages behind the newest copies they announce the ones that landed; warp 8
 // issues the twelve MMAs of a stage.  Bound: the latency of a CTA's stages (issue active 31-48 %, tensor pipe
 // 11-23 %) and L2 (three copies of X).  With M = output channels and one row ky per CTA, 32 output channels
@@ -472,6 +473,7 @@ struct LinWgrad {
     LinImage im;
     int Cin, Cout;
     int spx, spy;               // positions per staged group
+    int q0, q1;                 // the launch's positions
     int per, splits;            // positions per split
     // bias gradient: blocks behind the splits' (bias_blocks = 0: none), gw groups of 8 channels
     // and bias_per pixels each
@@ -574,7 +576,7 @@ __global__ void __launch_bounds__(kWgThreads) conv3x3_wgrad_lin_kernel(const __n
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int ci_tiles = g.Cin / CI;
     const int ci0 = (blockIdx.x % ci_tiles) * CI, co0 = (blockIdx.x / ci_tiles) * BN;
-    const int qbeg = blockIdx.y * g.per, qend = min(g.im.L, qbeg + g.per);
+    const int qbeg = g.q0 + blockIdx.y * g.per, qend = min(g.q1, qbeg + g.per);
     const int nst = (qend - qbeg + kWgK - 1) / kWgK;  // >= 1: no split is empty
     // the MMA reads 16 groups of X; behind the staged ones (3 CI / 8) it reads whatever lies
     // there, for rows whose sums are not used (wgrad_smem leaves room behind the last buffer)
@@ -867,10 +869,16 @@ cudaError_t conv_lin(const __nv_bfloat16 *in, const __nv_bfloat16 *w, const floa
 // most about two per SM, with at least 16 pixels a thread.
 struct WgLinPlan {
     int ci = 0, bn = 0, splits = 0, per = 0;
+    int run = 0;  // splits of one launch at most
     int gw = 0, bias_splits = 0;
     long long bias_per = 0;
     size_t smem = 0;
 };
+// Partial sums of one launch.  A split sums at most 1024 positions, so without a bound they grow with
+// the pixels: 2.4 GB for 16 x 256 x 256, 256 -> 256, and more splits than a grid has rows
+// from 2^26 positions on.  That layer takes 3.68 ms with 160 MB as with 64 and 3.24 in one launch (12.3 on the
+// im2col kernel); 1 x 241 x 241, 256 -> 256 takes 215 us with 160 MB, where it is one launch, and 254 with 64.
+constexpr long long kWgPartBytes = 160ll << 20;
 inline size_t wgrad_smem(int ci, int bn) {
     const int spx = lin_stride(kWgK + 2, ci / 8), spy = lin_stride(kWgK, bn / 8), x = 3 * ci / 8 * spx, y = bn / 8 * spy;
     return std::max<size_t>(16ull * (kWgStages * (x + y) + std::max(0, 16 * spx - x - y)), 8 * 256 * sizeof(float));
@@ -900,6 +908,8 @@ inline WgLinPlan make_wgrad_lin_plan(long long L, long long P, int Cin, int Cout
             }
         }
     }
+    const long long most = std::max(1ll, kWgPartBytes / (36ll * Cin * Cout)), launches = (w.splits + most - 1) / most;
+    w.run = (int)((w.splits + launches - 1) / launches);
     w.gw = 32;
     while ((Cout / 8) % w.gw) w.gw /= 2;
     const long long groups = Cout / 8 / w.gw, lanes = 256 / w.gw;
@@ -907,6 +917,11 @@ inline WgLinPlan make_wgrad_lin_plan(long long L, long long P, int Cin, int Cout
     w.bias_per = (P + bs - 1) / bs;
     w.bias_splits = (int)((P + w.bias_per - 1) / w.bias_per);
     return w;
+}
+
+// Workspace of a call's largest launch, in bytes.
+inline long long wgrad_bytes(const WgLinPlan &w, int Cin, int Cout) {
+    return ((long long)w.run * 9 * Cin + w.bias_splits) * Cout * (long long)sizeof(float);
 }
 
 inline WgLinPlan wgrad_lin_plan(long long L, long long P, int Cin, int Cout) {
@@ -935,8 +950,10 @@ cudaError_t launch_wgrad_lin(const __nv_bfloat16 *x, const __nv_bfloat16 *dy, fl
     return cudaGetLastError();
 }
 
+// `splits` of the plan's splits from s0 on; bpart: and the bias gradient over all P pixels.
 inline cudaError_t wgrad_lin(const __nv_bfloat16 *x, const __nv_bfloat16 *dy, float *part, float *bpart,
-                             const LinImage &im, long long P, int Cin, int Cout, const WgLinPlan &w, cudaStream_t s) {
+                             const LinImage &im, long long P, int Cin, int Cout, const WgLinPlan &w, int s0, int splits,
+                             cudaStream_t s) {
     LinWgrad g{};
     g.im = im;
     g.Cin = Cin;
@@ -944,7 +961,9 @@ inline cudaError_t wgrad_lin(const __nv_bfloat16 *x, const __nv_bfloat16 *dy, fl
     g.spx = lin_stride(kWgK + 2, w.ci / 8);
     g.spy = lin_stride(kWgK, w.bn / 8);
     g.per = w.per;
-    g.splits = w.splits;
+    g.splits = splits;
+    g.q0 = s0 * w.per;
+    g.q1 = (int)std::min<long long>(im.L, (long long)(s0 + splits) * w.per);
     g.bias_blocks = bpart ? w.bias_splits * (Cout / 8 / w.gw) : 0;
     g.gw = w.gw;
     g.P = P;

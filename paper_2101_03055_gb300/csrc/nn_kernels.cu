@@ -1468,7 +1468,7 @@ long long cdf_nn_conv3x3_bwd_weight_workspace(int N, int H, int W, int Cin, int 
     for (int n : {images, N % images})
         if (n > 0) {
             const WgLinPlan w = wgrad_lin_plan((long long)n * (H + 1) * (W + 1), (long long)n * H * W, Cin, Cout);
-            most = std::max(most, ((long long)w.splits * 9 * Cin + w.bias_splits) * Cout * (long long)sizeof(float));
+            most = std::max(most, wgrad_bytes(w, Cin, Cout));
         }
     return most;
 }
@@ -1495,17 +1495,22 @@ cdf_nn_status cdf_nn_conv3x3_bwd_weight(const void *x, const void *dy, float *dw
             LinImage im;
             if (!lin_image(n, H, W, &im)) return nn_fail("conv3x3_bwd_weight: too many positions");
             const WgLinPlan w = wgrad_lin_plan(im.L, Pn, Cin, Cout);
-            float *bpart = db ? part + (long long)w.splits * 9 * Cin * Cout : nullptr;  // after the weight partials
-            const cudaError_t e = wgrad_lin(xn, dyn, part, bpart, im, Pn, Cin, Cout, w, s);
-            if (e != cudaSuccess) { cudaGetLastError(); return nn_fail(cudaGetErrorString(e)); }
-            const auto sum = [&](auto r) {
-                constexpr int R = decltype(r)::value;
-                const int n4 = 9 * Cin * Cout / 4, wblocks = (n4 + R - 1) / R, bblocks = db ? (Cout / 4 + R - 1) / R : 0;
-                weight_sum_kernel<R><<<wblocks + bblocks, 256, 0, s>>>(part, dw, n4, w.splits, wblocks, bpart, db,
-                                                                       Cout / 4, w.bias_splits);
-            };
-            if (w.splits >= 128) sum(std::integral_constant<int, 8>{});
-            else sum(std::integral_constant<int, 32>{});
+            for (int s0 = 0; s0 < w.splits; s0 += w.run) {
+                const int splits = std::min(w.run, w.splits - s0);
+                // the bias gradient goes with the first launch, its partial sums behind the weights'
+                float *bpart = db && s0 == 0 ? part + (long long)w.run * 9 * Cin * Cout : nullptr;
+                const cudaError_t e = wgrad_lin(xn, dyn, part, bpart, im, Pn, Cin, Cout, w, s0, splits, s);
+                if (e != cudaSuccess) { cudaGetLastError(); return nn_fail(cudaGetErrorString(e)); }
+                const auto sum = [&](auto r) {
+                    constexpr int R = decltype(r)::value;
+                    const int n4 = 9 * Cin * Cout / 4, wblocks = (n4 + R - 1) / R;
+                    const int bblocks = bpart ? (Cout / 4 + R - 1) / R : 0;
+                    weight_sum_kernel<R><<<wblocks + bblocks, 256, 0, s>>>(part, dw, n4, splits, wblocks, bpart, db,
+                                                                           Cout / 4, w.bias_splits);
+                };
+                if (splits >= 128) sum(std::integral_constant<int, 8>{});
+                else sum(std::integral_constant<int, 32>{});
+            }
         }
     } else {
         // the warp-level MMA path: split-K partial sums added atomically (order-dependent)
