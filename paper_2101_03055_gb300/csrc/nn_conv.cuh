@@ -478,7 +478,7 @@ struct LinWgrad {
     // bias gradient: blocks behind the splits' (bias_blocks = 0: none), gw groups of 8 channels
     // and bias_per pixels each
     int bias_blocks, gw;
-    long long P, bias_per;
+    long long p0, P, bias_per;
     float *bpart;
 };
 
@@ -490,7 +490,7 @@ __device__ __forceinline__ void bias_partial(const __nv_bfloat16 *__restrict__ d
     const int gblocks = g.Cout / 8 / g.gw, split = block / gblocks, gb = block - split * gblocks;
     const int lanes = 256 / g.gw, gl = threadIdx.x % g.gw, pl = threadIdx.x / g.gw;
     const int c0 = (gb * g.gw + gl) * 8;
-    const long long p0 = split * g.bias_per, p1 = min(g.P, p0 + g.bias_per);
+    const long long p0 = g.p0 + split * g.bias_per, p1 = min(g.p0 + g.P, p0 + g.bias_per);
     const bool mine = threadIdx.x < 256;
     float s[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     if (mine) {
@@ -950,10 +950,10 @@ cudaError_t launch_wgrad_lin(const __nv_bfloat16 *x, const __nv_bfloat16 *dy, fl
     return cudaGetLastError();
 }
 
-// `splits` of the plan's splits from s0 on; bpart: and the bias gradient over all P pixels.
+// The positions [q0, q1) in `splits` splits; bpart: and the bias gradient over P pixels from p0 on.
 inline cudaError_t wgrad_lin(const __nv_bfloat16 *x, const __nv_bfloat16 *dy, float *part, float *bpart,
-                             const LinImage &im, long long P, int Cin, int Cout, const WgLinPlan &w, int s0, int splits,
-                             cudaStream_t s) {
+                             const LinImage &im, int q0, int q1, long long p0, long long P, int Cin, int Cout,
+                             const WgLinPlan &w, int splits, cudaStream_t s) {
     LinWgrad g{};
     g.im = im;
     g.Cin = Cin;
@@ -962,10 +962,11 @@ inline cudaError_t wgrad_lin(const __nv_bfloat16 *x, const __nv_bfloat16 *dy, fl
     g.spy = lin_stride(kWgK, w.bn / 8);
     g.per = w.per;
     g.splits = splits;
-    g.q0 = s0 * w.per;
-    g.q1 = (int)std::min<long long>(im.L, (long long)(s0 + splits) * w.per);
+    g.q0 = q0;
+    g.q1 = q1;
     g.bias_blocks = bpart ? w.bias_splits * (Cout / 8 / w.gw) : 0;
     g.gw = w.gw;
+    g.p0 = p0;
     g.P = P;
     g.bias_per = w.bias_per;
     g.bpart = bpart;

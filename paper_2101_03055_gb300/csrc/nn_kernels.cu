@@ -966,11 +966,38 @@ __global__ void __launch_bounds__(256) weight_sum_kernel(const float *__restrict
     }
 }
 
-// Images of one launch of the weight gradient: as many as keep the padded positions
-// below 2^30 (0: one image alone has more; the warp-level kernel takes it).
-int wgrad_images(int N, int H, int W) {
-    const long long one = ((long long)H + 1) * ((long long)W + 1);
-    return (int)std::min<long long>(N, ((1ll << 30) - 1) / one);
+// A part of the weight gradient's batch with fewer than 2^30 padded positions: n images of H rows
+// from pixel `first` on, of which the positions [q0, q1) and the pixels [p0, p0 + P) (of those
+// from `first` on) are summed.  Parts are runs of whole images, or bands of rows of one image
+// with the row above and below each band, which its taps read.
+struct WgradPart {
+    long long first;
+    int n, H, q0, q1;
+    long long p0, P;
+};
+// f(part) for every part, until one returns false; false also if three rows are too many
+// positions (W of some 2^28: the warp-level kernel takes those).
+template <class F>
+bool wgrad_parts(int N, int H, int W, const F &f) {
+    const long long row = (long long)W + 1, one = (H + 1ll) * row, most = (1ll << 30) - 1;
+    if (one <= most) {
+        const int images = (int)std::min<long long>(N, most / one);
+        for (int n0 = 0; n0 < N; n0 += images) {
+            const int n = std::min(images, N - n0);
+            if (!f(WgradPart{(long long)n0 * H * W, n, H, 0, (int)(n * one), 0, (long long)n * H * W})) return false;
+        }
+        return true;
+    }
+    const long long rows = most / row - 3;  // and a row above, one below and the padding row
+    if (rows < 1) return false;
+    for (int n = 0; n < N; ++n)
+        for (long long y0 = 0; y0 < H; y0 += rows) {
+            const int y1 = (int)std::min<long long>(H, y0 + rows), lo = (int)std::max(0ll, y0 - 1), hi = std::min(H, y1 + 1);
+            if (!f(WgradPart{((long long)n * H + lo) * W, 1, hi - lo, (int)((y0 - lo) * row), (int)((y1 - lo) * row),
+                             (y0 - lo) * W, (y1 - y0) * W}))
+                return false;
+        }
+    return true;
 }
 
 // ---------------------------------------------------------------------------
@@ -1461,15 +1488,12 @@ cdf_nn_status cdf_nn_conv3x3_bwd_data(const void *dy, const void *w, void *dx, i
 
 long long cdf_nn_conv3x3_bwd_weight_workspace(int N, int H, int W, int Cin, int Cout) {
     if (N < 1 || H < 1 || W < 1 || Cin < 16 || Cin % 16 || Cout < 32 || Cout % 32) return -1;
-    const int images = wgrad_images(N, H, W);
-    if (images == 0) return 4;  // the warp-level kernel adds to dw directly
-    // the largest of the launches: all images, or runs of `images` and a remainder with a tiling of its own
     long long most = 0;
-    for (int n : {images, N % images})
-        if (n > 0) {
-            const WgLinPlan w = wgrad_lin_plan((long long)n * (H + 1) * (W + 1), (long long)n * H * W, Cin, Cout);
-            most = std::max(most, wgrad_bytes(w, Cin, Cout));
-        }
+    if (!wgrad_parts(N, H, W, [&](const WgradPart &p) {
+            most = std::max(most, wgrad_bytes(wgrad_lin_plan(p.q1 - p.q0, p.P, Cin, Cout), Cin, Cout));
+            return true;
+        }))
+        return 4;  // the warp-level kernel adds to dw directly
     return most;
 }
 
@@ -1481,26 +1505,25 @@ cdf_nn_status cdf_nn_conv3x3_bwd_weight(const void *x, const void *dy, float *dw
     auto s = static_cast<cudaStream_t>(stream);
     const auto *xb = static_cast<const __nv_bfloat16 *>(x);
     const auto *dyb = static_cast<const __nv_bfloat16 *>(dy);
-    const int images = wgrad_images(N, H, W);
-    if (g_use_tc && images > 0) {
-        const long long need = cdf_nn_conv3x3_bwd_weight_workspace(N, H, W, Cin, Cout);
+    const long long need = g_use_tc ? cdf_nn_conv3x3_bwd_weight_workspace(N, H, W, Cin, Cout) : 4;
+    if (need > 4) {
         if (!workspace || workspace_bytes < need)
             return nn_fail("conv3x3_bwd_weight: the workspace is missing or smaller than "
                            "cdf_nn_conv3x3_bwd_weight_workspace()");
         float *part = static_cast<float *>(workspace);
-        for (int n0 = 0; n0 < N; n0 += images) {
-            const int n = std::min(images, N - n0);
-            const long long Pn = (long long)n * H * W;
-            const auto *xn = xb + (long long)n0 * H * W * Cin, *dyn = dyb + (long long)n0 * H * W * Cout;
+        cudaError_t e = cudaSuccess;
+        wgrad_parts(N, H, W, [&](const WgradPart &p) {
             LinImage im;
-            if (!lin_image(n, H, W, &im)) return nn_fail("conv3x3_bwd_weight: too many positions");
-            const WgLinPlan w = wgrad_lin_plan(im.L, Pn, Cin, Cout);
-            for (int s0 = 0; s0 < w.splits; s0 += w.run) {
+            if (!lin_image(p.n, p.H, W, &im)) e = cudaErrorInvalidValue;
+            const WgLinPlan w = wgrad_lin_plan(p.q1 - p.q0, p.P, Cin, Cout);
+            for (int s0 = 0; s0 < w.splits && e == cudaSuccess; s0 += w.run) {
                 const int splits = std::min(w.run, w.splits - s0);
                 // the bias gradient goes with the first launch, its partial sums behind the weights'
                 float *bpart = db && s0 == 0 ? part + (long long)w.run * 9 * Cin * Cout : nullptr;
-                const cudaError_t e = wgrad_lin(xn, dyn, part, bpart, im, Pn, Cin, Cout, w, s0, splits, s);
-                if (e != cudaSuccess) { cudaGetLastError(); return nn_fail(cudaGetErrorString(e)); }
+                e = wgrad_lin(xb + p.first * Cin, dyb + p.first * Cout, part, bpart, im, p.q0 + s0 * w.per,
+                              (int)std::min<long long>(p.q1, p.q0 + (long long)(s0 + splits) * w.per), p.p0, p.P, Cin,
+                              Cout, w, splits, s);
+                if (e != cudaSuccess) break;
                 const auto sum = [&](auto r) {
                     constexpr int R = decltype(r)::value;
                     const int n4 = 9 * Cin * Cout / 4, wblocks = (n4 + R - 1) / R;
@@ -1511,7 +1534,9 @@ cdf_nn_status cdf_nn_conv3x3_bwd_weight(const void *x, const void *dy, float *dw
                 if (splits >= 128) sum(std::integral_constant<int, 8>{});
                 else sum(std::integral_constant<int, 32>{});
             }
-        }
+            return e == cudaSuccess;
+        });
+        if (e != cudaSuccess) { cudaGetLastError(); return nn_fail(cudaGetErrorString(e)); }
     } else {
         // the warp-level MMA path: split-K partial sums added atomically (order-dependent)
         const long long per = 4096;

@@ -56,3 +56,47 @@ def test_several_launches(cdf, shape):
     from paper_2101_03055_gb300 import surrogate as S
     S.nn_lib()
     _check(S, torch, *shape, seed=sum(shape))
+
+
+@pytest.mark.parametrize("N,H,W", [(1, 33000, 33000), (3, 40000, 40000), (2, 5, 1 << 28)])
+def test_large_images_run_on_the_tensor_cores(N, H, W):
+    """An image of 2^30 positions and more goes in bands of rows; a workspace of 4 bytes would
+    mean the warp-level kernel."""
+    from paper_2101_03055_gb300 import surrogate
+    got = surrogate.nn_lib().cdf_nn_conv3x3_bwd_weight_workspace(N, H, W, 16, 32)
+    assert (got == 4) if W == 1 << 28 else 36 * 16 * 32 <= got <= BOUND
+
+
+@pytest.mark.gpu
+def test_bands_of_a_large_image(cdf):
+    """33000 x 33000 pixels, zero but for the first and last rows and those on either side of the
+    bands' edge: the sums of those rows."""
+    import torch
+    from paper_2101_03055_gb300 import surrogate as S
+    S.nn_lib()
+    H = W = 33000
+    if torch.cuda.mem_get_info()[0] < 130 << 30:
+        pytest.skip("needs 105 GB on the device")
+    edge = ((1 << 30) - 1) // (W + 1) - 3
+    rows = [*range(0, 3), *range(edge - 3, edge + 3), *range(H - 3, H)]
+    g = torch.Generator(device="cuda").manual_seed(5)
+    x = torch.zeros((1, H, W, 16), device="cuda", dtype=torch.bfloat16)
+    dy = torch.zeros((1, H, W, 32), device="cuda", dtype=torch.bfloat16)
+    for y in rows:
+        x[0, y] = torch.randn((W, 16), generator=g, device="cuda")
+        dy[0, y] = torch.randn((W, 32), generator=g, device="cuda")
+    dw, db = torch.zeros((32, 3, 3, 16), device="cuda"), torch.zeros(32, device="cuda")
+    S.conv3x3_bwd_weight(x, dy, dw, db)
+    want_w, want_b = torch.zeros((3, 3, 32, 16), device="cuda", dtype=torch.float64), 0
+    for y in rows:
+        d = dy[0, y].double()
+        want_b = want_b + d.sum(0)
+        for ky in range(3):
+            if 0 <= y + ky - 1 < H:
+                xp = torch.nn.functional.pad(x[0, y + ky - 1].double(), (0, 0, 1, 1))
+                for kx in range(3):
+                    want_w[ky, kx] += d.T @ xp[kx:kx + W]
+    want_w = want_w.permute(2, 0, 1, 3)
+    assert float((dw.double() - want_w).norm() / want_w.norm()) <= 1e-5
+    assert float((db.double() - want_b).norm() / want_b.norm()) <= 1e-5
+    assert S.tensor_error_flag() == 0
