@@ -891,8 +891,8 @@ __global__ void __launch_bounds__(kThreads) conv3x3_wgrad_kernel(const __nv_bflo
             const long long p = pk + kk;
             if (p < pend) {
                 const int n = (int)(p / ((long long)H * Wd));
-                const int rem = (int)(p - (long long)n * H * Wd);
-                const int yy = rem / Wd + dyy, xx = rem % Wd + dxx;
+                const unsigned rem = (unsigned)(p - (long long)n * H * Wd);  // (no device holds images of 2^32 pixels)
+                const int yy = (int)(rem / (unsigned)Wd) + dyy, xx = (int)(rem % (unsigned)Wd) + dxx;
                 if (yy >= 0 && yy < H && xx >= 0 && xx < Wd)
                     v = *reinterpret_cast<const uint4 *>(x + (((long long)n * H + yy) * Wd + xx) * Cin + ci0 + half);
             }
@@ -1539,11 +1539,12 @@ cdf_nn_status cdf_nn_conv3x3_bwd_weight(const void *x, const void *dy, float *dw
         if (e != cudaSuccess) { cudaGetLastError(); return nn_fail(cudaGetErrorString(e)); }
     } else {
         // the warp-level MMA path: split-K partial sums added atomically (order-dependent)
-        const long long per = 4096;
+        // (at most 65,535 splits, the layers of a grid)
+        const long long per = std::max(4096ll, ((P + 65534) / 65535 + kWBK - 1) / kWBK * kWBK);
         dim3 grid((unsigned)((Cout + kWBM - 1) / kWBM), 9 * (Cin / 16), (unsigned)((P + per - 1) / per));
         conv3x3_wgrad_kernel<<<grid, kThreads, 0, s>>>(xb, dyb, dw, N, H, W, Cin, Cout, per);
         if (db) {
-            dim3 g2(Cout / 8, (unsigned)((P + 256 * 64 - 1) / (256 * 64)));
+            dim3 g2(Cout / 8, (unsigned)std::min(65535ll, (P + 256 * 64 - 1) / (256 * 64)));
             bias_grad_kernel<<<g2, 256, 0, s>>>(dyb, db, P, Cout);
         }
     }

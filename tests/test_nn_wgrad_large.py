@@ -100,3 +100,31 @@ def test_bands_of_a_large_image(cdf):
     assert float((dw.double() - want_w).norm() / want_w.norm()) <= 1e-5
     assert float((db.double() - want_b).norm() / want_b.norm()) <= 1e-5
     assert S.tensor_error_flag() == 0
+
+
+@pytest.mark.gpu
+def test_warp_level_kernel_on_many_pixels(cdf):
+    """More pixels than 65,535 splits of 4096, zero but for a few rows."""
+    import torch
+    from paper_2101_03055_gb300 import surrogate as S
+    S.nn_lib()
+    H, W = 8200, 33000
+    if torch.cuda.mem_get_info()[0] < 40 << 30:
+        pytest.skip("needs 26 GB on the device")
+    g = torch.Generator(device="cuda").manual_seed(6)
+    x = torch.zeros((1, H, W, 16), device="cuda", dtype=torch.bfloat16)
+    dy = torch.zeros((1, H, W, 32), device="cuda", dtype=torch.bfloat16)
+    for y in (0, 4000, H - 1):
+        x[0, y] = torch.randn((W, 16), generator=g, device="cuda")
+        dy[0, y] = torch.randn((W, 32), generator=g, device="cuda")
+    got = []
+    for path in (1, 0):
+        dw, db = torch.zeros((32, 3, 3, 16), device="cuda"), torch.zeros(32, device="cuda")
+        S.set_tensor_path(path)
+        try:
+            S.conv3x3_bwd_weight(x, dy, dw, db)
+        finally:
+            S.set_tensor_path(True)
+        got.append((dw.double(), db.double()))
+    for a, b in zip(*got):  # both within 1e-5 of the exact sums
+        assert float((a - b).norm() / a.norm()) <= 2e-5
