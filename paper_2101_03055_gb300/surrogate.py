@@ -123,25 +123,22 @@ def conv3x3_bwd_data_relu(dy, w, y):
     return dx
 
 
-_workspace = {}
-
-
 @functools.lru_cache(maxsize=256)
 def _weight_workspace(N, H, W, Cin, Cout):
     return int(nn_lib().cdf_nn_conv3x3_bwd_weight_workspace(N, H, W, Cin, Cout))
 
 
-def conv3x3_bwd_weight(x, dy, dw, db):
-    """Accumulates the weight and bias gradients; the split partial sums go to a
-    device workspace kept per device (grown to the largest shape seen)."""
+def conv3x3_bwd_weight(x, dy, dw, db, workspace=None):
+    """Accumulates the weight and bias gradients; the split partial sums go to
+    `workspace` (float32, used on the current stream) if given and large enough, else to one of
+    this call's own: calls on several streams or threads never share a buffer."""
     import torch
     N, H, W, Cin = x.shape
     Cout = dy.shape[3]
     need = _weight_workspace(N, H, W, Cin, Cout)
-    ws = _workspace.get(x.device)
+    ws = workspace
     if ws is None or ws.numel() * 4 < need:
         ws = torch.empty((max(need, 4) + 3) // 4, dtype=torch.float32, device=x.device)
-        _workspace[x.device] = ws
     _call("cdf_nn_conv3x3_bwd_weight", _p(x), _p(dy), _p(dw), _p(db), N, H, W, Cin, Cout, _p(ws),
           ws.numel() * 4, _stream())
 
@@ -325,26 +322,34 @@ class UNet:
                 for (k, t), part in zip(self.master.items(), flat.split(sizes))}
 
     def backward(self, acts, dout):
+        import torch
         grads = self._zero_grads()
+        # one workspace for the pass's weight gradients, which follow each other on one stream
+        blocks = [f"d{L}" for L in range(self.levels - 1)] + [f"e{L}" for L in range(self.levels)]
+        need = 4
+        for b in blocks:
+            x, mid = acts[f"{b}.cat" if b[0] == "d" else f"{b}.in"].shape, acts[f"{b}a"].shape
+            need = max(need, _weight_workspace(*x, mid[3]), _weight_workspace(*mid, mid[3]))
+        ws = torch.empty((need + 3) // 4, dtype=torch.float32, device=dout.device)
         # dh: gradient of a block's output before its ReLU; dcat[L]: of the concatenation at level L
         dh = head_bwd_relu(acts["head.in"], self.master["head.w"], dout, grads["head.w"], grads["head.b"])
         dcat = [None] * self.levels
         for L in range(0, self.levels - 1):
-            dcat[L] = self._block_bwd(f"d{L}", acts[f"d{L}.cat"], acts, dh, grads)
+            dcat[L] = self._block_bwd(f"d{L}", acts[f"d{L}.cat"], acts, dh, grads, ws)
             below = f"d{L + 1}b" if L + 2 < self.levels else f"e{L + 1}b"
             dh = upsample2_bwd_relu(dcat[L], acts[below])
         for L in range(self.levels - 1, -1, -1):
-            dx = self._block_bwd(f"e{L}", acts[f"e{L}.in"], acts, dh, grads, need_dx=L > 0)
+            dx = self._block_bwd(f"e{L}", acts[f"e{L}.in"], acts, dh, grads, ws, need_dx=L > 0)
             if L > 0:
                 dh = pool_skip_bwd_relu(dx, dcat[L - 1], acts[f"e{L - 1}b"])
         return grads
 
-    def _block_bwd(self, name, x_in, acts, dh, grads, need_dx=True):
+    def _block_bwd(self, name, x_in, acts, dh, grads, ws, need_dx=True):
         """Weight gradients of a block's two convolutions and, if asked for, its input's gradient."""
         mid = acts[f"{name}a"]
-        conv3x3_bwd_weight(mid, dh, grads[f"{name}b.w"], grads[f"{name}b.b"])
+        conv3x3_bwd_weight(mid, dh, grads[f"{name}b.w"], grads[f"{name}b.b"], ws)
         d1 = conv3x3_bwd_data_relu(dh, self.bf16[f"{name}b.w"], mid)
-        conv3x3_bwd_weight(x_in, d1, grads[f"{name}a.w"], grads[f"{name}a.b"])
+        conv3x3_bwd_weight(x_in, d1, grads[f"{name}a.w"], grads[f"{name}a.b"], ws)
         return conv3x3_bwd_data(d1, self.bf16[f"{name}a.w"], x_in.shape[3]) if need_dx else None
 
     def adam_step(self, grads, lr):
