@@ -36,7 +36,7 @@ cdf_nn_status cdf_nn_conv3x3_bwd_data(const void *dy, const void *w, void *dx, i
 /* dw[co][t][ci] += sum_p dy[p][co] x[p + d(t)][ci] and db[co] += sum_p dy[p][co]
  * (FP32, accumulated: zero them first).  db may be NULL.  On the tensor-core path
  * the pixels are split over the GPU for dw and, separately, for db; each split's
- * partial sums go to `workspace` (device memory of at least
+ * partial sums go to `workspace` (device memory on a multiple of 16 bytes, of at least
  * cdf_nn_conv3x3_bwd_weight_workspace() bytes, owned by the caller, contents
  * overwritten; about 160 MB at most, or one split's sums, 36 Cin Cout bytes, where those are
  * more) and are added in a fixed order: the result is the same bits on

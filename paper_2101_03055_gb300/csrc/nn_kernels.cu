@@ -1510,6 +1510,9 @@ cdf_nn_status cdf_nn_conv3x3_bwd_weight(const void *x, const void *dy, float *dw
         if (!workspace || workspace_bytes < need)
             return nn_fail("conv3x3_bwd_weight: the workspace is missing or smaller than "
                            "cdf_nn_conv3x3_bwd_weight_workspace()");
+        // weight_sum_kernel reads it 16 bytes at a time
+        if (reinterpret_cast<uintptr_t>(workspace) & 15)
+            return nn_fail("conv3x3_bwd_weight: the workspace must begin on a multiple of 16 bytes");
         float *part = static_cast<float *>(workspace);
         cudaError_t e = cudaSuccess;
         wgrad_parts(N, H, W, [&](const WgradPart &p) {

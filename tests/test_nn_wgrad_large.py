@@ -128,3 +128,12 @@ def test_warp_level_kernel_on_many_pixels(cdf):
         got.append((dw.double(), db.double()))
     for a, b in zip(*got):  # both within 1e-5 of the exact sums
         assert float((a - b).norm() / a.norm()) <= 2e-5
+
+
+def test_workspace_off_16_bytes_is_refused():
+    """The check comes before any launch: the addresses here are never used."""
+    from paper_2101_03055_gb300 import surrogate as S
+    L = S.nn_lib()
+    for ws in (0x10004, 0x10008):
+        assert L.cdf_nn_conv3x3_bwd_weight(0x1000, 0x2000, 0x3000, None, 1, 8, 8, 16, 32, ws, 1 << 30, None) != 0
+        assert b"16 bytes" in L.cdf_nn_last_error()
