@@ -94,10 +94,12 @@ const char *cdf_nn_last_error(void);
  * 5th-generation tensor cores (tcgen05.mma, accumulators in tensor memory) without
  * im2col copies: the positions a tile reads are staged once with all input channels
  * and every tap's operand is the same rows seen through a shifted descriptor, for any
- * image size whose staged positions fit in shared memory (at 32 channels up to about
- * W = 1500, at 256 up to W = 140); wider images take the im2col staging that is faster
- * for the layer's depth -- three cp.async stage buffers when the GEMM input has at
- * least 128 channels, two buffers filled by ordinary loads below that;
+ * image size whose staged positions fit in shared memory and where that is the faster way
+ * (at 32 channels up to about W = 1200, at 256 up to W = 90); wider images take, forward with
+ * 16, 32 or 64 input channels and rows of whole 128-pixel tiles, the kernel that stages the three
+ * input rows of a tile, else the im2col staging that is faster for the layer's depth -- three
+ * cp.async stage buffers when the GEMM input has at least 128 channels, two buffers filled
+ * by ordinary loads below that;
  * 2: tcgen05 with the two-buffer im2col staging for every layer; 3: the forward pass
  * on a persistent warp-specialised im2col kernel, the backward pass on im2col staging;
  * 0: the warp-level MMA kernels.  The weight gradient runs on tcgen05 for 1 to 4 (an

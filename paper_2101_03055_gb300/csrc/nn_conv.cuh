@@ -715,19 +715,19 @@ constexpr int kMaxSmemCta = 222 * 1024;  // dynamic; the static arrays take the 
 template <class Plan>
 struct PlanCache {
     struct Entry {
-        long long key[6];
+        long long key[7];
         Plan plan;
         bool used = false;
     };
     Entry entry[64];
     template <class Make>
-    const Plan &get(const long long (&key)[6], const Make &make) {
+    const Plan &get(const long long (&key)[7], const Make &make) {
         unsigned long long h = 0;
         for (long long k : key) h = (h ^ (unsigned long long)k) * 0x9E3779B97F4A7C15ull;
         Entry &e = entry[h >> 58];
-        if (!e.used || !std::equal(key, key + 6, e.key)) {
+        if (!e.used || !std::equal(key, key + 7, e.key)) {
             e.plan = make();
-            std::copy(key, key + 6, e.key);
+            std::copy(key, key + 7, e.key);
             e.used = true;
         }
         return e.plan;
@@ -741,14 +741,37 @@ struct PlanCache {
 // operands' reads from shared memory, and 80 cycles a slice of all T tiles to issue)
 // and its stores; two slabs overlap the three inside a CTA, and so do the CTAs of an SM.
 // More positions per item stage less halo, fewer fill more SMs: a layer of 2592
-// positions takes T = 1 with narrow BN, one of a million T = 8 with two slabs.
+// positions takes T = 1 with narrow BN, one of a million T = 8 with two slabs.  On rows of 300
+// pixels and more the halo of two rows is most of what an item stages, and the copies of all CTAs of an SM
+// together count, 1.6 cycles each (1 x 4096 x 512, 16 -> 32: 123 -> 82 us).
 struct LinPlan {
     int bn = 0, t = 0, sp = 0, nbuf = 0, cols = 0, stages = 0, occ = 0;
     size_t smem = 0;
+    bool slower = false;  // than the kernel that takes the layer otherwise
 };
-inline LinPlan lin_plan(const LinImage &im, int Cin, int Cout, const DeviceShape &d) {
+// SM cycles of the kernels that take a layer when conv3x3_lin_kernel does not: a start, and per slice of
+// 16 channels of K the longer of one tile's own chain and the SM's rate times its tiles.
+// Fitted to 12 layers of 16-384 channels on images of 8 x 8 to 4096 x 512 (within 10 % on average).
+inline double staged_cycles(bool bwd, long long P, int W, int K, int M, int sms) {
+    const bool slab = !bwd && slab_shape(W, K, M), pipe = K >= 128;
+    int bn = M % 128 == 0 ? 128 : (M % 64 == 0 ? 64 : (M % 32 == 0 ? 32 : 16));
+    double chain, rate;
+    if (slab) {
+        bn = K == 64 ? std::min(bn, 64) : bn;
+        chain = rate = bn == 128 ? 560 : (bn == 64 ? 328 : 225);
+    } else if (!bwd) {
+        chain = bn == 128 ? (pipe ? 1340 : 2440) : (bn == 64 ? (pipe ? 1070 : 1880) : 1570);
+        rate = bn == 128 ? (pipe ? 800 : 1270) : (bn == 64 ? (pipe ? 600 : 800) : 580);
+    } else {
+        chain = bn == 128 ? 2500 : (bn == 64 ? (pipe ? 1630 : 2210) : (bn == 32 ? 1890 : 1220));
+        rate = bn == 128 ? 1480 : (bn == 64 ? (pipe ? 1020 : 1080) : (bn == 32 ? 650 : 450));
+    }
+    const double tiles = (double)((P + 127) / 128 * (M / bn));
+    return 12000 + 9.0 * K / 16 * std::max(chain, rate * std::ceil(tiles / sms));
+}
+inline LinPlan lin_plan(const LinImage &im, long long P, int Cin, int Cout, const DeviceShape &d, bool bwd) {
     LinPlan best;
-    double least = 1e30;
+    double least = 1e30, cycles = 0;
     const int G = Cin / 8, slices = 9 * Cin / 16, nst = (9 * Cin + kLinK - 1) / kLinK;
     for (int bn : {256, 128, 64, 32, 16}) {
         if (Cout % bn) continue;
@@ -770,14 +793,23 @@ inline LinPlan lin_plan(const LinImage &im, int Cin, int Cout, const DeviceShape
                 const double copy = slab / 16.0 + 1500, store = 800 + t * (100 + bn * 10.0);
                 const double mma = (double)slices * std::max(t * std::max(bn / 2.0, 32 + bn / 4.0), 80.0);
                 const double one = nbuf == 2 ? std::max({copy, mma, store}) : copy + mma + store;
-                const double time = copy + mma + store + (n - 1) * std::max(mma, one / std::min((double)occ, n));
+                const double copies = (double)G * count, wide = im.W >= 300 ? 1.6 * copies : 0;
+                const double apart = one / std::min((double)occ, n);
+                const double time = copy + mma + store + (n - 1) * std::max({mma, apart, wide});
                 if (time < least) {
                     least = time;
+                    // (the estimate that fits absolute times best; `time` ranks the plans)
+                    cycles = 10000 + std::max(1.13 * (copy + mma + store + (n - 1) * std::max(mma, apart)),
+                                              2.15 * n * copies);
                     best = LinPlan{bn, t, sp, nbuf, cols, stages, occ, smem};
                 }
             }
         }
     }
+    // The other kernel only where it is clearly ahead.  Of 855 layers and sizes measured 53 go there, all but four of them
+    // rightly (7 % slower at most).  Where rows get wide: 1 x 682 x 1536, 32 -> 32 takes 493 us here and 94 on the
+    // slab kernel, 1 x 697 x 752, 64 -> 64 1012 and 396 (im2col), 1 x 1024 x 128, 256 -> 256 1466 and 753.
+    best.slower = staged_cycles(bwd, P, im.W, Cin, Cout, d.sms) < 0.9 * cycles;
     return best;
 }
 
@@ -802,10 +834,10 @@ cudaError_t launch_conv_lin(const CUtensorMap &map, const __nv_bfloat16 *in, con
     return cudaGetLastError();
 }
 
-// Runs the layer on conv3x3_lin_kernel if it can (*ran).  It cannot where the
+// Runs the layer on conv3x3_lin_kernel if it can and pays (*ran).  It cannot where the
 // positions that one tile reads do not fit in shared memory with all input channels
-// (wide images with many channels, e.g. 384 channels from W = 114 on), for 2^30 positions and
-// more, and for weights off a 16-byte boundary (TMA); the staged im2col kernels take those.
+// (wide images with many channels, e.g. 384 channels from W = 71 on), for 2^30 positions and
+// more, and for weights off a 16-byte boundary (TMA).
 template <bool kBwd>
 cudaError_t conv_lin(const __nv_bfloat16 *in, const __nv_bfloat16 *w, const float *bias,
                      const __nv_bfloat16 *mask, __nv_bfloat16 *out, int N, int H, int W, int Cin, int Cout, int relu, cudaStream_t s, bool *ran) {
@@ -820,8 +852,10 @@ cudaError_t conv_lin(const __nv_bfloat16 *in, const __nv_bfloat16 *w, const floa
     g.boxk = Cin % 64 ? 32 : 64;
     g.relu = relu;
     thread_local PlanCache<LinPlan> plans;
-    const LinPlan pl = plans.get({g.im.L, W, Cin, Cout, d.sms, d.smem_sm}, [&] { return lin_plan(g.im, Cin, Cout, d); });
-    if (!pl.bn) return cudaSuccess;
+    const long long P = (long long)N * H * W;
+    const LinPlan pl = plans.get({g.im.L, P, W, Cin, Cout, d.sms, d.smem_sm},
+                                 [&] { return lin_plan(g.im, P, Cin, Cout, d, kBwd); });
+    if (!pl.bn || pl.slower) return cudaSuccess;
     g.dc = fast_div((uint32_t)Cin);
     g.T = pl.t;
     g.sp = pl.sp;
@@ -926,7 +960,7 @@ inline long long wgrad_bytes(const WgLinPlan &w, int Cin, int Cout) {
 
 inline WgLinPlan wgrad_lin_plan(long long L, long long P, int Cin, int Cout) {
     thread_local PlanCache<WgLinPlan> plans;
-    return plans.get({L, P, Cin, Cout, 0, 0}, [&] { return make_wgrad_lin_plan(L, P, Cin, Cout); });
+    return plans.get({L, P, Cin, Cout, 0, 0, 0}, [&] { return make_wgrad_lin_plan(L, P, Cin, Cout); });
 }
 
 template <int CI, int BN>
