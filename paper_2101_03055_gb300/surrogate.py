@@ -128,6 +128,13 @@ def _weight_workspace(N, H, W, Cin, Cout):
     return int(nn_lib().cdf_nn_conv3x3_bwd_weight_workspace(N, H, W, Cin, Cout))
 
 
+@functools.lru_cache(maxsize=256)
+def _pass_workspace(N, H, W, layers):
+    """The largest of a pass's layers (level, input channels, output channels), which follow
+    each other on one stream."""
+    return max(_weight_workspace(N, H >> L, W >> L, ci, co) for L, ci, co in layers)
+
+
 def conv3x3_bwd_weight(x, dy, dw, db, workspace=None):
     """Accumulates the weight and bias gradients; the split partial sums go to
     `workspace` (float32, used on the current stream) if given and large enough, else to one of
@@ -274,6 +281,7 @@ class UNet:
             shapes[f"d{L}b"] = (self.ch[L], self.ch[L])
         self.conv_names = list(shapes)
         self.shapes = shapes
+        self.layers = tuple((int(k[1:-1]), ci, co) for k, (co, ci) in shapes.items())
         self.master, self.bf16, self.m, self.v = {}, {}, {}, {}
         for name, (co, ci) in shapes.items():
             fan_in = 9 * ci
@@ -324,12 +332,8 @@ class UNet:
     def backward(self, acts, dout):
         import torch
         grads = self._zero_grads()
-        # one workspace for the pass's weight gradients, which follow each other on one stream
-        blocks = [f"d{L}" for L in range(self.levels - 1)] + [f"e{L}" for L in range(self.levels)]
-        need = 4
-        for b in blocks:
-            x, mid = acts[f"{b}.cat" if b[0] == "d" else f"{b}.in"].shape, acts[f"{b}a"].shape
-            need = max(need, _weight_workspace(*x, mid[3]), _weight_workspace(*mid, mid[3]))
+        N, H, W, _ = acts["e0.in"].shape
+        need = _pass_workspace(N, H, W, self.layers)
         ws = torch.empty((need + 3) // 4, dtype=torch.float32, device=dout.device)
         # dh: gradient of a block's output before its ReLU; dcat[L]: of the concatenation at level L
         dh = head_bwd_relu(acts["head.in"], self.master["head.w"], dout, grads["head.w"], grads["head.b"])
