@@ -5,6 +5,7 @@
 // channel copies for skip connections, 1x1 output head, MSE loss, Adam).
 // Activations are NHWC with the channel count a multiple of 16; 3x3 weights
 // are [Cout][3][3][Cin].
+#include <cooperative_groups.h>
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -1551,42 +1552,84 @@ __global__ void head_bwd_data_kernel(const float *__restrict__ dout, const float
     store_chan<V>(dx + (long long)i * V, r);
 }
 
-// dw[o][c] += sum_p dout[p][o] x[p][c]; db[o] += sum_p dout[p][o].  A warp takes 64
-// consecutive pixels (lane = channel, four outputs at a time), the block's eight
-// warps are added in shared memory, one atomic addition per block and weight.
-constexpr int kHeadRun = 64;
-__global__ void __launch_bounds__(256) head_bwd_weight_kernel(const __nv_bfloat16 *__restrict__ x,
-                                                              const float *__restrict__ dout,
-                                                              float *__restrict__ dw, float *__restrict__ db,
-                                                              long long P, int C, int O) {
-    __shared__ float red[8][5][32];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long p0 = ((long long)blockIdx.x * 8 + warp) * kHeadRun, p1 = min(P, p0 + kHeadRun);
-    for (int o0 = 0; o0 < O; o0 += 4)
-        for (int c0 = 0; c0 < C; c0 += 32) {
-            const int c = c0 + lane;
-            const bool bias = c0 == 0 && lane < min(4, O - o0);  // these lanes also add up dout
-            float s[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
-            for (long long p = p0; p < p1; ++p) {
-                const float xv = c < C ? __bfloat162float(x[p * C + c]) : 0.f;
+template <int N>
+using Int = std::integral_constant<int, N>;
+
+// dw[o][c] += sum_p dout[p][o] x[p][c]; db[o] += sum_p dout[p][o], for four outputs (blockIdx.y) and W
+// channels (blockIdx.z).  A warp adds up `run` pixels, 32 / W at a time (lane = channel, pixel),
+// in chains of 32 terms; the chains, the block's warps and the blocks of a cluster are added as
+// trees, the latter through distributed shared memory, and a cluster makes one atomic addition per weight.
+// run: at most 128, so that atomics come once in 8192 pixels, and less on small layers, down to four
+// pixels and about 16 clusters.  Bound by the loads of a warp's pixels, about five each.  Relative error against
+// 64 bits at 8192 pixels, 32 channels, five outputs: 1.1e-7; with 64-term chains and an atomic every 512 pixels
+// 1.4e-7, with one block per weight and 8192 pixels 1.0e-7.  Time with the input's gradient, in the same order:
+// 5.4, 19.5 and 4.9 us for 32 x 32 pixels (a launch with clusters costs about 1 us more), 22, 24 and 67 us for
+// 32 x 64 x 64.
+constexpr int kHeadRun = 128, kHeadCluster = 8;
+template <int W>
+__global__ void __cluster_dims__(kHeadCluster, 1, 1) __launch_bounds__(256)
+    head_bwd_weight_kernel(const __nv_bfloat16 *__restrict__ x, const float *__restrict__ dout, float *__restrict__ dw,
+                           float *__restrict__ db, long long P, int C, int O, int run) {
+    constexpr int S = 32 / W;  // pixels of a warp side by side
+    __shared__ float red[8][5][W], sum[5][W];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, sub = lane / W, cl = lane % W;
+    const int o0 = blockIdx.y * 4, c = blockIdx.z * W + cl, no = min(4, O - o0);
+    const long long p0 = ((long long)blockIdx.x * 8 + warp) * run, p1 = min(P, p0 + run);
+    // (lanes beyond the channels and, for the bias, beyond the outputs read valid places in vain)
+    const __nv_bfloat16 *xp = x + (p0 + sub) * C + min(c, C - 1);
+    const float *dp = dout + (p0 + sub) * O + o0;
+    const int bo = min(cl, no - 1);
+    float s[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+    const auto add = [&](auto outputs) {
+        constexpr int NO = decltype(outputs)::value;
+        for (long long q = p0; q < p1; q += 32 * S) {
+            float t[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+            const auto term = [&] {
+                const float xv = __bfloat162float(*xp);
 #pragma unroll
-                for (int o = 0; o < 4; ++o)
-                    if (o0 + o < O) s[o] += dout[p * O + o0 + o] * xv;
-                if (bias) s[4] += dout[p * O + o0 + lane];
+                for (int o = 0; o < NO; ++o) t[o] += dp[o] * xv;
+                t[4] += dp[bo];
+                xp += S * C;
+                dp += S * O;
+            };
+            if (q + 32 * S <= p1) {
+#pragma unroll 8
+                for (int j = 0; j < 32; ++j) term();
+            } else {
+                for (long long p = q + sub; p < p1; p += S) term();
             }
-            __syncthreads();
 #pragma unroll
-            for (int o = 0; o < 5; ++o) red[warp][o][lane] = s[o];
-            __syncthreads();
-            if (warp < 5) {
-                float t = 0.f;
-#pragma unroll
-                for (int k = 0; k < 8; ++k) t += red[k][warp][lane];
-                if (warp < 4 && o0 + warp < O && c < C) atomicAdd(dw + (o0 + warp) * C + c, t);
-                if (warp == 4 && bias) atomicAdd(db + o0 + lane, t);
-            }
+            for (int o = 0; o < 5; ++o) s[o] += t[o];
         }
+    };
+    if (no == 4) add(Int<4>{});
+    else if (no == 3) add(Int<3>{});
+    else if (no == 2) add(Int<2>{});
+    else add(Int<1>{});
+#pragma unroll
+    for (int d = W; d < 32; d *= 2)
+#pragma unroll
+        for (int o = 0; o < 5; ++o) s[o] += __shfl_xor_sync(0xffffffffu, s[o], d);
+    if (sub == 0)
+#pragma unroll
+        for (int o = 0; o < 5; ++o) red[warp][o][cl] = s[o];
+    __syncthreads();
+    const int i = threadIdx.x, o = i / W, k = i % W;  // a sum of this thread, o < 5
+    if (o < 5)
+        sum[o][k] = ((red[0][o][k] + red[1][o][k]) + (red[2][o][k] + red[3][o][k])) +
+                    ((red[4][o][k] + red[5][o][k]) + (red[6][o][k] + red[7][o][k]));
+    const auto cluster = cooperative_groups::this_cluster();
+    cluster.sync();
+    if (cluster.block_rank() == 0 && o < 5) {
+        float v[kHeadCluster];
+#pragma unroll
+        for (int r = 0; r < kHeadCluster; ++r) v[r] = *cluster.map_shared_rank(&sum[o][k], r);
+        const float t = ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
+        const int ck = blockIdx.z * W + k;
+        if (o < no && ck < C) atomicAdd(dw + (o0 + o) * C + ck, t);
+        if (o == 4 && blockIdx.z == 0 && k < no) atomicAdd(db + o0 + k, t);
+    }
+    cluster.sync();  // no block leaves while its sums are read
 }
 
 // Mean squared error over n values; loss (FP32 sum, one atomic addition per block of 2048 values) and
@@ -1645,8 +1688,6 @@ bool by_eight(std::initializer_list<long long> counts, std::initializer_list<con
     return true;
 }
 // f(Int<V>, index type) for n elements: 8 a thread and 32-bit indexes where possible.
-template <int N>
-using Int = std::integral_constant<int, N>;
 template <class F>
 void with_width(bool eight, long long n, const F &f) {
     if (eight && n < (1ll << 30)) f(Int<8>{}, 0);
@@ -1871,7 +1912,16 @@ static cdf_nn_status head_bwd(const void *x, const float *w, const float *dout, 
         head_bwd_data_kernel<V, decltype(index)><<<blocks_for(P * C / V), 256, 0, s>>>(
             dout, w, relu ? xb : nullptr, static_cast<__nv_bfloat16 *>(dx), P, C, O);
     });
-    head_bwd_weight_kernel<<<blocks_for(P, 8 * kHeadRun), 256, 0, s>>>(xb, dout, dw, db, P, C, O);
+    const auto weights = [&](auto width) {
+        constexpr int W = decltype(width)::value;
+        const int run = (int)std::min<long long>(kHeadRun, std::max(4ll, (P + 1023) / 1024));
+        const long long clusters = (P + 8 * kHeadCluster * run - 1) / (8 * kHeadCluster * run);
+        head_bwd_weight_kernel<W><<<dim3((unsigned)(clusters * kHeadCluster), (O + 3) / 4, (C + W - 1) / W), 256, 0, s>>>(
+            xb, dout, dw, db, P, C, O, run);
+    };
+    if (C <= 8) weights(Int<8>{});
+    else if (C <= 16) weights(Int<16>{});
+    else weights(Int<32>{});
     return launched();
 }
 
