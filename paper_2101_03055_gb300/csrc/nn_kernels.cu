@@ -1399,11 +1399,11 @@ __global__ void copy_channels_kernel(const __nv_bfloat16 *__restrict__ x, __nv_b
     const int c = (int)(i % G) * V;
     Chan<V> v = load_chan<V>(x + p * Cx + src_off + c);
     __nv_bfloat16 *const d = y + p * Cy + dst_off + c;
-    const Chan<V> old = accumulate ? load_chan<V>(d) : v;
+    if (accumulate) {
+        const Chan<V> old = load_chan<V>(d);
 #pragma unroll
-    for (int k = 0; k < V; ++k) {
-        const float f = __bfloat162float(v.e[k]);
-        v.e[k] = __float2bfloat16_rn(accumulate ? f + __bfloat162float(old.e[k]) : f);
+        for (int k = 0; k < V; ++k)
+            v.e[k] = __float2bfloat16_rn(__bfloat162float(v.e[k]) + __bfloat162float(old.e[k]));
     }
     store_chan<V>(d, v);
 }
@@ -1690,9 +1690,8 @@ bool by_eight(std::initializer_list<long long> counts, std::initializer_list<con
 // f(Int<V>, index type) for n elements: 8 a thread and 32-bit indexes where possible.
 template <class F>
 void with_width(bool eight, long long n, const F &f) {
-    if (eight && n < (1ll << 30)) f(Int<8>{}, 0);
-    else if (eight) f(Int<8>{}, 0ll);
-    else f(Int<1>{}, 0ll);
+    if (n < (1ll << 30)) eight ? f(Int<8>{}, 0) : f(Int<1>{}, 0);
+    else eight ? f(Int<8>{}, 0ll) : f(Int<1>{}, 0ll);
 }
 
 thread_local char g_nn_err[256] = "";
