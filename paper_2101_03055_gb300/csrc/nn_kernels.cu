@@ -1634,14 +1634,16 @@ __global__ void __cluster_dims__(kHeadCluster, 1, 1) __launch_bounds__(256)
     cluster.sync();  // no block leaves while its sums are read
 }
 
-// Mean squared error over n values; loss (FP32 sum, one atomic addition per block of 2048 values) and
-// its gradient 2 (pred - target) / n.
+// Mean squared error over n values; loss (FP32 sum, one atomic addition per block of 256 K values) and
+// its gradient 2 (pred - target) / n.  K: eight values a thread, fewer where the blocks would not fill the
+// chip.
+template <int K>
 __global__ void __launch_bounds__(256) mse_kernel(const float *__restrict__ pred, const float *__restrict__ target,
                                                   float *__restrict__ grad, float *__restrict__ loss, long long n) {
-    const long long i0 = (long long)blockIdx.x * 2048 + threadIdx.x;
+    const long long i0 = (long long)blockIdx.x * (256 * K) + threadIdx.x;
     float e = 0.f;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
+    for (int k = 0; k < K; ++k) {
         const long long i = i0 + 256 * k;
         if (i < n) {
             const float d = pred[i] - target[i];
@@ -2003,7 +2005,12 @@ cdf_nn_status cdf_nn_pool_skip_bwd_relu(const void *dp, const void *dcat, const 
 
 cdf_nn_status cdf_nn_mse(const float *pred, const float *target, float *grad, float *loss, long long n, void *stream) {
     if (!pred || !target || !grad || !loss) return nn_fail("mse: NULL argument");
-    mse_kernel<<<blocks_for(n, 2048), 256, 0, static_cast<cudaStream_t>(stream)>>>(pred, target, grad, loss, n);
+    const auto run = [&](auto values) {
+        constexpr int K = decltype(values)::value;
+        mse_kernel<K><<<blocks_for(n, 256 * K), 256, 0, static_cast<cudaStream_t>(stream)>>>(pred, target, grad, loss, n);
+    };
+    if (n <= 256 * 152) run(Int<1>{});
+    else run(Int<8>{});
     return launched();
 }
 

@@ -72,3 +72,22 @@ def test_head_fwd_on_odd_channels_is_not_slower(S):
         x, w, b = rand(torch, 1, 64, 64, C).to(torch.bfloat16), rand(torch, 5, C), rand(torch, 5)
         t.append(seconds(torch, lambda: sur.head_fwd(x, w, b)))
     assert t[0] <= 1.2 * t[1]
+
+
+@pytest.mark.parametrize("n", [1, 255, 257, 5120, 38912, 38913, 40959, 100001])
+def test_mse(S, n):
+    """The gradient bit for bit; the loss within its FP32 rounding: three roundings a term and chains
+    below 300 additions of positive terms."""
+    sur, torch = S
+    p, t = rand(torch, 2, n)
+    loss, grad = sur.mse(p, t)
+    want = ((p.double() - t.double()) ** 2).mean()
+    assert torch.equal(grad, 2.0 * (p - t) / n)
+    assert abs(float(loss) / float(want) - 1) <= 303 * 2.0 ** -24
+
+
+def test_mse_of_few_values_fills_the_chip(S):
+    """5120 values, eight a thread, took 1.9 times the time of 64."""
+    sur, torch = S
+    a, b = rand(torch, 5120), rand(torch, 64)
+    assert seconds(torch, lambda: sur.mse(a, a)) <= 1.5 * seconds(torch, lambda: sur.mse(b, b))
