@@ -82,7 +82,7 @@ def test_mse(S, n):
     p, t = rand(torch, 2, n)
     loss, grad = sur.mse(p, t)
     want = ((p.double() - t.double()) ** 2).mean()
-    assert torch.equal(grad, 2.0 * (p - t) / n)
+    assert torch.equal(grad, 2.0 * (p - t) / torch.full_like(p, n))  # (by a tensor: an IEEE quotient)
     assert abs(float(loss) / float(want) - 1) <= 303 * 2.0 ** -24
 
 
