@@ -494,7 +494,9 @@ struct ModeChoice {
 std::map<TuneKey, ModeChoice> g_bmode;
 
 cdf_status bautotune(cdf_batch *b) {
-    TuneKey key{b->nodes, (long long)b->count, b->m, b->params[0].chemotaxis};
+    // what decides which kernels run belongs to the key: the closure kind and the two-step tiling
+    const int kernels = 2 * (2 * (b->kind + 1) + (fused_fits(b) ? 1 : 0)) + b->params[0].chemotaxis;
+    TuneKey key{b->nodes, (long long)b->count, b->m, kernels};
     {
         std::lock_guard<std::mutex> lk(g_btune_mu);
         auto it = g_bmode.find(key);

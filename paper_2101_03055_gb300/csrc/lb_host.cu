@@ -97,6 +97,9 @@ bool positive_definite(int n, const double *s) {
 
 size_t elem_size(int storage) { return storage == CDF_FP32 ? 4 : 2; }
 
+// The closure's part of a tuner's key: each closure kind has kernels of its own, and within those for
+// any closure chemotaxis decides what runs.
+int closure_key(const LbParams &p) { return 2 * (batch_closure_kind(&p, 1) + 1) + p.chemotaxis; }
 using TuneKey = std::tuple<int, int, int, int, int>;
 std::mutex g_tune_mu;
 std::map<TuneKey, dim3> g_tune_cache;
@@ -378,11 +381,11 @@ void drop_graphs(cdf_lb *h) {
 }
 
 // Time the step kernel for a few CTA shapes on the (zeroed) buffers and keep the
-// fastest; results are cached per (nx, ny, m, storage).  The shapes are timed
+// fastest; results are cached per (nx, ny, m, storage, closure).  The shapes are timed
 // through the path the steps run in (CUDA graphs of 32 launches): a short step
 // launched one by one from the host would time the host's launch rate.
 cdf_status autotune(cdf_lb *h) {
-    TuneKey key{h->nx, h->ny, h->m, h->storage * 2 + h->P.case1, h->P.chemotaxis};
+    TuneKey key{h->nx, h->ny, h->m, h->storage * 2 + h->P.case1, closure_key(h->P)};
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         auto it = g_tune_cache.find(key);
@@ -459,7 +462,7 @@ cdf_status setup_pair(cdf_lb *h, const cdf_options *opt) {
         h->pair_th = opt->temporal_tile_y;
         return CDF_OK;
     }
-    PairKey key{h->nx, h->ny, (h->m * 4 + h->storage) * 2 + h->P.case1, h->P.chemotaxis, h->P.periodic_x,
+    PairKey key{h->nx, h->ny, (h->m * 4 + h->storage) * 2 + h->P.case1, closure_key(h->P), h->P.periodic_x,
                 h->P.periodic_y};
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
@@ -564,7 +567,7 @@ cdf_status setup_resident(cdf_lb *h, const cdf_options *opt) {
     if (st != CDF_OK || opt->resident == 1) return st;
     // opt->resident == 0: keep the faster mode (the tuner runs on the zeroed
     // buffers; the state is set by the init calls afterwards)
-    TuneKey key{h->nx, h->ny, h->m, h->storage * 2 + h->P.case1, h->P.chemotaxis};
+    TuneKey key{h->nx, h->ny, h->m, h->storage * 2 + h->P.case1, closure_key(h->P)};
     bool use = false;
     bool cached = false;
     {
