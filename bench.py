@@ -361,19 +361,8 @@ class _Batch:
                            f"CTAs of {info.chain_block_x}x{info.chain_block_y}, output tiles "
                            f"{info.chain_block_x - 2}x{info.chain_tile_y}; graph of 32 steps over a 32-stream pool)")
         else:
-            # instances in the groups of one launch: a multiple of four groups of about 20 MiB of populations
-            # (both buffers), at most 64 instances each
-            size = [8 * (9 + 5 * pb.m + (info.bytes_per_lup > 8 * (9 + 5 * pb.m))) * ((pb.nx + 31) // 32 * 32) * pb.ny
-                    for pb in pbs]
-            want = (sum(size) // (20 << 20) + 4) // 4 * 4
-            before, last, run, self.groups = 0, 0, 0, 1
-            for k, b in enumerate(size):
-                g = int((before + 0.5 * b) / sum(size) * want)
-                if k and (g != last or run == 64):
-                    self.groups, run = self.groups + 1, 0
-                before, last, run = before + b, g, run + 1
             self.kernel = (f"step2_batch_kernel<{self.m}> (two time steps of a group of instances per launch, "
-                           f"{self.groups} groups; graph of 32 steps over 4 streams)")
+                           f"{self.s.launches(2)} groups; graph of 32 steps over 4 streams)")
         self.mode = info.mode
         self.count = info.count
 
@@ -388,11 +377,7 @@ class _Batch:
         return 2 if (self.mode != 1 and n >= 2) else 1
 
     def launches(self, n):
-        if self.mode == 1:
-            return n * self.count
-        if self.mode == 2:
-            return (n // 2 + n % 2) * self.count
-        return n // 2 * self.groups + n % 2
+        return self.s.launches(n)
 
     stream = property(lambda self: self.s.stream)
 

@@ -350,10 +350,11 @@ void cdf_split_destroy(cdf_split *s);
 
 /* ---- batched solver --------------------------------------------------------
  * Many independent lattices of uneven size (a parameter sweep) advanced together,
- * in one of two modes chosen by measurement: a persistent kernel that schedules
+ * in one of three modes chosen by measurement: whole-batch launches of two steps (where a
+ * periodic axis is shorter than 6 nodes instead a persistent kernel that schedules
  * (instance, tile) units with a bounded grid barrier between the time steps of
- * a launch, or one CUDA graph of per-instance chains of step kernels fanned out
- * over a stream pool (the instances are independent, so the chains need no
+ * a launch), or one CUDA graph of per-instance chains of one-step or of two-step kernels fanned
+ * out over a stream pool (the instances are independent, so the chains need no
  * barrier).  Each instance
  * is the model of cdf_lb_create (same equations, same boundary rules) with its
  * own grid, D, nu, S, F and boundaries; all share m, the source kind and FP32
@@ -364,7 +365,8 @@ typedef struct {
     double rho0;
     void *cuda_stream;           /* caller's stream, NULL = legacy default */
     int tile_x, tile_y;          /* tile shape (nodes); 0 = autotuned */
-    int steps_per_launch;        /* time steps per persistent launch; 0 = 32 */
+    int steps_per_launch;        /* time steps per launch of the persistent kernel; 0 = 32 (the other
+                                    kernels ignore it) */
     double barrier_timeout_s;    /* bound of every grid-barrier wait; 0 = 1 s */
     int test_unreachable_barrier;/* test hook: the barrier expects one block more than runs,
                                     so every wait runs out and cdf_batch_step returns CDF_ETIMEOUT */
@@ -385,6 +387,9 @@ typedef struct {
     int count, m;
     long long nodes, tiles;
     int tile_x, tile_y, grid_blocks, steps_per_launch;
+                                 /* (tiles to here: of the persistent kernel, in mode 0 of an odd last
+                                    step where the two-step launches run, which cut every lattice
+                                    into tiles of its own size) */
     double bytes_per_lup;
     long long t;
     int mode;                    /* 0 whole-batch kernels, 1 graph of per-instance chains,
@@ -425,6 +430,10 @@ cdf_status cdf_batch_moments_device(cdf_batch *b, int k, float *dev_out);
 cdf_status cdf_batch_snapshot(cdf_batch *b);
 cdf_status cdf_batch_residuals(cdf_batch *b, double *residual);
 cdf_status cdf_batch_get_info(const cdf_batch *b, cdf_batch_info *out);
+/* Kernel launches of cdf_batch_step(b, n): with the two-step launches of mode 0 one for every
+ * two steps and group of instances, and one for an odd step; with the persistent kernel
+ * one for every steps_per_launch steps; with chains one for every instance and step or two. */
+long long cdf_batch_launches(const cdf_batch *b, long long n);
 void *cdf_batch_stream(const cdf_batch *b);
 void cdf_batch_destroy(cdf_batch *b);
 

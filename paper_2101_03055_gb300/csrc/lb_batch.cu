@@ -853,6 +853,14 @@ cdf_status cdf_batch_get_info(const cdf_batch *b, cdf_batch_info *out) {
     return CDF_OK;
 }
 
+long long cdf_batch_launches(const cdf_batch *b, long long n) {
+    if (!b || n < 0) return -1;
+    if (b->mode == 1) return n * b->count;
+    if (b->mode == 2) return (n / 2 + n % 2) * b->count;
+    if (b->fused) return n / 2 * ((long long)b->group_start.size() - 1) + n % 2;
+    return (n + b->steps_per_launch - 1) / b->steps_per_launch;
+}
+
 cdf_status cdf_batch_snapshot(cdf_batch *b) {
     if (!b) return bfail(CDF_EINVAL, "NULL handle");
     BCK(cudaEventRecord(b->ev_in, b->user));

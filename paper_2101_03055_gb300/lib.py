@@ -180,6 +180,7 @@ SIGNATURES = {
     "cdf_batch_init_moments_device": (ctypes.c_int, [_H, ctypes.c_int, _FP]),
     "cdf_batch_moments_device": (ctypes.c_int, [_H, ctypes.c_int, _FP]),
     "cdf_batch_get_info": (ctypes.c_int, [_H, ctypes.POINTER(cdf_batch_info)]),
+    "cdf_batch_launches": (ctypes.c_longlong, [_H, ctypes.c_longlong]),
     "cdf_batch_snapshot": (ctypes.c_int, [_H]),
     "cdf_batch_residuals": (ctypes.c_int, [_H, _DP]),
     "cdf_batch_stream": (ctypes.c_void_p, [_H]),
@@ -653,6 +654,10 @@ def cdf_batch_get_info(h) -> cdf_batch_info:
     return info
 
 
+def cdf_batch_launches(h, n: int) -> int:
+    return load().cdf_batch_launches(h, n)
+
+
 def cdf_batch_stream(h) -> int:
     return load().cdf_batch_stream(h) or 0
 
@@ -747,6 +752,10 @@ class BatchSolver:
 
     def info(self) -> cdf_batch_info:
         return cdf_batch_get_info(self.h)
+
+    def launches(self, n: int) -> int:
+        """Kernel launches of step(n)."""
+        return cdf_batch_launches(self.h, n)
 
     def residuals_after(self, n: int) -> np.ndarray:
         """Advance n steps and return each instance's residual over those steps."""
