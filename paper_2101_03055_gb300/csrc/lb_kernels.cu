@@ -88,6 +88,16 @@ int closure_kind(const LbParams &p) {
 // Case 1 has no force: its kernels exist for the plain kind and for any closure.
 constexpr int case1_kind(int kind) { return kind == kKindPlain ? kKindPlain : kAnyClosure; }
 
+// Does one FP32 step per launch run the forced and the plume kind on their own kernels?  Where both buffers lie
+// well inside the L2 (100 of 126 MB): from there on the kernels for any closure reach the memory's rate,
+// theirs do not (1024 x 1024 cavity 25.2 us a step against 26.8, plume 26.2 against 27.7).  The forced kind's also
+// lose where a lattice is about one wave, bound by latency: 96 x 96 nodes 1.9 against 2.5 us,
+// 512 x 256 3.8 against 4.05, even at 192,000 nodes, 640 x 480 6.5 against 6.45.
+bool one_step_kind_pays(const LbParams &p) {
+    const long long nodes = (long long)p.nx * p.ny;
+    return nodes * 8 * 19 < (100ll << 20) && (closure_kind(p) != kKindForced || nodes >= 250000);
+}
+
 // 16-bit storage keeps no reference gradient.
 constexpr int mr_kind(int kind) { return kind < 0 ? kind : (kind & ~kShift); }
 
@@ -1341,6 +1351,9 @@ cudaError_t step_dispatch(const LbParams &p, const void *in, void *out, const fl
         dim3 fb(block.x), grid((unsigned)((n + block.x - 1) / block.x));
         const cudaError_t e = for_model(p, [&](auto m, auto kind) {
             constexpr int M = decltype(m)::value, K = decltype(kind)::value;
+            if constexpr (K == kKindForced || K == kKindPlume)
+                if (!one_step_kind_pays(p))
+                    return launch_pdl(step_kernel_flat<M, T, kAnyClosure>, grid, fb, s, p, pl, sp_in, sp_out, mom);
             return launch_pdl(step_kernel_flat<M, T, K>, grid, fb, s, p, pl, sp_in, sp_out, mom);
         });
         return e != cudaSuccess ? e : cudaGetLastError();
@@ -1348,6 +1361,9 @@ cudaError_t step_dispatch(const LbParams &p, const void *in, void *out, const fl
     dim3 grid((p.nx + block.x - 1) / block.x, (p.ny + block.y - 1) / block.y);
     const cudaError_t e = for_model(p, [&](auto m, auto kind) {
         constexpr int M = decltype(m)::value, K = decltype(kind)::value;
+        if constexpr (K == kKindForced || K == kKindPlume)
+            if (!one_step_kind_pays(p))
+                return launch_pdl(step_kernel<M, T, kAnyClosure>, grid, block, s, p, pl, sp_in, sp_out, mom);
         return launch_pdl(step_kernel<M, T, K>, grid, block, s, p, pl, sp_in, sp_out, mom);
     });
     return e != cudaSuccess ? e : cudaGetLastError();
