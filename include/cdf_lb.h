@@ -371,8 +371,10 @@ typedef struct {
     int test_unreachable_barrier;/* test hook: the barrier expects one block more than runs,
                                     so every wait runs out and cdf_batch_step returns CDF_ETIMEOUT */
     int mode;                    /* with tile_x > 0: 0 = whole-batch kernels: two steps of all instances
-                                    per launch (every periodic axis at least 6 nodes long), else (and
-                                    with the test hook) the persistent kernel with this tile shape,
+                                    per launch (every periodic axis at least 6 nodes long, and where
+                                    that is the faster one: thin lattices and three or four scalars
+                                    are timed), else (and with the test hook) the persistent kernel
+                                    with this tile shape,
                                     1 = graph of per-instance kernel chains (tile = CTA shape),
                                     2 = the same chains of two-step launches (step2_kernel of
                                     cdf_options.temporal; tile = its CTA shape, tile_x 32 or 64);

@@ -131,9 +131,8 @@ cdf_status bfail(cdf_status st, const char *msg) {
         }                                                                             \
     } while (0)
 
-using TuneKey = std::tuple<long long, long long, int, int>;
+using TuneKey = std::tuple<long long, long long, int, int, int>;
 std::mutex g_btune_mu;
-std::map<TuneKey, dim3> g_btune;
 
 }  // namespace
 }  // namespace cdflb
@@ -463,13 +462,30 @@ bool chain_pair_fits(const cdf_batch *b, dim3 blk, int th) {
     return true;
 }
 
-// Two steps of all instances per launch: wherever every instance has a tiling (not with
-// the barrier's test hook), it is faster than the persistent kernel, which moves twice the bytes.
+// Can two steps of all instances run in a launch: every instance has a tiling (and the barrier's
+// test hook is off)?
 bool fused_fits(const cdf_batch *b) {
     int tw, th;
     for (const LbParams &p : b->params)
         if (!pair_tile(p, tile_nodes(b->nodes), &tw, &th) || (9 + 5 * b->m) * p.plane >= (1ll << 31)) return false;
     return !b->extra_arrivals;
+}
+
+// Are the two-step launches surely faster than the persistent kernel, which moves twice the bytes?  With one or
+// two scalars and tiles of 96 nodes and more, their ring included, on average they were on every
+// batch measured.  Thin lattices leave most of a CTA's eight warps idle, and three and four scalars let fewer CTAs
+// on an SM: 500 lattices of 2000 x 1 take 83 us a step (two scalars) against 37, 1500 of 7 x 7 17.5 against 16.3, 166
+// of 2000 x 3 with three scalars 67 against 47, but 166 of 3 x 2000 with four 185 against 716.  Those are timed.
+bool fused_surely(const cdf_batch *b) {
+    double nodes = 0, tiles = 0;
+    for (const LbParams &p : b->params) {
+        int tw = 1, th = 1;
+        pair_tile(p, tile_nodes(b->nodes), &tw, &th);
+        const double tx = (p.nx + tw - 1) / tw, ty = (p.ny + th - 1) / th;
+        nodes += (p.nx + 2 * (tx - 1) + 2 * p.periodic_x) * (p.ny + 2 * (ty - 1) + 2 * p.periodic_y);
+        tiles += tx * ty;
+    }
+    return b->m <= 2 && nodes >= 96 * tiles;
 }
 
 cdf_status check_err(cdf_batch *b) {
@@ -490,13 +506,78 @@ struct ModeChoice {
     int mode;
     dim3 shape;
     int th;
+    bool fused;  // mode 0: the two-step launches
 };
 std::map<TuneKey, ModeChoice> g_bmode;
+std::map<std::tuple<TuneKey, unsigned, unsigned>, bool> g_bfused;  // mode 0 with a given tile
+
+// what decides which kernels run and how well belongs to the key: the closure kind, the two-step tiling
+TuneKey tune_key(const cdf_batch *b) {
+    const int kernels = 2 * (2 * (b->kind + 1) + (fused_fits(b) ? 1 : 0)) + b->params[0].chemotaxis;
+    long long rows = 0;
+    for (const LbParams &p : b->params) rows += 3ll * p.ny + p.periodic_x + (p.periodic_y ? 1ll << 40 : 0);
+    return TuneKey{b->nodes, rows, b->count, b->m, kernels};
+}
+
+// Milliseconds of run(nsteps) after a warm-up (and graph capture), the least of up to four where they are short
+// enough for the host to disturb, or -1.
+template <class Run>
+float time_batch(cdf_batch *b, int nsteps, const Run &run) {
+    cudaEvent_t e[2] = {nullptr, nullptr};
+    bool ok = cudaEventCreate(&e[0]) == cudaSuccess && cudaEventCreate(&e[1]) == cudaSuccess && run(nsteps) == CDF_OK;
+    float least = 1e30f, all = 0;
+    for (int r = 0; ok && r < 4 && all < 1.f; ++r) {
+        float ms = 0;
+        ok = cudaEventRecord(e[0], b->s) == cudaSuccess && run(nsteps) == CDF_OK &&
+             cudaEventRecord(e[1], b->s) == cudaSuccess && cudaEventSynchronize(e[1]) == cudaSuccess &&
+             check_err(b) == CDF_OK && cudaEventElapsedTime(&ms, e[0], e[1]) == cudaSuccess;
+        least = std::min(least, ms);
+        all += ms;
+    }
+    for (cudaEvent_t ev : e)
+        if (ev) cudaEventDestroy(ev);
+    return ok ? least : -1.f;
+}
+// The same of 32 steps of the whole-batch kernel that b->fused names, with the tile that is set up.
+float time_whole(cdf_batch *b) {
+    if (b->fused) return time_batch(b, kChainGraphSteps, [&](int n) { return run_chains(b, n, false); });
+    const int steps = b->nodes > (1 << 22) ? 4 : 16;
+    const float ms = time_batch(b, steps, [&](int n) { return launch_batch(b, n, false); });
+    return ms * ((float)kChainGraphSteps / steps);
+}
+
+// Mode 0 with a given tile: the two-step launches, or the persistent kernel with this tile where
+// those are not surely and not measurably faster.
+cdf_status setup_whole(cdf_batch *b, dim3 tile) {
+    b->fused = fused_fits(b);
+    cdf_status st = setup_tiles(b, tile);
+    if (st != CDF_OK || !b->fused || fused_surely(b)) return st;
+    const auto key = std::make_tuple(tune_key(b), tile.x, tile.y);
+    {
+        std::lock_guard<std::mutex> lk(g_btune_mu);
+        const auto it = g_bfused.find(key);
+        if (it != g_bfused.end()) {
+            b->fused = it->second;
+            return CDF_OK;
+        }
+    }
+    float ms[2];
+    for (int f = 1; f >= 0; --f) {
+        b->fused = f;
+        ms[f] = time_whole(b);
+        set_chain_block(b, b->chain_block);  // drops the captured launches
+        b->cur = 0;
+        b->t = 0;
+        if (ms[f] < 0) return bfail(CDF_ECUDA, "timing the whole-batch kernels failed");
+    }
+    b->fused = ms[1] < ms[0];
+    std::lock_guard<std::mutex> lk(g_btune_mu);
+    g_bfused[key] = b->fused;
+    return CDF_OK;
+}
 
 cdf_status bautotune(cdf_batch *b) {
-    // what decides which kernels run belongs to the key: the closure kind and the two-step tiling
-    const int kernels = 2 * (2 * (b->kind + 1) + (fused_fits(b) ? 1 : 0)) + b->params[0].chemotaxis;
-    TuneKey key{b->nodes, (long long)b->count, b->m, kernels};
+    const TuneKey key = tune_key(b);
     {
         std::lock_guard<std::mutex> lk(g_btune_mu);
         auto it = g_bmode.find(key);
@@ -507,54 +588,45 @@ cdf_status bautotune(cdf_batch *b) {
                 b->chain_th = it->second.th;
                 return setup_tiles(b, dim3(64, 4));
             }
-            b->fused = fused_fits(b);
+            b->fused = it->second.fused;
             return setup_tiles(b, it->second.shape);
         }
     }
-    cudaEvent_t e0, e1;
-    BCK(cudaEventCreate(&e0));
-    BCK(cudaEventCreate(&e1));
     float best = 1e30f;
-    ModeChoice choice{0, dim3(64, 4), 0};
-    const int steps = b->nodes > (1 << 22) ? 4 : 16;
-    auto time_it = [&](auto &&run, int nsteps) -> float {
-        if (run(nsteps) != CDF_OK) return -1.f;  // warm-up (and graph capture)
-        if (cudaEventRecord(e0, b->s) != cudaSuccess) return -1.f;
-        if (run(nsteps) != CDF_OK) return -1.f;
-        if (cudaEventRecord(e1, b->s) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess) return -1.f;
-        if (check_err(b) != CDF_OK) return -1.f;
-        float ms = 0;
-        cudaEventElapsedTime(&ms, e0, e1);
-        return ms;
-    };
+    ModeChoice choice{0, dim3(64, 4), 0, false};
     const dim3 tiles[] = {dim3(64, 4), dim3(32, 4), dim3(32, 8), dim3(64, 2), dim3(128, 1), dim3(128, 2),
                           dim3(256, 1)};
     b->mode = 0;
-    b->fused = fused_fits(b);
-    for (const dim3 &c : tiles) {
-        cdf_status st = setup_tiles(b, c);
+    const bool fits = fused_fits(b), surely = fits && fused_surely(b);
+    if (fits) {  // (the tile shape matters to the persistent kernel only)
+        b->fused = true;
+        cdf_status st = setup_tiles(b, tiles[0]);
         if (st != CDF_OK) return st;
-        float ms;
-        if (b->fused) {
-            ms = time_it([&](int n) { return run_chains(b, n, false); }, kChainGraphSteps);
-        } else {
-            ms = time_it([&](int n) { return launch_batch(b, n, false); }, steps);
-            if (ms >= 0) ms *= (float)kChainGraphSteps / steps;  // per 32 steps, comparable with the chains
-        }
-        if (ms < 0) return bfail(CDF_ECUDA, "autotuning the whole-batch kernels failed");
-        if (ms < best) { best = ms; choice = {0, c, 0}; }
-        if (b->fused) break;  // the tile shape matters to the persistent kernel only
+        best = time_whole(b);
+        if (best < 0) return bfail(CDF_ECUDA, "autotuning the whole-batch kernels failed");
+        choice = {0, tiles[0], 0, true};
     }
     b->fused = false;
     set_chain_block(b, b->chain_block);  // drops the captured launches
+    b->cur = 0;  // (the persistent kernel has one S(t - 1) for both parities)
+    if (!surely)
+        for (const dim3 &c : tiles) {
+            cdf_status st = setup_tiles(b, c);
+            if (st != CDF_OK) return st;
+            const float ms = time_whole(b);
+            if (ms < 0) return bfail(CDF_ECUDA, "autotuning the whole-batch kernels failed");
+            if (ms < best) { best = ms; choice = {0, c, 0, false}; }
+        }
+    // (chains have to be 5 % ahead of the two-step launches: their graphs of a branch per instance cost a
+    // call more; 20 lattices of 64 x 64 take 3.8 us a step as chains, 3.6 in two-step launches)
     const dim3 blocks[] = {dim3(128, 1), dim3(128, 2), dim3(256, 1), dim3(64, 4), dim3(32, 8), dim3(128, 0),
                            dim3(256, 0)};  // y == 0: flat launch
     b->mode = 1;
     for (const dim3 &c : blocks) {
         set_chain_block(b, c);
-        float ms = time_it([&](int n) { return run_chains(b, n, false); }, kChainGraphSteps);
+        const float ms = time_batch(b, kChainGraphSteps, [&](int n) { return run_chains(b, n, false); });
         if (ms < 0) return bfail(CDF_ECUDA, "autotuning the kernel chains failed");
-        if (ms < best) { best = ms; choice = {1, c, 0}; }
+        if (ms < best * (choice.fused ? 0.95f : 1.f)) { best = ms; choice = {1, c, 0, false}; }
     }
     // chains of two-step launches: CTA shape and tile height (the paired-lane
     // kernel, chain_lanes = 2, measured slower on GB300 and is not timed here)
@@ -565,12 +637,10 @@ cdf_status bautotune(cdf_batch *b) {
         if (!chain_pair_fits(b, c.first, c.second)) continue;
         set_chain_block(b, c.first);
         b->chain_th = c.second;
-        float ms = time_it([&](int n) { return run_chains(b, n, false); }, kChainGraphSteps);
+        const float ms = time_batch(b, kChainGraphSteps, [&](int n) { return run_chains(b, n, false); });
         if (ms < 0) return bfail(CDF_ECUDA, "autotuning the two-step kernel chains failed");
-        if (ms < best) { best = ms; choice = {2, c.first, c.second}; }
+        if (ms < best * (choice.fused ? 0.95f : 1.f)) { best = ms; choice = {2, c.first, c.second, false}; }
     }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
     b->t = 0;
     b->cur = 0;
     {
@@ -583,7 +653,7 @@ cdf_status bautotune(cdf_batch *b) {
         b->chain_th = choice.th;
         return setup_tiles(b, dim3(64, 4));
     }
-    b->fused = fused_fits(b);
+    b->fused = choice.fused;
     return setup_tiles(b, choice.shape);
 }
 
@@ -704,10 +774,7 @@ cdf_status cdf_batch_create(int count, const cdf_grid *grids, int m, const cdf_d
     }
     cdf_status st;
     if (opt->mode >= 1 && opt->tile_x > 0) st = setup_tiles(b, dim3(64, 4));
-    else if (opt->tile_x > 0) {
-        b->fused = fused_fits(b);
-        st = setup_tiles(b, dim3(opt->tile_x, opt->tile_y));
-    }
+    else if (opt->tile_x > 0) st = setup_whole(b, dim3(opt->tile_x, opt->tile_y));
     else if (b->extra_arrivals) st = setup_tiles(b, dim3(64, 4));
     else st = bautotune(b);
     if (st == CDF_OK && cudaStreamSynchronize(b->s) != cudaSuccess) st = bfail(CDF_ECUDA, "set-up failed");

@@ -70,6 +70,32 @@ def test_mode_0_kernels(cdf):
         assert c.launches(2) == per_two and c.launches(3) == per_two + 4
 
 
+@pytest.mark.parametrize("m,nx,ny,count,pair", [(2, 2000, 1, 500, False), (4, 2000, 1, 300, False), (2, 64, 64, 40, True),
+                                                (4, 3, 2000, 60, True)])
+def test_thin_lattices_run_on_the_faster_kernel(cdf, m, nx, ny, count, pair):
+    """Rows of one node leave the two-step launches' CTAs mostly idle: 2.2 times the persistent kernel's time with two
+    scalars, 3.4 with four; columns of three nodes waste its 128 x 1 tiles: 3.9 times the two-step launches'."""
+    from test_parity_gpu import _rand_problem
+    pb = _rand_problem(nx, ny, m, 3, "mixed", "noslip_noflux")
+    b = cdf.BatchSolver([pb] * count, tile=(128, 1), mode=0, init=False)
+    assert (b.launches(64) > 2) == pair
+    b.close()
+
+
+@pytest.mark.parametrize("tile", [(64, 4), None])
+@pytest.mark.parametrize("m,nx,ny", [(3, 60, 2), (4, 9, 9), (1, 7, 7), (3, 40, 30)])
+def test_timed_batches_keep_the_bits(cdf, tile, m, nx, ny):
+    from test_parity_gpu import _rand_problem
+    pbs = [_rand_problem(nx, ny, m, 3 + k, "periodic", "noslip_noflux") for k in range(5)]
+    b = cdf.BatchSolver(pbs, **(dict(tile=tile, mode=0) if tile else {}))
+    b.step(33)
+    b.step(2)
+    for k, pb in enumerate(pbs):
+        s = cdf.Solver(pb)
+        s.step(35)
+        assert np.array_equal(b.moments(k), s.moments()), k
+
+
 if __name__ == "__main__":
     from paper_2101_03055_gb300 import lib
     assert lib.CHECKS and lib.cdf_checks_enabled(), "the checks library was not loaded"
