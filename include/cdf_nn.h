@@ -40,7 +40,9 @@ cdf_nn_status cdf_nn_conv3x3_bwd_data(const void *dy, const void *w, void *dx, i
  * cdf_nn_conv3x3_bwd_weight_workspace() bytes, owned by the caller, contents
  * overwritten; about 160 MB at most, or one split's sums, 36 Cin Cout bytes, where those are
  * more) and are added in a fixed order: the result is the same bits on
- * every run.  The warp-level MMA path adds its partial sums
+ * every run.  A padding position counts as dy = 0 times the x beside it, so where x is not finite in
+ * an image's first or last row or column, the taps that do not reach it may come out NaN beside its
+ * channel's other taps, which are not finite either.  The warp-level MMA path adds its partial sums
  * atomically (order-dependent) and ignores the workspace. */
 cdf_nn_status cdf_nn_conv3x3_bwd_weight(const void *x, const void *dy, float *dw, float *db, int N, int H, int W,
                                         int Cin, int Cout, void *workspace, long long workspace_bytes, void *stream);

@@ -383,21 +383,6 @@ __global__ void __launch_bounds__(FW ? FW * FY : step2_max_threads(M), FW ? step
     }
 }
 
-// The same for up to kBatchGroup instances of a batch in one launch: CTA (t, k) works on tile
-// t of instance k of `pack`, whose parameters lie in the constant bank.
-// Every instance has output tiles of its own size tw x th, as even a division
-// of its lattice as fits (pair_tile in lb_batch.cu): a 64 x 64 lattice is eight tiles of
-// 32 x 16, where 30 x 14 tiles would be fifteen, 65 % full.  So the nodes of R1 and of the
-// tile are walked as lists (NodeWalk), whatever the width; the row pitch and the plane
-// stride in shared memory are constants.
-// Bound by instruction issue and the latency of a CTA's few rounds (issue active 63 %, four
-// CTAs of 256 threads an SM).  512 cavities of 64 x 64, 64 steps with initialisation and moments: 8.7 ms
-// on the persistent kernel; 3.9 with the parameters staged in shared memory, a
-// runtime pitch and a row-order walk; 3.2 with the parameters in the constant bank (no
-// spills, uniform operands) and constant strides; 2.7 with the inner nodes first; 2.5 with
-// the groups of lattices that run side by side held in L2 (lb_batch.cu).  Chains of step2_kernel per
-// instance: 72.5 us a step for these against 36.9, and 67.6 against 65.8 for 64 plumes of 128-512 x
-// 64-256, but 6.5 against 7.8 for 8 lattices of 300 x 200; the autotuner times both.
 // A rectangle [xa, xb) x [ya, yb) of nodes walked by a CTA, 32 a round: first its part away from
 // the lattice's edges, in row order, then the strips along the edges (at most two nodes wide,
 // left, right, lower, upper), so that a round runs either the pull without boundary
@@ -457,6 +442,21 @@ struct NodeWalk {
     }
 };
 
+// step2_kernel for up to kBatchGroup instances of a batch in one launch: CTA (t, k) works on tile
+// t of instance k of `pack`, whose parameters lie in the constant bank.
+// Every instance has output tiles of its own size tw x th, as even a division
+// of its lattice as fits (pair_tile in lb_batch.cu): a 64 x 64 lattice is eight tiles of
+// 32 x 16, where 30 x 14 tiles would be fifteen, 65 % full.  So the nodes of R1 and of the
+// tile are walked as lists (NodeWalk), whatever the width; the row pitch and the plane
+// stride in shared memory are constants.
+// Bound by instruction issue and the latency of a CTA's few rounds (issue active 63 %, four
+// CTAs of 256 threads an SM).  512 cavities of 64 x 64, 64 steps with initialisation and moments: 8.7 ms
+// on the persistent kernel; 3.9 with the parameters staged in shared memory, a
+// runtime pitch and a row-order walk; 3.2 with the parameters in the constant bank (no
+// spills, uniform operands) and constant strides; 2.7 with the inner nodes first; 2.5 with
+// the groups of lattices that run side by side held in L2 (lb_batch.cu).  Chains of step2_kernel per
+// instance: 72.5 us a step for these against 36.9, and 67.6 against 65.8 for 64 plumes of 128-512 x
+// 64-256, but 6.5 against 7.8 for 8 lattices of 300 x 200; the autotuner times both.
 template <int M, int K>
 __global__ void __launch_bounds__(256, step2_max_threads(M) / 256)
     step2_batch_kernel(const __grid_constant__ BatchPack pack, const float *in, float *out, const float *sp_in,
